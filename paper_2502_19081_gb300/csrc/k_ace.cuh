@@ -11,12 +11,13 @@
 //      shared memory, then each lane accumulates fixed (lm, 4 q) outputs;
 //   3. nu <= 2 readout; omega = dE/dA initialised;
 //   4. nu = 3, one l-triple (l1, l2, l3) after the other.  The triple's tables
-//      (W[q1 q2][q3], the Gaunt entries in three orderings and their offsets)
-//      form one tile; the CTA streams the tiles from global memory into two
+//      (W[q1 q2][q3]; float64 also the Gaunt entries in two orderings and their
+//      offsets) form one tile; the CTA streams the tiles from global memory into two
 //      shared-memory buffers with cp.async, fetching tile t+1 while the warps
 //      work on tile t, so a tile crosses L2 once per group of atoms rather
-//      than once per atom.  Per warp, one pass over lane units (q1, block of qb
-//      consecutive q2; the W rows of the block sit in registers) does all of
+//      than once per atom.  Float: k_nu3.cuh.  Float64, per warp: one pass over
+//      lane units (q1, block of qb consecutive q2; the W rows of the block sit
+//      in registers) does all of
 //        U[m3][q1][q2] = sum_q3 W[q1 q2][q3] A3[m3][q3]
 //        Z[m3][q1 q2]  = sum_(m1 m2) G A1[m1][q1] A2[m2][q2]     (Gaunt-sparse)
 //        E += sum Z U;  omega3 += W^T Z;  omega1 += G A2 U
@@ -37,32 +38,12 @@
 // in a fixed order (compensated for float).
 #pragma once
 
+#include "k_ace_ops.h"
+#include "k_nu3.cuh"
 #include "mix_launch.h"
 #include "tc.cuh"
 
 namespace mixd {
-
-// The Gaunt coefficients ordered by m3 for every l-triple, shared by all
-// potentials (AceTileHdr): a copy in the constant memory of each module that
-// holds the float expensive kernels, so that the warp-uniform entry reads of
-// the nu = 3 pass are constant-bank loads.
-static __constant__ GEnt<float> c_gent_f[GAUNT_ENT_CAP];
-static __constant__ int c_grow[GAUNT_ROW_CAP];
-
-// this module's copy of the table (host side)
-static inline cudaError_t gaunt_upload_module(const void* ent_f, int n_ent, const int* rows, int n_rows) {
-    if (n_ent > GAUNT_ENT_CAP || n_rows > GAUNT_ROW_CAP) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemcpyToSymbol(c_gent_f, ent_f, (size_t)n_ent * sizeof(GEnt<float>));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_grow, rows, (size_t)n_rows * sizeof(int));
-    return e;
-}
-
-// entry i of the constant-memory table
-__device__ __forceinline__ void gent_c(int i, int& pk, float& g) {
-    const GEnt<float> x = c_gent_f[i];
-    pk = x.pk;
-    g = x.g;
-}
 
 template <typename T> struct V4;
 template <> struct V4<float> {
@@ -85,12 +66,7 @@ __device__ __forceinline__ V4<double> ld4<double>(const double* p) {
     const double2 b = reinterpret_cast<const double2*>(p)[1];
     return {a.x, a.y, b.x, b.y};
 }
-// one Gaunt entry of a tile in shared memory (one 8- or 16-byte load)
-__device__ __forceinline__ void ld_gent(const GEnt<float>* p, int& pk, float& g) {
-    const int2 v = *reinterpret_cast<const int2*>(p);
-    pk = v.x;
-    g = __int_as_float(v.y);
-}
+// one Gaunt entry of a tile in shared memory (one 16-byte load)
 __device__ __forceinline__ void ld_gent(const GEnt<double>* p, int& pk, double& g) {
     const int4 v = *reinterpret_cast<const int4*>(p);
     pk = v.x;
@@ -251,7 +227,8 @@ struct AceLay {
     int o_p1;                  // omega1 partials, inside the scratch area
     int o_slot;                // list slots of the pair-gradient step, inside the scratch area
     int total;
-    __host__ __device__ AceLay(int tile_max, int cap, int n, int qb, int L, int NP, int ts, int warps,
+    // rows: nu3_rows(L)
+    __host__ __device__ AceLay(int tile_max, int cap, int n, int qb, int L, int rows, int NP, int ts, int warps,
                                int nbuf = 2) {
         const int nlm = (L + 1) * (L + 1), D = 2 * L + 1;
         const int du = 2 * L - 3 > 1 ? 2 * L - 3 : 1;
@@ -261,7 +238,8 @@ struct AceLay {
         o_om = o_at + ace_a16(nlm * NP * ts);     // omega[lm][q]
         o_scr = o_om + ace_a16(nlm * NP * ts);
         o_p1 = ace_a16(du * n * NP * ts);         // after U[m3][q1][q2]; P1[m1][unit]
-        const int nu3 = o_p1 + D * n * (NP / qb) * ts;
+        // float: the U / Z row buffer alone
+        const int nu3 = ts == 4 ? rows * n * NP * ts : o_p1 + D * n * (NP / qb) * ts;
         const int chunk = (32 * NP + 32 * nlm) * ts;   // R[32][NP], Y[32][nlm]
         o_slot = ace_a16(4 * cap * ts);           // after [cap][4]: unit vector, r
         const int pairs = o_slot + 4 * cap;
@@ -288,55 +266,6 @@ __device__ __forceinline__ void tile_fetch(const unsigned char* tiles, const int
     cp_async_commit();
 }
 
-// Reduce-scatter of C <= 16 per-lane values over the warp.  At lane bit MASK
-// (16, 8, 4, 2, 1 in turn) the lanes with the bit set keep the upper half of
-// their block (padded with a zero when the count is odd) and send the lower
-// half to their partner, the others the reverse, and each adds what it
-// receives, so the count halves at every bit; once one value is left the
-// remaining bits sum it (both partners add the same two numbers).  The
-// additions are in a fixed order.  rs_entry gives the entry a lane ends with.
-template <typename T, int C, int MASK>
-__device__ __forceinline__ T warp_rs(T* v, int lane) {
-    if constexpr (MASK == 0) {
-        return v[0];
-    } else if constexpr (C == 1) {
-        v[0] += __shfl_xor_sync(0xffffffffu, v[0], MASK);
-        return warp_rs<T, 1, MASK / 2>(v, lane);
-    } else {
-        constexpr int H = (C + 1) / 2;
-        const bool up = (lane & MASK) != 0;
-#pragma unroll
-        for (int i = 0; i < H; ++i) {
-            const T hi = i + H < C ? v[i + H] : T(0);
-            const T send = up ? v[i] : hi;
-            const T keep = up ? hi : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, MASK);
-        }
-        return warp_rs<T, H, MASK / 2>(v, lane);
-    }
-}
-
-// The entry of warp_rs<T, C, 16> a lane holds (idx), and whether the lane is
-// the one of its group that writes it (a real entry, the lowest lane of the
-// lanes that hold the same sum).
-template <int C, int MASK>
-__device__ __forceinline__ void rs_entry(int lane, int& idx, int& real, bool& writer) {
-    if constexpr (MASK == 0) {
-        writer = real >= 1;
-    } else if constexpr (C == 1) {
-        writer = real >= 1 && (lane & (2 * MASK - 1)) == 0;
-    } else {
-        constexpr int H = (C + 1) / 2;
-        if (lane & MASK) {
-            idx += H;
-            real = real > H ? real - H : 0;
-        } else {
-            real = real < H ? real : H;
-        }
-        rs_entry<H, MASK / 2>(lane, idx, real, writer);
-    }
-}
-
 // nu = 3 of one l-triple for this warp's atom, in one pass over lane units
 // (q1, block of QB consecutive q2).  A unit keeps the W rows of its block in
 // registers; for each m3 (uniform over the warp, so entry and A3 loads are
@@ -354,8 +283,8 @@ __device__ __forceinline__ void rs_entry(int lane, int& idx, int& real, bool& wr
 //             partials of the units of one q1 are summed after the last m3;
 // and, for distinct l's only (omega2 needs it after the pass), stores U.
 // All three l's equal: U is not formed (no adjoint needs it) and the energy is
-// taken as sum A3 (W^T Z), the same sum reordered.  This is the float64 pass;
-// float runs nu3_units_f, the same arithmetic on packed pairs.
+// taken as sum A3 (W^T Z), the same sum reordered.  This is the float64 pass
+// (float: k_nu3.cuh).
 template <typename T, int NP, int QB>
 __device__ __forceinline__ void nu3_units(const AceTileHdr& h, const T* W, const GEnt<T>* ge3, const int* g3o,
                                           const T* A1, const T* A2, const T* A3, int n, int lane, T* U1, T* P1,
@@ -464,207 +393,20 @@ __device__ __forceinline__ void nu3_units(const AceTileHdr& h, const T* W, const
     }
 }
 
-// QB / 2 pairs of consecutive floats from shared memory (QB in {2, 4, 6},
-// 8-byte aligned; QB = 4 16-byte aligned)
-template <int QB>
-__device__ __forceinline__ void ld_pairs(const float* p, float2* out) {
-    if constexpr (QB == 4) {
-        const float4 v = *reinterpret_cast<const float4*>(p);
-        out[0] = make_float2(v.x, v.y);
-        out[1] = make_float2(v.z, v.w);
-    } else {
-#pragma unroll
-        for (int k = 0; k < QB / 2; ++k) out[k] = reinterpret_cast<const float2*>(p)[k];
-    }
-}
-
-// The float unit pass: the arithmetic of nu3_units on packed pairs
-// (__ffma2_rn: two float fused multiply-adds an instruction), which halves the
-// instructions of its dense products.  W rows are held as pairs of
-// consecutive q3: U = W A3 runs as two interleaved sums (even and odd q3)
-// added at the end, and the omega3 partials pair consecutive q3 against a
-// broadcast Z (the same order of additions as the float64 pass).  Z, the
-// omega1 dot product and the energy pair consecutive q2.
-//
-// TCM != 0 (the tensor-core readout): omega3 and the energy are not formed
-// here.  Z goes, rounded to bf16 (TCM == 2: also its remainder, the lo part),
-// into this atom's rows of the MMA operand tile (row m3, column q1 n + q2 of
-// the K-major layout of tc.cuh), from which the tensor cores form V = Z W
-// (omega3 = mult3 V, E = sum A3 V) after the pass.
-template <int NP, int QB, int TCM>
-__device__ __forceinline__ void nu3_units_f(const AceTileHdr& h, const float* W, const float* A1, const float* A2,
-                                            const float* A3, int n, int lane, float* U1, float* P1, float* o3,
-                                            float mult3, float& ep, unsigned char* zhi, unsigned char* zlo,
-                                            int zsbo) {
-    static_assert(QB % 2 == 0 && NP % 4 == 0, "the float pass works on pairs");
-    constexpr int nqb = NP / QB, NH = NP / 2, QH = QB / 2;
-    const int units = n * nqb;
-    const int d3 = 2 * h.l3 + 1, rb = h.cg;
-    const bool withu = h.mode != 3;
-    const bool keepu = h.mode == 0;
-    int q3o = 0, q3real = NP;
-    bool q3w = false;
-    rs_entry<NP, 16>(lane, q3o, q3real, q3w);
-    float2 e2 = make_float2(0.f, 0.f);
-    for (int u0 = 0; u0 < units; u0 += 32) {
-        const int u = u0 + lane;
-        const bool uv = u < units;
-        const int uu = uv ? u : 0;
-        const int q1 = uu / nqb;
-        const int q2 = (uu - q1 * nqb) * QB;
-        const float* A1q = A1 + q1;
-        const float* A2q = A2 + q2;
-        int zcol[TCM != 0 ? QH : 1];   // column part of the operand offset of each pair
-#pragma unroll
-        for (int k = 0; k < (TCM != 0 ? QH : 1); ++k) zcol[k] = tc_off(0, q1 * n + q2 + 2 * k, TC_LBO_A, 0);
-        int e = c_grow[rb], pkn;   // the entries of all m3 rows follow each other
-        float gn;
-        gent_c(e, pkn, gn);
-        float2 w[QB][NH];
-#pragma unroll
-        for (int r = 0; r < QB; ++r) {
-            const bool ok = uv && q2 + r < n;
-            const float* wr = W + (q1 * n + (ok ? q2 + r : 0)) * NP;
-#pragma unroll
-            for (int p = 0; p < NP; p += 4) {
-                float4 v = *reinterpret_cast<const float4*>(wr + p);
-                if (!ok) v = make_float4(0.f, 0.f, 0.f, 0.f);
-                w[r][p / 2] = make_float2(v.x, v.y);
-                w[r][p / 2 + 1] = make_float2(v.z, v.w);
-            }
-        }
-        for (int m3 = 0; m3 < d3; ++m3) {
-            float2 uo[QH], z[QH];
-#pragma unroll
-            for (int k = 0; k < QH; ++k) {
-                uo[k] = make_float2(0.f, 0.f);
-                z[k] = make_float2(0.f, 0.f);
-            }
-            if (withu) {
-                float2 a[NH];
-#pragma unroll
-                for (int p = 0; p < NP; p += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(A3 + m3 * NP + p);
-                    a[p / 2] = make_float2(v.x, v.y);
-                    a[p / 2 + 1] = make_float2(v.z, v.w);
-                }
-#pragma unroll
-                for (int r = 0; r < QB; ++r) {
-                    float2 s = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int j = 0; j < NH; ++j) s = __ffma2_rn(w[r][j], a[j], s);
-                    if (r & 1) uo[r / 2].y = s.x + s.y;
-                    else uo[r / 2].x = s.x + s.y;
-                }
-            }
-            const int e1 = c_grow[rb + m3 + 1];
-            float2 c1 = make_float2(0.f, 0.f);
-            for (; e < e1; ++e) {
-                const int pk = pkn;
-                const float g = gn;
-                // the next entry (of this row, the next row or triple, or the
-                // zero entry after the last) is in flight while this one works
-                gent_c(e + 1, pkn, gn);
-                const float ga = g * A1q[(pk & 255) * NP];
-                const float2 ga2 = make_float2(ga, ga);
-                float2 a2[QH];
-                ld_pairs<QB>(A2q + ((pk >> 8) & 255) * NP, a2);
-#pragma unroll
-                for (int k = 0; k < QH; ++k) z[k] = __ffma2_rn(ga2, a2[k], z[k]);
-                if (withu) {
-                    float2 dd = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int k = 0; k < QH; ++k) dd = __ffma2_rn(a2[k], uo[k], dd);
-                    c1 = __ffma2_rn(make_float2(g, g), dd, c1);
-                    if (pk & GE_RUN_END) {   // uniform over the warp
-                        if (uv) P1[(pk & 255) * units + u] += c1.x + c1.y;
-                        c1 = make_float2(0.f, 0.f);
-                    }
-                }
-            }
-            if (withu) {
-                if constexpr (TCM == 0) {
-#pragma unroll
-                    for (int k = 0; k < QH; ++k) e2 = __ffma2_rn(uo[k], z[k], e2);
-                }
-                if (keepu && uv) {
-#pragma unroll
-                    for (int k = 0; k < QH; ++k)
-                        *reinterpret_cast<float2*>(U1 + (m3 * n + q1) * NP + q2 + 2 * k) = uo[k];
-                }
-            }
-            if constexpr (TCM != 0) {
-                if (uv && (n & 1) == 0) {
-                    // even n: columns q1 n + q2 + r, r even, are even, so each
-                    // pair lies in one 4-byte word of a core-matrix row; the
-                    // row part of the offset is the m3 one, the column part the unit's
-                    const int orow = tc_off(m3, 0, TC_LBO_A, zsbo);
-#pragma unroll
-                    for (int k = 0; k < QH; ++k) {
-                        if (q2 + 2 * k < n) {
-                            const int o = orow + zcol[k];
-                            const __nv_bfloat162 hi = __float22bfloat162_rn(z[k]);
-                            *reinterpret_cast<__nv_bfloat162*>(zhi + o) = hi;
-                            if constexpr (TCM == 2) {
-                                const float2 hf = __bfloat1622float2(hi);
-                                *reinterpret_cast<__nv_bfloat162*>(zlo + o) =
-                                    __float22bfloat162_rn(make_float2(z[k].x - hf.x, z[k].y - hf.y));
-                            }
-                        }
-                    }
-                } else if (uv) {
-#pragma unroll
-                    for (int r = 0; r < QB; ++r) {
-                        if (q2 + r < n) {
-                            const float zr = (r & 1) ? z[r / 2].y : z[r / 2].x;
-                            const int o = tc_off(m3, q1 * n + q2 + r, TC_LBO_A, zsbo);
-                            const __nv_bfloat16 hi = __float2bfloat16_rn(zr);
-                            *reinterpret_cast<__nv_bfloat16*>(zhi + o) = hi;
-                            if constexpr (TCM == 2)
-                                *reinterpret_cast<__nv_bfloat16*>(zlo + o) =
-                                    __float2bfloat16_rn(zr - __bfloat162float(hi));
-                        }
-                    }
-                }
-            } else {
-                // omega3 row m3
-                float pv[16];
-#pragma unroll
-                for (int j = 0; j < NH; ++j) {
-                    float2 s = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int r = 0; r < QB; ++r) {
-                        const float zr = (r & 1) ? z[r / 2].y : z[r / 2].x;
-                        s = __ffma2_rn(w[r][j], make_float2(zr, zr), s);
-                    }
-                    pv[2 * j] = s.x;
-                    pv[2 * j + 1] = s.y;
-                }
-                const float s3 = warp_rs<float, NP, 16>(pv, lane);
-                if (q3w && q3o < n) {
-                    o3[m3 * NP + q3o] += mult3 * s3;
-                    if (!withu) ep += A3[m3 * NP + q3o] * s3;
-                }
-            }
-        }
-    }
-    ep += e2.x + e2.y;
-}
-
-// One l-triple for this warp's atom, from the tile in shared memory.
-// PART 1: the unit pass; PART 2: omega1 from the unit partials and omega2;
-// PART 3: both.
-template <typename T, int NP, int TCM = 0, int PART = 3>
-__device__ __forceinline__ void nu3_tile(const unsigned char* tile, const AceTab<T>& tab, const T* At, T* om,
-                                         T* U1, T* P1, int lane, T& ep, unsigned char* zhi = nullptr,
-                                         unsigned char* zlo = nullptr, int zsbo = 0) {
-    constexpr int QM = 4;     // largest power-of-two q2 block of a lane unit
+// One l-triple for this warp's atom in float64, from the tile in shared memory:
+// the unit pass, then omega1 from the unit partials and omega2.
+template <int NP>
+__device__ __forceinline__ void nu3_tile(const unsigned char* tile, const AceTab<double>& tab, const double* At,
+                                         double* om, double* U1, double* P1, int lane, double& ep) {
+    using T = double;
     const AceTileHdr h = *reinterpret_cast<const AceTileHdr*>(tile);
     const T* W = reinterpret_cast<const T*>(tile + sizeof(AceTileHdr));
     const GEnt<T>* ge = reinterpret_cast<const GEnt<T>*>(tile + h.o_ge);   // ordered by m2
     const int* g2o = reinterpret_cast<const int*>(tile + h.o_go);
-    const int n = tab.n;
-    const int d1 = 2 * h.l1 + 1, d2 = 2 * h.l2 + 1, d3 = 2 * h.l3 + 1;
+    const GEnt<T>* ge3 = reinterpret_cast<const GEnt<T>*>(tile + h.o_ge3);   // ordered by m3
+    const int* g3o = reinterpret_cast<const int*>(tile + h.o_go3);
+    const int n = tab.n, qb = tab.qb;
+    const int d1 = 2 * h.l1 + 1, d2 = 2 * h.l2 + 1;
     // coinciding l's (W symmetrised on the host): scale instead of recompute
     const T mult1 = h.mode == 1 ? T(2) : T(1);
     const T mult3 = h.mode == 3 ? T(3) : (h.mode == 2 ? T(2) : T(1));
@@ -672,33 +414,11 @@ __device__ __forceinline__ void nu3_tile(const unsigned char* tile, const AceTab
     const T* A2 = At + h.l2 * h.l2 * NP;
     const T* A3 = At + h.l3 * h.l3 * NP;
     T* o3 = om + h.l3 * h.l3 * NP;
-    const int qb = tab.qb;
-    if constexpr ((PART & 1) != 0) {
-        if constexpr (sizeof(T) == 4) {
-            if constexpr (NP == 12) {
-                // n = 11 or 12: 6-wide blocks keep the units within one warp pass
-                if (qb == 6)
-                    nu3_units_f<NP, 6, TCM>(h, W, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep, zhi, zlo,
-                                            zsbo);
-            }
-            if (qb == QM)
-                nu3_units_f<NP, QM, TCM>(h, W, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep, zhi, zlo, zsbo);
-            else if (qb == QM / 2)
-                nu3_units_f<NP, QM / 2, TCM>(h, W, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep, zhi, zlo,
-                                             zsbo);
-        } else {
-            static_assert(sizeof(T) == 4 || TCM == 0, "the tensor-core readout is float only");
-            // float64 reads the ordering by m3 from its tile
-            const GEnt<T>* ge3 = reinterpret_cast<const GEnt<T>*>(tile + h.o_ge3);
-            const int* g3o = reinterpret_cast<const int*>(tile + h.o_go3);
-            if (qb == QM)
-                nu3_units<T, NP, QM>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
-            else
-                nu3_units<T, NP, QM / 2>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
-        }
-        __syncwarp();
-    }
-    if constexpr ((PART & 2) == 0) return;
+    if (qb == 4)
+        nu3_units<T, NP, 4>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
+    else
+        nu3_units<T, NP, 2>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
+    __syncwarp();
     // omega1 (equal to omega3 when all three l's coincide): sum the unit
     // partials of each (m1, q1) and clear them for the next triple
     if (h.mode != 3) {
@@ -729,38 +449,19 @@ __device__ __forceinline__ void nu3_tile(const unsigned char* tile, const AceTab
                 ld_gent(ge + e, pk, gv);
                 const T* ar = A1 + (pk & 255) * NP;
                 const T* ur = U1 + (pk >> 8) * n * NP + q2;
-                if constexpr (sizeof(T) == 4) {
-                    // the same fused multiply-adds, two an instruction
-                    float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
-                    for (int q1 = 0; q1 < n; ++q1) {
-                        const float av = ar[q1];
-                        const float2 a2 = make_float2(av, av);
-                        const V4<T> u4 = ld4<T>(ur + q1 * NP);
-                        s01 = __ffma2_rn(a2, make_float2(u4.x, u4.y), s01);
-                        s23 = __ffma2_rn(a2, make_float2(u4.z, u4.w), s23);
-                    }
-                    const float2 g2 = make_float2(gv, gv);
-                    const float2 c01 = __ffma2_rn(g2, s01, make_float2(c0, c1));
-                    const float2 c23 = __ffma2_rn(g2, s23, make_float2(c2, c3));
-                    c0 = c01.x;
-                    c1 = c01.y;
-                    c2 = c23.x;
-                    c3 = c23.y;
-                } else {
-                    T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
-                    for (int q1 = 0; q1 < n; ++q1) {
-                        const T av = ar[q1];
-                        const V4<T> u4 = ld4<T>(ur + q1 * NP);
-                        s0 += av * u4.x;
-                        s1 += av * u4.y;
-                        s2 += av * u4.z;
-                        s3 += av * u4.w;
-                    }
-                    c0 += gv * s0;
-                    c1 += gv * s1;
-                    c2 += gv * s2;
-                    c3 += gv * s3;
+                T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
+                for (int q1 = 0; q1 < n; ++q1) {
+                    const T av = ar[q1];
+                    const V4<T> u4 = ld4<T>(ur + q1 * NP);
+                    s0 += av * u4.x;
+                    s1 += av * u4.y;
+                    s2 += av * u4.z;
+                    s3 += av * u4.w;
                 }
+                c0 += gv * s0;
+                c1 += gv * s1;
+                c2 += gv * s2;
+                c3 += gv * s3;
             }
             T* orow = o2 + m2 * NP + q2;
             orow[0] += c0;
@@ -770,6 +471,53 @@ __device__ __forceinline__ void nu3_tile(const unsigned char* tile, const AceTab
         }
     }
     __syncwarp();
+}
+
+// the float triple's multiplicity of omega3 (coinciding l's, as in nu3_tile)
+__device__ __forceinline__ float nu3_mult3(const AceTileHdr& h) { return h.mode == 3 ? 3.f : (h.mode == 2 ? 2.f : 1.f); }
+
+// nu <= 2 in float: omega[lm][q] = sum_q2 S2[l][q][q2] A[lm][q2] (+ c1 at lm = 0)
+// and its energy.  A lane keeps the S2 row of its (l, q) in registers for every
+// m it takes (32 / NP lanes share the m's of an l), the next l's row in flight.
+template <int L, int NP>
+__device__ __forceinline__ void nu2_float(const AceTab<float>& tab, const float* At, float* om, int lane, float& ep) {
+    constexpr int NH = NP / 2, MS = 32 / NP;   // lanes over m
+    const int n = tab.n, q = lane % NP, ms = lane / NP;
+    const bool on = ms < MS, row = on && q < n && tab.nu >= 2;
+    float2 s[NH], sn[NH];
+    auto load = [&](int l, float2* r) {   // rows padded to NP, 16-byte aligned
+        const float4* p = reinterpret_cast<const float4*>(tab.S2p + (l * n + (row ? q : 0)) * NP);
+#pragma unroll
+        for (int k = 0; k < NP / 4; ++k) {
+            const float4 v = row ? __ldg(p + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+            r[2 * k] = make_float2(v.x, v.y);
+            r[2 * k + 1] = make_float2(v.z, v.w);
+        }
+    };
+    const float c = on && q < n ? __ldg(tab.c1 + q) : 0.f;
+    load(0, sn);
+#pragma unroll 1
+    for (int l = 0; l <= L; ++l) {
+#pragma unroll
+        for (int k = 0; k < NH; ++k) s[k] = sn[k];
+        if (l < L) load(l + 1, sn);
+        if (on) {
+            for (int lm = l * l + ms; lm < (l + 1) * (l + 1); lm += MS) {
+                float2 a[NH], v2 = make_float2(0.f, 0.f);
+                ld_row<NP>(At + lm * NP, a);
+#pragma unroll
+                for (int k = 0; k < NH; ++k) v2 = __ffma2_rn(s[k], a[k], v2);
+                float val = v2.x + v2.y;
+                const float av = At[lm * NP + q];
+                ep += 0.5f * av * val;
+                if (lm == 0) {
+                    ep += c * av;
+                    val += c;
+                }
+                om[lm * NP + q] = val;
+            }
+        }
+    }
 }
 
 // State of the tensor-core readout of one thread (TCM != 0).
@@ -792,7 +540,7 @@ constexpr int TC_WAIT_POLLS = 1 << 20;
 // below nexp), warp w on atom a0 + w; every thread of the CTA calls it.
 // TCM != 0 (float only): the nu = 3 readout V = Z W runs on the tensor cores
 // for the CTA's TC_ACE_WARPS atoms at once (16 rows (atom, m3) per atom).
-template <typename T, int L, int NP, int TCM = 0>
+template <typename T, int L, int NP, int QB, int TCM = 0>
 __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, int a0, int nexp, unsigned char* smem,
                                           TcState* tc = nullptr, int wn = ACE_GROUP) {
     const int WN = TCM != 0 ? TC_ACE_WARPS : wn;   // warps (atoms) of the CTA
@@ -804,7 +552,8 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
     using V = typename Vec4<T>::type;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = tab.n, cap = d.cap, ntau = tab.ntau;
-    const AceLay lay(tab.tile_max, cap, n, tab.qb, L, NP, (int)sizeof(T), WN, TCM != 0 ? tc->nbuf : 2);
+    constexpr int ROWS = nu3_rows(L);
+    const AceLay lay(tab.tile_max, cap, n, tab.qb, L, ROWS, NP, (int)sizeof(T), WN, TCM != 0 ? tc->nbuf : 2);
     // the first tile lands while the warps run steps 1-3
     if (ntau > 0) tile_fetch(tab.tiles, tab.tile_off, 0, smem);
 
@@ -908,39 +657,43 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
         __syncwarp();
 
         // 3. nu = 1 and nu = 2; initialises omega
-        for (int o = lane; o < NLM * NP; o += 32) {
-            const int lm = o / NP, q = o - lm * NP;
-            T val = T(0);
-            if (q < n) {
-                int l = 0;
-                while ((l + 1) * (l + 1) <= lm) ++l;
-                if (tab.nu >= 2) {
-                    // even and odd q2 in two chains; unrolled over the padded
-                    // count so that the row's coefficient loads are all in flight
-                    const T* S2 = tab.S2 + ((int64_t)l * n + q) * n;
-                    const T* Ar = At + lm * NP;
-                    T v2 = T(0);
-#pragma unroll
-                    for (int q2 = 0; q2 < NP; ++q2) {
-                        if (q2 < n) {
-                            if (q2 & 1) v2 += __ldg(S2 + q2) * Ar[q2];
-                            else val += __ldg(S2 + q2) * Ar[q2];
+        if constexpr (sizeof(T) == 4) {
+            nu2_float<L, NP>(tab, At, om, lane, ep);
+        } else {
+            for (int o = lane; o < NLM * NP; o += 32) {
+                const int lm = o / NP, q = o - lm * NP;
+                T val = T(0);
+                if (q < n) {
+                    int l = 0;
+                    while ((l + 1) * (l + 1) <= lm) ++l;
+                    if (tab.nu >= 2) {
+                        // even and odd q2 in two chains; unrolled over the padded
+                        // count so that the row's coefficient loads are all in flight
+                        const T* S2 = tab.S2 + ((int64_t)l * n + q) * n;
+                        const T* Ar = At + lm * NP;
+                        T v2 = T(0);
+    #pragma unroll
+                        for (int q2 = 0; q2 < NP; ++q2) {
+                            if (q2 < n) {
+                                if (q2 & 1) v2 += __ldg(S2 + q2) * Ar[q2];
+                                else val += __ldg(S2 + q2) * Ar[q2];
+                            }
                         }
+                        val += v2;
                     }
-                    val += v2;
+                    const T av = At[o];
+                    ep += T(0.5) * av * val;
+                    if (lm == 0) {
+                        const T c = __ldg(tab.c1 + q);
+                        ep += c * av;
+                        val += c;
+                    }
                 }
-                const T av = At[o];
-                ep += T(0.5) * av * val;
-                if (lm == 0) {
-                    const T c = __ldg(tab.c1 + q);
-                    ep += c * av;
-                    val += c;
-                }
+                om[o] = val;
             }
-            om[o] = val;
         }
-        // the omega1 partials start at zero (each triple clears what it used)
-        if (ntau > 0)
+        // float64: the omega1 partials start at zero (each triple clears what it used)
+        if (sizeof(T) == 8 && ntau > 0)
             for (int o = lane; o < D * n * (NP / tab.qb); o += 32) P1[o] = T(0);
         __syncwarp();
     }
@@ -951,7 +704,17 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
             cp_async_wait_all();
             __syncthreads();   // tile t visible; every warp is done with the other buffer
             if (t + 1 < ntau) tile_fetch(tab.tiles, tab.tile_off, t + 1, smem + ((t + 1) & 1) * lay.tile);
-            if (has) nu3_tile<T, NP>(smem + (t & 1) * lay.tile, tab, At, om, U1, P1, lane, ep);
+            const unsigned char* tile = smem + (t & 1) * lay.tile;
+            if constexpr (sizeof(T) == 8) {
+                if (has) nu3_tile<NP>(tile, tab, At, om, U1, P1, lane, ep);
+            } else if (has) {
+                const AceTileHdr h = *reinterpret_cast<const AceTileHdr*>(tile);
+                const float* W = reinterpret_cast<const float*>(tile + sizeof(AceTileHdr));
+                const int o3 = h.l3 * h.l3 * NP, d3 = 2 * h.l3 + 1;
+                if (h.mode != 3) nu3_dense_u<NP, QB>(W, At + o3, n, d3, lane, U1);
+                nu3_mid_of<L, NP, QB, 0>(h.tri, At, om, U1, n, lane, Nu3Op{});
+                nu3_dense_w<NP, QB>(W, At + o3, n, d3, U1, om + o3, nu3_mult3(h), lane, ep);
+            }
         }
     } else {
         // Per triple: the warps write Z rows (and form U, omega1, omega2 as in
@@ -983,7 +746,12 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
             if (tc->nbuf == 2 && t + 1 < ntau)
                 tile_fetch(tab.tiles, tab.tile_off, t + 1, smem + ((t + 1) & 1) * lay.tile);
             const AceTileHdr h = *reinterpret_cast<const AceTileHdr*>(tile);
-            if (has) nu3_tile<T, NP, TCM, 1>(tile, tab, At, om, U1, P1, lane, ep, zh, zl, tc->sbo);
+            if (has) {
+                if (h.mode != 3)
+                    nu3_dense_u<NP, QB>(reinterpret_cast<const float*>(tile + sizeof(AceTileHdr)),
+                                        At + h.l3 * h.l3 * NP, n, 2 * h.l3 + 1, lane, U1);
+                nu3_mid_of<L, NP, QB, TCM>(h.tri, At, om, U1, n, lane, Nu3Op{zh, zl, tc->sbo});
+            }
             fence_async_smem();    // this thread's Z rows, visible to the tensor cores
             __syncthreads();
             if (tid == 0 && !tc->abort) {
@@ -1002,7 +770,10 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
                 }
                 tc_commit(tc->bar);
             }
-            if (has) nu3_tile<T, NP, TCM, 2>(tile, tab, At, om, U1, P1, lane, ep, zh, zl, tc->sbo);
+            if (has && h.mode == 0) {
+                nu3_omega2<NP>(U1, om + h.l2 * h.l2 * NP, n, 2 * h.l2 + 1, lane);
+                __syncwarp();   // the rows are rewritten by the next triple
+            }
             if (!tc->abort && !mbar_wait(tc->bar, tc->phase, TC_WAIT_POLLS)) {
                 tc->abort = 1;
                 set_status(d.status, ST_TC_TIMEOUT);
@@ -1012,7 +783,7 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
             float v[16];
             tmem_ld16(tc->tmem + ((uint32_t)(32 * (warp & 3)) << 16), v);
             if (has && own && m3r < 2 * h.l3 + 1 && !tc->abort) {
-                const T mult3 = h.mode == 3 ? T(3) : (h.mode == 2 ? T(2) : T(1));
+                const T mult3 = nu3_mult3(h);
                 T* o3 = om + (h.l3 * h.l3 + m3r) * NP;
                 const T* a3 = At + (h.l3 * h.l3 + m3r) * NP;
 #pragma unroll
@@ -1183,7 +954,7 @@ __device__ __forceinline__ void ace_groups_done(const Dev& d) {
     }
 }
 
-template <typename T, int L, int NP>
+template <typename T, int L, int NP, int QB>
 __global__ void __launch_bounds__(ACE_MAX_WARPS * 32, ace_min_ctas_max<T>()) k_ace(Dev d, AceTab<T> tab) {
     const int WN = (int)(blockDim.x >> 5);   // ACE_GROUP or ACE_MAX_WARPS atoms a CTA
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1191,22 +962,14 @@ __global__ void __launch_bounds__(ACE_MAX_WARPS * 32, ace_min_ctas_max<T>()) k_a
     const int count = d.status[SW_NEXP];
     const int ng = (count + WN - 1) / WN;
     for (int g = ace_next_group(d, &s_g); g < ng; g = ace_next_group(d, &s_g))
-        ace_group<T, L, NP>(d, tab, g * WN, count, smem_raw, nullptr, WN);
+        ace_group<T, L, NP, QB>(d, tab, g * WN, count, smem_raw, nullptr, WN);
     ace_groups_done(d);
 }
 
 // Many systems: walks the flattened list {system, first atom of a group} of
 // one group of systems sharing (T, L, NP); the CTA reloads the system's Dev and
 // tables into shared memory when the system changes.
-template <typename T>
-struct AceBatch {
-    const Dev* devs;
-    const AceTab<T>* tabs;
-    const int2* list;
-    const int* count;
-};
-
-template <typename T, int L, int NP>
+template <typename T, int L, int NP, int QB>
 __global__ void __launch_bounds__(ace_warps<T>() * 32, ace_min_ctas<T>()) kb_ace(AceBatch<T> b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Dev s_dev;
@@ -1222,15 +985,16 @@ __global__ void __launch_bounds__(ace_warps<T>() * 32, ace_min_ctas<T>()) kb_ace
             __syncthreads();
             cur = e.x;
         }
-        ace_group<T, L, NP>(s_dev, s_tab, e.y, s_dev.status[SW_NEXP], smem_raw);
+        ace_group<T, L, NP, QB>(s_dev, s_tab, e.y, s_dev.status[SW_NEXP], smem_raw);
     }
 }
 
 // launch shape: the shared memory of the layout, and as many resident CTAs as fit
-template <typename T, int L, int NP>
+template <typename T, int L, int NP, int QB>
 inline cudaError_t ace_shape(const void* kern, int n, int cap, int tile_max, int qb, size_t* smem, int* grid,
                              int wn = ACE_GROUP) {
-    const AceLay lay(tile_max, cap, n, qb, L, NP, (int)sizeof(T), wn);
+    constexpr int ROWS = nu3_rows(L);
+    const AceLay lay(tile_max, cap, n, qb, L, ROWS, NP, (int)sizeof(T), wn);
     const size_t bytes = (size_t)lay.total;
     cudaError_t e = raise_smem_limit(kern, bytes);
     if (e != cudaSuccess) return e;
@@ -1243,77 +1007,60 @@ inline cudaError_t ace_shape(const void* kern, int n, int cap, int tile_max, int
     return cudaSuccess;
 }
 
-template <typename T, int L, int NP>
+template <typename T, int L, int NP, int QB>
 inline cudaError_t ace_cfg(bool batch, int n, int cap, int tile_max, int qb, size_t* smem, int* grid, int wn) {
-    const void* kern = batch ? (const void*)kb_ace<T, L, NP> : (const void*)k_ace<T, L, NP>;
-    return ace_shape<T, L, NP>(kern, n, cap, tile_max, qb, smem, grid, batch ? ACE_GROUP : wn);
+    const void* kern = batch ? (const void*)kb_ace<T, L, NP, QB> : (const void*)k_ace<T, L, NP, QB>;
+    return ace_shape<T, L, NP, QB>(kern, n, cap, tile_max, qb, smem, grid, batch ? ACE_GROUP : wn);
 }
 
-template <typename T, int NP>
+template <typename T, int NP, int QB>
 inline cudaError_t ace_cfg_l(bool batch, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid,
                              int wn) {
     switch (L) {
-        case 0: return ace_cfg<T, 0, NP>(batch, n, cap, tile_max, qb, smem, grid, wn);
-        case 1: return ace_cfg<T, 1, NP>(batch, n, cap, tile_max, qb, smem, grid, wn);
-        case 2: return ace_cfg<T, 2, NP>(batch, n, cap, tile_max, qb, smem, grid, wn);
-        case 3: return ace_cfg<T, 3, NP>(batch, n, cap, tile_max, qb, smem, grid, wn);
-        case 4: return ace_cfg<T, 4, NP>(batch, n, cap, tile_max, qb, smem, grid, wn);
-        case 5: return ace_cfg<T, 5, NP>(batch, n, cap, tile_max, qb, smem, grid, wn);
-        case 6: return ace_cfg<T, 6, NP>(batch, n, cap, tile_max, qb, smem, grid, wn);
+        case 0: return ace_cfg<T, 0, NP, QB>(batch, n, cap, tile_max, qb, smem, grid, wn);
+        case 1: return ace_cfg<T, 1, NP, QB>(batch, n, cap, tile_max, qb, smem, grid, wn);
+        case 2: return ace_cfg<T, 2, NP, QB>(batch, n, cap, tile_max, qb, smem, grid, wn);
+        case 3: return ace_cfg<T, 3, NP, QB>(batch, n, cap, tile_max, qb, smem, grid, wn);
+        case 4: return ace_cfg<T, 4, NP, QB>(batch, n, cap, tile_max, qb, smem, grid, wn);
+        case 5: return ace_cfg<T, 5, NP, QB>(batch, n, cap, tile_max, qb, smem, grid, wn);
+        case 6: return ace_cfg<T, 6, NP, QB>(batch, n, cap, tile_max, qb, smem, grid, wn);
     }
     return cudaErrorInvalidValue;
 }
 
-template <typename T>
-inline cudaError_t ace_cfg_t(bool batch, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid,
-                             int wn = ACE_GROUP) {
-    if (n <= 4) return ace_cfg_l<T, 4>(batch, L, n, cap, tile_max, qb, smem, grid, wn);
-    if (n <= 8) return ace_cfg_l<T, 8>(batch, L, n, cap, tile_max, qb, smem, grid, wn);
-    if (n <= 12) return ace_cfg_l<T, 12>(batch, L, n, cap, tile_max, qb, smem, grid, wn);
-    return ace_cfg_l<T, 16>(batch, L, n, cap, tile_max, qb, smem, grid, wn);
-}
-
-template <typename T, int NP>
+template <typename T, int NP, int QB>
 inline void ace_launch_l(const Dev& d, const AceTab<T>& tab, int L, size_t smem, int grid, int wn, cudaStream_t s) {
     const int th = wn * 32;
     switch (L) {
-        case 0: k_ace<T, 0, NP><<<grid, th, smem, s>>>(d, tab); break;
-        case 1: k_ace<T, 1, NP><<<grid, th, smem, s>>>(d, tab); break;
-        case 2: k_ace<T, 2, NP><<<grid, th, smem, s>>>(d, tab); break;
-        case 3: k_ace<T, 3, NP><<<grid, th, smem, s>>>(d, tab); break;
-        case 4: k_ace<T, 4, NP><<<grid, th, smem, s>>>(d, tab); break;
-        case 5: k_ace<T, 5, NP><<<grid, th, smem, s>>>(d, tab); break;
-        case 6: k_ace<T, 6, NP><<<grid, th, smem, s>>>(d, tab); break;
+        case 0: k_ace<T, 0, NP, QB><<<grid, th, smem, s>>>(d, tab); break;
+        case 1: k_ace<T, 1, NP, QB><<<grid, th, smem, s>>>(d, tab); break;
+        case 2: k_ace<T, 2, NP, QB><<<grid, th, smem, s>>>(d, tab); break;
+        case 3: k_ace<T, 3, NP, QB><<<grid, th, smem, s>>>(d, tab); break;
+        case 4: k_ace<T, 4, NP, QB><<<grid, th, smem, s>>>(d, tab); break;
+        case 5: k_ace<T, 5, NP, QB><<<grid, th, smem, s>>>(d, tab); break;
+        case 6: k_ace<T, 6, NP, QB><<<grid, th, smem, s>>>(d, tab); break;
     }
 }
 
-template <typename T>
-inline void ace_launch_t(const Dev& d, const AceTab<T>& tab, int L, size_t smem, int grid, int wn, cudaStream_t s) {
-    if (tab.np == 4) ace_launch_l<T, 4>(d, tab, L, smem, grid, wn, s);
-    else if (tab.np == 8) ace_launch_l<T, 8>(d, tab, L, smem, grid, wn, s);
-    else if (tab.np == 12) ace_launch_l<T, 12>(d, tab, L, smem, grid, wn, s);
-    else ace_launch_l<T, 16>(d, tab, L, smem, grid, wn, s);
-}
-
-template <typename T, int NP>
+template <typename T, int NP, int QB>
 inline void ace_batch_launch_l(const AceBatch<T>& b, int L, size_t smem, int grid, cudaStream_t s) {
     switch (L) {
-        case 0: kb_ace<T, 0, NP><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
-        case 1: kb_ace<T, 1, NP><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
-        case 2: kb_ace<T, 2, NP><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
-        case 3: kb_ace<T, 3, NP><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
-        case 4: kb_ace<T, 4, NP><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
-        case 5: kb_ace<T, 5, NP><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
-        case 6: kb_ace<T, 6, NP><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
+        case 0: kb_ace<T, 0, NP, QB><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
+        case 1: kb_ace<T, 1, NP, QB><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
+        case 2: kb_ace<T, 2, NP, QB><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
+        case 3: kb_ace<T, 3, NP, QB><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
+        case 4: kb_ace<T, 4, NP, QB><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
+        case 5: kb_ace<T, 5, NP, QB><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
+        case 6: kb_ace<T, 6, NP, QB><<<grid, ace_warps<T>() * 32, smem, s>>>(b); break;
     }
 }
 
-template <typename T>
-inline void ace_batch_launch_t(const AceBatch<T>& b, int n, int L, size_t smem, int grid, cudaStream_t s) {
-    if (n <= 4) ace_batch_launch_l<T, 4>(b, L, smem, grid, s);
-    else if (n <= 8) ace_batch_launch_l<T, 8>(b, L, smem, grid, s);
-    else if (n <= 12) ace_batch_launch_l<T, 12>(b, L, smem, grid, s);
-    else ace_batch_launch_l<T, 16>(b, L, smem, grid, s);
+// the table of the float class N
+template <int N>
+constexpr AceOps<float> ace_f32_ops() {
+    constexpr int NP = (N + 3) / 4 * 4, QB = nu3_qb(N);
+    return {ace_cfg_l<float, NP, QB>, ace_launch_l<float, NP, QB>, ace_batch_launch_l<float, NP, QB>,
+            gaunt_upload_module};
 }
 
 }  // namespace mixd

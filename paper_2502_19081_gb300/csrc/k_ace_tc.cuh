@@ -23,7 +23,7 @@
 
 namespace mixd {
 
-template <int L, int NP, int TCM>
+template <int L, int NP, int QB, int TCM>
 __global__ void __launch_bounds__(TC_ACE_WARPS * 32, TC_MIN_CTAS) k_ace_tc(Dev d, AceTab<float> tab, int nbuf) {
     extern __shared__ __align__(128) unsigned char smem_tc[];
     __shared__ __align__(8) unsigned long long s_bar;
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(TC_ACE_WARPS * 32, TC_MIN_CTAS) k_ace_tc(Dev d
     const int ng = (count + TC_ACE_WARPS - 1) / TC_ACE_WARPS;
     __shared__ int s_g;
     for (int g = ace_next_group(d, &s_g); g < ng; g = ace_next_group(d, &s_g))
-        ace_group<float, L, NP, TCM>(d, tab, g * TC_ACE_WARPS, count, sm + NZ * zbytes, &tc);
+        ace_group<float, L, NP, QB, TCM>(d, tab, g * TC_ACE_WARPS, count, sm + NZ * zbytes, &tc);
     ace_groups_done(d);
     tc_fence_before();
     __syncthreads();
@@ -68,19 +68,20 @@ __global__ void __launch_bounds__(TC_ACE_WARPS * 32, TC_MIN_CTAS) k_ace_tc(Dev d
 }
 
 // dynamic shared memory of k_ace_tc (with 128 bytes for the base alignment)
-inline size_t ace_tc_bytes(int tcm, int L, int NP, int n, int cap, int tile_max, int qb, int nbuf) {
+inline size_t ace_tc_bytes(int tcm, int L, int rows, int NP, int n, int cap, int tile_max, int qb, int nbuf) {
     const int kp = (n * n + 15) & ~15;
     const size_t zbytes = (size_t)(TC_M / 8) * (kp / 8) * TC_LBO_A;
-    const AceLay lay(tile_max, cap, n, qb, L, NP, 4, TC_ACE_WARPS, nbuf);
+    const AceLay lay(tile_max, cap, n, qb, L, rows, NP, 4, TC_ACE_WARPS, nbuf);
     return 128 + (size_t)(tcm == 2 ? 2 : 1) * zbytes + (size_t)lay.total;
 }
 
 // launch shape: one or two tile buffers, whichever lets more CTAs share an SM
 // (two on a tie: the next tile then streams in during the current one); as
 // many resident CTAs as fit (each holds 32 TMEM columns of 512)
-template <int L, int NP, int TCM>
+template <int L, int NP, int QB, int TCM>
 inline cudaError_t ace_tc_shape(int n, int cap, int tile_max, int qb, size_t* smem, int* grid, int* nbuf) {
-    const void* kern = (const void*)k_ace_tc<L, NP, TCM>;
+    const void* kern = (const void*)k_ace_tc<L, NP, QB, TCM>;
+    constexpr int ROWS = nu3_rows(L);
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -90,7 +91,7 @@ inline cudaError_t ace_tc_shape(int n, int cap, int tile_max, int qb, size_t* sm
     int best = 0, best_nb = 0;
     size_t best_bytes = 0;
     for (int nb = 2; nb >= 1; --nb) {
-        const size_t bytes = ace_tc_bytes(TCM, L, NP, n, cap, tile_max, qb, nb);
+        const size_t bytes = ace_tc_bytes(TCM, L, ROWS, NP, n, cap, tile_max, qb, nb);
         if (bytes + fa.sharedSizeBytes > (size_t)optin) continue;
         e = raise_smem_limit(kern, bytes);
         if (e != cudaSuccess) return e;
@@ -121,50 +122,40 @@ inline cudaError_t ace_tc_shape(int n, int cap, int tile_max, int qb, size_t* sm
     return cudaSuccess;
 }
 
-template <int NP, int TCM>
+template <int NP, int QB, int TCM>
 inline cudaError_t ace_tc_cfg_l(int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid, int* nbuf) {
     switch (L) {
-        case 0: return ace_tc_shape<0, NP, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
-        case 1: return ace_tc_shape<1, NP, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
-        case 2: return ace_tc_shape<2, NP, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
-        case 3: return ace_tc_shape<3, NP, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
-        case 4: return ace_tc_shape<4, NP, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
-        case 5: return ace_tc_shape<5, NP, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
-        case 6: return ace_tc_shape<6, NP, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
+        case 0: return ace_tc_shape<0, NP, QB, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
+        case 1: return ace_tc_shape<1, NP, QB, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
+        case 2: return ace_tc_shape<2, NP, QB, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
+        case 3: return ace_tc_shape<3, NP, QB, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
+        case 4: return ace_tc_shape<4, NP, QB, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
+        case 5: return ace_tc_shape<5, NP, QB, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
+        case 6: return ace_tc_shape<6, NP, QB, TCM>(n, cap, tile_max, qb, smem, grid, nbuf);
     }
     return cudaErrorInvalidValue;
 }
 
-template <int TCM>
-inline cudaError_t ace_tc_cfg(int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid, int* nbuf) {
-    if (n <= 4) return ace_tc_cfg_l<4, TCM>(L, n, cap, tile_max, qb, smem, grid, nbuf);
-    if (n <= 8) return ace_tc_cfg_l<8, TCM>(L, n, cap, tile_max, qb, smem, grid, nbuf);
-    if (n <= 12) return ace_tc_cfg_l<12, TCM>(L, n, cap, tile_max, qb, smem, grid, nbuf);
-    return ace_tc_cfg_l<16, TCM>(L, n, cap, tile_max, qb, smem, grid, nbuf);
-}
-
-template <int NP, int TCM>
+template <int NP, int QB, int TCM>
 inline void ace_tc_launch_l(const Dev& d, const AceTab<float>& tab, int L, size_t smem, int grid, int nbuf,
                             cudaStream_t s) {
     constexpr int T = TC_ACE_WARPS * 32;
     switch (L) {
-        case 0: k_ace_tc<0, NP, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
-        case 1: k_ace_tc<1, NP, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
-        case 2: k_ace_tc<2, NP, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
-        case 3: k_ace_tc<3, NP, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
-        case 4: k_ace_tc<4, NP, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
-        case 5: k_ace_tc<5, NP, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
-        case 6: k_ace_tc<6, NP, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
+        case 0: k_ace_tc<0, NP, QB, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
+        case 1: k_ace_tc<1, NP, QB, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
+        case 2: k_ace_tc<2, NP, QB, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
+        case 3: k_ace_tc<3, NP, QB, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
+        case 4: k_ace_tc<4, NP, QB, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
+        case 5: k_ace_tc<5, NP, QB, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
+        case 6: k_ace_tc<6, NP, QB, TCM><<<grid, T, smem, s>>>(d, tab, nbuf); break;
     }
 }
 
-template <int TCM>
-inline void ace_tc_launch(const Dev& d, const AceTab<float>& tab, int L, size_t smem, int grid, int nbuf,
-                          cudaStream_t s) {
-    if (tab.np == 4) ace_tc_launch_l<4, TCM>(d, tab, L, smem, grid, nbuf, s);
-    else if (tab.np == 8) ace_tc_launch_l<8, TCM>(d, tab, L, smem, grid, nbuf, s);
-    else if (tab.np == 12) ace_tc_launch_l<12, TCM>(d, tab, L, smem, grid, nbuf, s);
-    else ace_tc_launch_l<16, TCM>(d, tab, L, smem, grid, nbuf, s);
+// the table of class N
+template <int N, int TCM>
+constexpr AceTcOps ace_tc_ops() {
+    constexpr int NP = (N + 3) / 4 * 4, QB = nu3_qb(N);
+    return {ace_tc_cfg_l<NP, QB, TCM>, ace_tc_launch_l<NP, QB, TCM>, gaunt_upload_module};
 }
 
 }  // namespace mixd

@@ -1,0 +1,8 @@
+// Expensive-potential kernels with the bf16 tensor-core readout for n <= 16 (k_ace_tc.cuh).
+#include "k_ace_tc.cuh"
+
+namespace mixd {
+
+const AceTcOps ace_tc1_n16 = ace_tc_ops<16, 1>();
+
+}  // namespace mixd

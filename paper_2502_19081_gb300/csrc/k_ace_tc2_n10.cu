@@ -1,0 +1,8 @@
+// Expensive-potential kernels with the bf16 hi/lo tensor-core readout for n <= 10 (k_ace_tc.cuh).
+#include "k_ace_tc.cuh"
+
+namespace mixd {
+
+const AceTcOps ace_tc2_n10 = ace_tc_ops<10, 2>();
+
+}  // namespace mixd

@@ -10,6 +10,8 @@
 #include <string>
 #include <vector>
 
+#include "k_ace_ops.h"
+#include "k_nu3.cuh"
 #include "mix_launch.h"
 #include "tc.cuh"
 
@@ -103,19 +105,14 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w) {
 // with l1 <= MIX_MAX_LMAX (the kernels' order of the factors: the third, of
 // smallest l, is contracted densely), by quadrature exact for the degree of
 // the product (Gauss-Legendre in cos(theta) times a uniform grid in phi).  One
-// set serves every potential: the coefficients depend on the l's alone.  Also
-// the ordering the expensive kernels read from constant memory: by m3, m1
-// ascending within a row (m1 | m2 << 8, GE_RUN_END on the last entry of each
-// run of equal m1), with the row offsets of each triple.
+// set serves every potential: the coefficients depend on the l's alone.
 struct GauntAll {
-    std::vector<int> l1, l2, l3;             // the triples
-    std::vector<std::vector<double>> G;      // [t][(m1 d2 + m2) d3 + m3]
-    std::vector<int> row0;                   // [t] first row offset of triple t in rows
-    std::vector<int> rows;                   // entry offsets, 2 l3 + 2 per triple (the last: the end)
-    std::vector<GEnt<float>> ent_f;
+    std::vector<std::vector<double>> G;   // by triple number (tri_l): [(m1 d2 + m2) d3 + m3]
     int index(int a, int b, int c) const {
-        for (size_t t = 0; t < l1.size(); ++t)
-            if (l1[t] == a && l2[t] == b && l3[t] == c) return (int)t;
+        for (int t = 0; t < TRI_COUNT; ++t) {
+            const TriL l = tri_l(t);
+            if (l.l1 == a && l.l2 == b && l.l3 == c) return t;
+        }
         return -1;
     }
 };
@@ -138,67 +135,58 @@ const GauntAll& gaunt_all() {
                 Yq.push_back(Y);
                 wq.push_back(gw[iz] * 2.0 * M_PI / nphi);
             }
-        for (int l3 = 0; l3 <= L; ++l3)
-            for (int l2 = l3; l2 <= L; ++l2)
-                for (int l1 = l2; l1 <= L; ++l1) {
-                    if (((l1 + l2 + l3) & 1) || l1 > l2 + l3) continue;
-                    const int d1 = 2 * l1 + 1, d2 = 2 * l2 + 1, d3 = 2 * l3 + 1;
-                    std::vector<double> G((size_t)d1 * d2 * d3, 0.0);
-                    for (size_t k = 0; k < wq.size(); ++k) {
-                        const std::vector<double>& Y = Yq[k];
-                        for (int m1 = 0; m1 < d1; ++m1)
-                            for (int m2 = 0; m2 < d2; ++m2) {
-                                const double y12 = wq[k] * Y[l1 * l1 + m1] * Y[l2 * l2 + m2];
-                                for (int m3 = 0; m3 < d3; ++m3) G[((size_t)m1 * d2 + m2) * d3 + m3] += y12 * Y[l3 * l3 + m3];
-                            }
+        for (int t = 0; t < TRI_COUNT; ++t) {
+            const TriL l = tri_l(t);
+            const int d1 = 2 * l.l1 + 1, d2 = 2 * l.l2 + 1, d3 = 2 * l.l3 + 1;
+            std::vector<double> G((size_t)d1 * d2 * d3, 0.0);
+            for (size_t k = 0; k < wq.size(); ++k) {
+                const std::vector<double>& Y = Yq[k];
+                for (int m1 = 0; m1 < d1; ++m1)
+                    for (int m2 = 0; m2 < d2; ++m2) {
+                        const double y12 = wq[k] * Y[l.l1 * l.l1 + m1] * Y[l.l2 * l.l2 + m2];
+                        for (int m3 = 0; m3 < d3; ++m3) G[((size_t)m1 * d2 + m2) * d3 + m3] += y12 * Y[l.l3 * l.l3 + m3];
                     }
-                    g.l1.push_back(l1);
-                    g.l2.push_back(l2);
-                    g.l3.push_back(l3);
-                    g.row0.push_back((int)g.rows.size());
-                    for (int m3 = 0; m3 < d3; ++m3) {
-                        g.rows.push_back((int)g.ent_f.size());
-                        for (int m1 = 0; m1 < d1; ++m1) {
-                            int last = -1;
-                            for (int m2 = 0; m2 < d2; ++m2) {
-                                const double v = G[((size_t)m1 * d2 + m2) * d3 + m3];
-                                if (std::fabs(v) <= GAUNT_ZERO) continue;
-                                last = (int)g.ent_f.size();
-                                GEnt<float> ef;
-                                std::memset(&ef, 0, sizeof ef);
-                                ef.pk = m1 | (m2 << 8);
-                                ef.g = (float)v;
-                                g.ent_f.push_back(ef);
-                            }
-                            if (last >= 0) g.ent_f[last].pk |= GE_RUN_END;
-                        }
-                    }
-                    g.rows.push_back((int)g.ent_f.size());
-                    g.G.push_back(std::move(G));
-                }
-        // one zero entry past the last, which the kernels' prefetch may read
-        GEnt<float> ef;
-        std::memset(&ef, 0, sizeof ef);
-        g.ent_f.push_back(ef);
+            }
+            g.G.push_back(std::move(G));
+        }
         return g;
     }();
     return tab;
 }
 
-// Copies the table into the constant memory of each float kernel module on
-// the current device, once per device.
-int gaunt_upload() {
+// Copies the coefficients of the compile-time pattern (k_nu3.cuh: by triple,
+// m2, m3, then the one or two m1) into the constant memory of the module that
+// serves tcm and n_rad, once per device and module (loading the other modules
+// would cost every program their load time).  A non-zero coefficient outside
+// the pattern would be lost: MIX_EINVAL.
+int gaunt_upload(int tcm, int n_rad) {
     static std::mutex mu;
     static std::vector<int> done;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return MIX_ECUDA;
+    const int key = (dev * 3 + tcm) * 8 + ace_class(n_rad);
     std::lock_guard<std::mutex> lock(mu);
-    if (std::find(done.begin(), done.end(), dev) != done.end()) return MIX_OK;
-    const GauntAll& g = gaunt_all();
-    if ((int)g.ent_f.size() > GAUNT_ENT_CAP || (int)g.rows.size() > GAUNT_ROW_CAP) return MIX_EINVAL;
-    const cudaError_t e = ace_gaunt_upload(g.ent_f.data(), (int)g.ent_f.size(), g.rows.data(), (int)g.rows.size());
-    if (e != cudaSuccess) return MIX_ECUDA;
-    done.push_back(dev);
+    if (std::find(done.begin(), done.end(), key) != done.end()) return MIX_OK;
+    const GauntAll& ga = gaunt_all();
+    std::vector<float> v;
+    for (int t = 0; t < TRI_COUNT; ++t) {
+        const TriL l = tri_l(t);
+        const int d2 = 2 * l.l2 + 1, d3 = 2 * l.l3 + 1;
+        size_t kept = 0, nonzero = 0;
+        for (int m2 = -l.l2; m2 <= l.l2; ++m2)
+            for (int m3 = -l.l3; m3 <= l.l3; ++m3)
+                for (int k = 0; k < gp_count(l.l1, m2, m3); ++k) {
+                    const int m1 = gp_m1(l.l1, m2, m3, k) + l.l1;
+                    const double x = ga.G[t][((size_t)m1 * d2 + m2 + l.l2) * d3 + m3 + l.l3];
+                    const bool nz = std::fabs(x) > GAUNT_ZERO;
+                    v.push_back(nz ? (float)x : 0.f);
+                    kept += nz;
+                }
+        for (double x : ga.G[t]) nonzero += std::fabs(x) > GAUNT_ZERO;
+        if (kept != nonzero) return MIX_EINVAL;
+    }
+    if (ace_gaunt_upload(tcm, n_rad, v.data(), (int)v.size()) != cudaSuccess) return MIX_ECUDA;
+    done.push_back(key);
     return MIX_OK;
 }
 
@@ -235,14 +223,13 @@ double bf16_value(uint16_t b) {
 
 // The nu = 3 tables as one tile per l-triple (layout in AceTileHdr): W3 holds
 // the symmetrised coefficients [t][q1 q2][q3], tau the triples (l1, l2, l3,
-// first offset row), tcg each triple's first row in the constant-memory
-// Gaunt table, goff/gidx/gval the Gaunt entries in three orderings (the tile
-// takes the one by m2).
+// first offset row), tnum each triple's number (tri_l), goff/gidx/gval the
+// Gaunt entries in three orderings (float64 tiles take those by m2 and m3).
 // tcm (tensor-core readout): 1 appends W as the bf16 B operand, 2 also its
 // bf16 remainders; tiles are then 128-byte multiples.
 template <typename T>
 std::vector<unsigned char> ace_tiles(int n, int np, const std::vector<int>& tau, const std::vector<int>& tmode,
-                                     const std::vector<int>& tcg, const std::vector<int>& goff,
+                                     const std::vector<int>& tnum, const std::vector<int>& goff,
                                      const std::vector<int>& gidx, const std::vector<double>& gval,
                                      const std::vector<double>& W3, std::vector<int>& off, int& tile_max,
                                      int tcm = 0) {
@@ -254,23 +241,23 @@ std::vector<unsigned char> ace_tiles(int n, int np, const std::vector<int>& tau,
     tile_max = 0;
     for (int t = 0; t < ntau; ++t) {
         const int l1 = tau[4 * t], l2 = tau[4 * t + 1], l3 = tau[4 * t + 2], gb = tau[4 * t + 3];
-        // the ordering by m2 only (the kernels read the ordering by m3 from the
-        // constant-memory table): its 2 l2 + 2 offset rows follow the 2 l3 + 2
-        // of the ordering by m3 and the 2 l1 + 2 of the ordering by m1
+        // the ordering by m2: its 2 l2 + 2 offset rows follow the 2 l3 + 2 of the
+        // ordering by m3 and the 2 l1 + 2 of the ordering by m1
         const int r2 = gb + (2 * l3 + 2) + (2 * l1 + 2), rows = 2 * l2 + 2;
-        const int e0 = goff[r2], ne = goff[r2 + rows - 1] - e0;
+        const int e0 = goff[r2], ne = sizeof(T) == 8 ? goff[r2 + rows - 1] - e0 : 0;
         AceTileHdr h;
         std::memset(&h, 0, sizeof h);
         h.l1 = l1;
         h.l2 = l2;
         h.l3 = l3;
         h.mode = tmode[t];
-        h.cg = tcg[t];
-        size_t o = sizeof(AceTileHdr) + (size_t)n * n * np * sizeof(T);
+        h.tri = tnum[t];
+        const int wr = sizeof(T) == 8 ? n : np;   // rows W[q1 wr + q2][q3]
+        size_t o = sizeof(AceTileHdr) + (size_t)n * wr * np * sizeof(T);
         h.o_ge = (int)o;
         o += (size_t)ne * sizeof(GEnt<T>);
         h.o_go = (int)o;
-        o += (size_t)rows * sizeof(int);
+        if (sizeof(T) == 8) o += (size_t)rows * sizeof(int);
         o = (o + 15) & ~(size_t)15;
         h.o_wb = 0;
         if (tcm) {
@@ -284,7 +271,8 @@ std::vector<unsigned char> ace_tiles(int n, int np, const std::vector<int>& tau,
         std::memcpy(tile.data(), &h, sizeof h);
         T* W = reinterpret_cast<T*>(tile.data() + sizeof(AceTileHdr));
         for (int q12 = 0; q12 < n * n; ++q12)
-            for (int q3 = 0; q3 < n; ++q3) W[(size_t)q12 * np + q3] = (T)W3[((size_t)t * n * n + q12) * n + q3];
+            for (int q3 = 0; q3 < n; ++q3)
+                W[((size_t)(q12 / n) * wr + q12 % n) * np + q3] = (T)W3[((size_t)t * n * n + q12) * n + q3];
         for (int k = 0; k < ne; ++k) {
             GEnt<T> g;
             std::memset(&g, 0, sizeof g);
@@ -292,12 +280,12 @@ std::vector<unsigned char> ace_tiles(int n, int np, const std::vector<int>& tau,
             g.g = (T)gval[e0 + k];
             std::memcpy(tile.data() + h.o_ge + (size_t)k * sizeof g, &g, sizeof g);
         }
-        for (int r = 0; r < rows; ++r) {
+        for (int r = 0; sizeof(T) == 8 && r < rows; ++r) {
             const int v = goff[r2 + r] - e0;
             std::memcpy(tile.data() + h.o_go + (size_t)r * sizeof(int), &v, sizeof v);
         }
         if (sizeof(T) == 8) {
-            // the ordering by m3, with the run-end flags of the constant table
+            // the ordering by m3, with its run-end flags
             const int r3 = 2 * l3 + 2, f0 = goff[gb], nf = goff[gb + r3 - 1] - f0;
             size_t o3 = tile.size();
             h.o_ge3 = (int)o3;
@@ -449,7 +437,7 @@ int build_tables(mix_ctx* c, const mix_ace* a, const mix_spline* sp) {
     std::vector<double> W3;
     std::vector<int> goff, gidx;
     std::vector<double> gval;
-    std::vector<int> tcg;   // per triple: its first row in the constant-memory table
+    std::vector<int> tnum;   // per triple: its number
     if (a->nu_max >= 3) {
         const GauntAll& ga = gaunt_all();
         // The potential indexes its coefficients by the ascending triple
@@ -467,7 +455,7 @@ int build_tables(mix_ctx* c, const mix_ace* a, const mix_spline* sp) {
                     const int tg = ga.index(l1, l2, l3);
                     if (tg < 0) return fail(c, MIX_EINVAL, "l-triple beyond the Gaunt table");
                     const std::vector<double>& G = ga.G[tg];
-                    tcg.push_back(ga.row0[tg]);
+                    tnum.push_back(tg);
                     auto nz_ = [&](int m1, int m2, int m3) { return std::fabs(G[((size_t)m1 * d2 + m2) * d3 + m3]) > GAUNT_ZERO; };
                     auto gv = [&](int m1, int m2, int m3) { return G[((size_t)m1 * d2 + m2) * d3 + m3]; };
                     const int t = (int)(tau.size() / 4);
@@ -589,20 +577,18 @@ int build_tables(mix_ctx* c, const mix_ace* a, const mix_spline* sp) {
         if (mref == 0) fr += 2.0 * nnz * nn * nn;
         c->nu3_flops_ref += fr;
     }
-    // q2 block of a lane unit (q1, qb consecutive q2) in the nu = 3 pass: every
-    // pass of the warp over its units repeats the per-m3 work (a warp-wide
-    // reduction among it), so choose the block with the least estimated work,
-    // passes x (2 qb np multiply-adds + ~120 instructions of per-m3 overhead):
-    // 4 or 2 (and for float 6 as well where np = 12: n = 12 gives 24 units in
-    // one pass instead of 36 in two)
-    {
-        std::vector<int> cand = {4, 2};
-        if (c->precision != MIX_FP64 && np == 12) cand.push_back(6);
+    // q2 block of a lane unit (q1, qb consecutive q2) in the nu = 3 pass.  Float
+    // has one per instantiation class (nu3_qb).  Float64: every pass of the warp
+    // over its units repeats the per-m3 work (a warp-wide reduction among it), so
+    // choose 4 or 2, whichever has the least estimated work, passes x (2 qb np
+    // multiply-adds + ~120 instructions of per-m3 overhead)
+    c->qb = nu3_qb(n);
+    if (c->precision == MIX_FP64) {
         double best = 0.0;
-        for (int qb : cand) {
+        for (int qb : {4, 2}) {
             const int units = n * (np / qb);
             const double cost = (double)((units + 31) / 32) * (2.0 * qb * np + 120.0);
-            if (qb == cand[0] || cost < best - 1e-9) {
+            if (qb == 4 || cost < best - 1e-9) {
                 best = cost;
                 c->qb = qb;
             }
@@ -628,16 +614,20 @@ int build_tables(mix_ctx* c, const mix_ace* a, const mix_spline* sp) {
     if (c->precision == MIX_FP64) {
         c->o_c1 = A.put(c1);
         c->o_S2 = A.put(S2);
-        c->o_tiles = A.put(ace_tiles<double>(n, np, tau, tmode, tcg, goff, gidx, gval, W3, toff, c->tile_max));
+        c->o_tiles = A.put(ace_tiles<double>(n, np, tau, tmode, tnum, goff, gidx, gval, W3, toff, c->tile_max));
         c->o_ylmk = A.put(ylmk);
         c->o_pair = A.put(pair);
         c->o_sc2 = A.put(sc2);
         c->o_sc3 = A.put(sc3);
     } else {
         c->o_c1 = A.put(conv<float>(c1));
-        c->o_S2 = A.put(conv<float>(S2));
+        std::vector<float> S2p((size_t)L1 * n * np, 0.f);   // rows padded to np
+        for (int l = 0; l <= L; ++l)
+            for (int p = 0; p < n; ++p)
+                for (int q = 0; q < n; ++q) S2p[((size_t)l * n + p) * np + q] = (float)S2[((size_t)l * n + p) * n + q];
+        c->o_S2 = A.put(S2p);
         c->ace_tcm = c->ntau == 0 ? 0 : (c->precision == MIX_BF16 ? 1 : (c->precision == MIX_BF16_SPLIT ? 2 : 0));
-        c->o_tiles = A.put(ace_tiles<float>(n, np, tau, tmode, tcg, goff, gidx, gval, W3, toff, c->tile_max, c->ace_tcm));
+        c->o_tiles = A.put(ace_tiles<float>(n, np, tau, tmode, tnum, goff, gidx, gval, W3, toff, c->tile_max, c->ace_tcm));
         c->o_ylmk = A.put(conv<float>(ylmk));
         c->o_pair = A.put(conv<float>(pair));
         c->o_sc2 = A.put(conv<float>(sc2));
@@ -658,7 +648,7 @@ void fill_tabs(mix_ctx* c, unsigned char* base, AceTab<T>& at, SplTab<T>& st) {
     at.np = c->np;
     at.rc = c->ace_rc;
     at.c1 = reinterpret_cast<const T*>(base + c->o_c1);
-    at.S2 = reinterpret_cast<const T*>(base + c->o_S2);
+    at.S2 = at.S2p = reinterpret_cast<const T*>(base + c->o_S2);
     at.tiles = base + c->o_tiles;
     at.tile_off = reinterpret_cast<const int*>(base + c->o_toff);
     at.tile_max = c->tile_max;
@@ -1034,7 +1024,7 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
     std::memset(&c->regions, 0, sizeof c->regions);
     c->regions.blend = opt->blend;
     int st = build_tables(c, a, sp);
-    if (st == MIX_OK && c->ntau > 0) st = gaunt_upload();
+    if (st == MIX_OK && c->ntau > 0 && c->precision != MIX_FP64) st = gaunt_upload(c->ace_tcm, c->n);
     if (st) {
         delete c;
         return st;
@@ -1043,7 +1033,7 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
     // large float systems: CTAs of 4 warps share the coefficient tiles between
     // twice the atoms, so more warps fit an SM (their expensive sets are many
     // waves large); small sets keep groups of 2, which spread them more evenly
-    c->ace_wn = (c->precision != MIX_FP64 && sys->n_atoms >= 50000) ? ACE_MAX_WARPS : ACE_GROUP;
+    c->ace_wn = (c->precision != MIX_FP64 && sys->n_atoms >= 20000) ? ACE_MAX_WARPS : ACE_GROUP;
     cudaError_t e = c->ace_tcm
                         ? ace_tc_configure(c->ace_tcm, c->L, c->n, c->cap, c->tile_max, c->qb, &c->ace_smem,
                                            &c->ace_grid, &c->ace_nbuf)
@@ -1783,7 +1773,6 @@ int fused_build(mix_batch* b) {
         regs[s] = b->m[s]->regions;
     }
     // expensive groups
-    auto npad = [](int n) { return n <= 4 ? 4 : n <= 8 ? 8 : n <= 12 ? 12 : 16; };
     std::vector<int> egroup(ns), elast(ns, 0);
     b->groups.clear();
     std::vector<int64_t> gatoms;
@@ -1791,7 +1780,7 @@ int fused_build(mix_batch* b) {
         const mix_ctx* c = b->m[s];
         int g = -1;
         for (size_t k = 0; k < b->groups.size(); ++k)
-            if (b->groups[k].L == c->L && npad(b->groups[k].n) == npad(c->n)) g = (int)k;
+            if (b->groups[k].L == c->L && ace_class(b->groups[k].n) == ace_class(c->n)) g = (int)k;
         if (g < 0) {
             b->groups.push_back({c->L, c->n, c->cap, c->tile_max, c->qb, 0, 0, 0});
             gatoms.push_back(0);

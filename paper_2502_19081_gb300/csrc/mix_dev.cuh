@@ -222,12 +222,12 @@ template <> struct Vec4<float> { using type = float4; };
 // group (a warp per atom), and the CTAs per SM each kernel is compiled for.
 // Two atoms a CTA spread a small expensive set evenly over the SMs (1396
 // atoms: at most 10 a SM against 12 with groups of 4); the float kernel's
-// ~36 KB of shared memory a CTA (Fe, n = 10, lmax = 4, 128 neighbour slots)
-// leaves room for 6 CTAs, the float64 kernel's ~71 KB for 3.
+// ~26 KB of shared memory a CTA (Fe, n = 10, lmax = 4, 128 neighbour slots) and
+// 128 registers a thread leave room for 8 CTAs, the float64 kernel's ~54 KB for 4.
 // A single context's CTA may also hold 4 warps (ACE_MAX_WARPS): the two
 // tile buffers are then shared by twice the atoms, which lets more warps fit an
-// SM when the evaluated set is many waves large (the 256,000-atom cylinder:
-// 3 CTAs of 4 warps against 5 of 2).  The batched kernel keeps groups of 2.
+// SM when the evaluated set is many waves large (n = 12, lmax = 5: 4 CTAs of 4
+// warps against 6 of 2).  The batched kernel keeps groups of 2.
 constexpr int ACE_GROUP = 2;
 constexpr int ACE_MAX_WARPS = 4;
 template <typename T>
@@ -236,7 +236,7 @@ __host__ __device__ constexpr int ace_warps() {
 }
 template <typename T>
 __host__ __device__ constexpr int ace_min_ctas() {
-    return sizeof(T) == 4 ? 6 : 2;
+    return sizeof(T) == 4 ? 8 : 2;
 }
 // the same register budget for CTAs of ACE_MAX_WARPS warps
 template <typename T>
@@ -253,7 +253,7 @@ constexpr int TC_MIN_CTAS = 3;
 
 // One Gaunt coefficient with the packed m indices of its two other factors
 // (ma | mb << 8, 0-based; the ordering by m3 also flags run ends, see
-// AceTileHdr), loaded as one 8- or 16-byte word.
+// AceTileHdr), loaded as one 16-byte word (float64 tiles).
 constexpr int GE_RUN_END = 1 << 24;   // last entry of a run of equal m1 in an m3 row
 
 template <typename T>
@@ -263,17 +263,17 @@ struct __align__(sizeof(T) == 4 ? 8 : 16) GEnt {
 };
 
 // Header of one l-triple tile of the nu = 3 tables.  A tile is one contiguous,
-// 16-byte aligned block (a multiple of 16 bytes) holding, at these byte offsets:
-//   W[q1 q2][q3]  (n*n rows of np, zero padded) right after the header,
-//   the Gaunt entries GEnt<T> ordered by m2 (m1 | m3 << 8) at o_ge,
-//   their offset rows (2 l2 + 2 ints: the first entry of each m2, then the
-//     end; entry indices relative to o_ge) at o_go.
-// The ordering by m3 (m1 | m2 << 8, m1 ascending within a row, GE_RUN_END on
-// the last entry of each run of equal m1) is the same for every potential and
-// sits in constant memory, from row cg on; float64 tiles also hold it, at
-// o_ge3 with its 2 l3 + 2 offset rows at o_go3 (the float64 kernel reads it
-// there: its entries are twice the size, and where few warps run a shared-
-// memory read is the quicker).
+// 16-byte aligned block (a multiple of 16 bytes) holding W[q1 q2][q3] right after
+// the header, rows of np: float64 n*n of them (q1 n + q2), float n*np (q1 np + q2),
+// zero beyond n.  Float tiles hold no Gaunt
+// coefficients: the kernel has the triple's pattern compiled in (k_nu3.cuh, by
+// the triple number tri).  Float64 tiles also hold, at these byte offsets:
+//   the Gaunt entries GEnt<T> ordered by m2 (m1 | m3 << 8) at o_ge and their
+//   offset rows (2 l2 + 2 ints: the first entry of each m2, then the end;
+//   entry indices relative to o_ge) at o_go;
+//   the ordering by m3 (m1 | m2 << 8, m1 ascending within a row, GE_RUN_END on
+//   the last entry of each run of equal m1) at o_ge3 with its 2 l3 + 2 offset
+//   rows at o_go3.
 // mode: 0 l's distinct, 1 l1 == l2, 2 l2 == l3, 3 all equal (W symmetrised over
 // the matching n indices).  Tiles of the tensor-core readout (bf16 modes) also
 // hold, at o_wb (128-byte aligned; 0 otherwise), W as the MMA's B operand: 16
@@ -283,16 +283,12 @@ struct __align__(sizeof(T) == 4 ? 8 : 16) GEnt {
 struct AceTileHdr {
     int l1, l2, l3, mode;
     int o_ge, o_go, bytes, o_wb;
-    int cg;             // first row of the triple in the constant-memory Gaunt table
-    int o_ge3, o_go3;   // float64 tiles: their own ordering by m3 and its offset rows (0 in float tiles)
+    int tri;            // number of the triple (tri_l)
+    int o_ge3, o_go3;
     int pad;            // 16-byte multiple: W follows
 };
 
-// The constant-memory Gaunt table of the expensive kernels (every l-triple
-// l1 >= l2 >= l3 up to MIX_MAX_LMAX, ordered by m3; built on the host): entry
-// and row capacities, and the magnitude below which a quadrature value is zero.
-constexpr int GAUNT_ENT_CAP = 2048;
-constexpr int GAUNT_ROW_CAP = 192;
+// magnitude below which a quadrature value of a Gaunt coefficient is zero
 constexpr double GAUNT_ZERO = 1e-12;
 
 template <typename T>
@@ -303,7 +299,8 @@ struct AceTab {
     int tile_max;       // bytes of the largest nu = 3 tile
     double rc;
     const T* c1;        // [n]
-    const T* S2;        // [L+1][n][n]  symmetric: W2 + W2^T, W2 upper-triangular c2
+    const T* S2;        // [L+1][n][n]  symmetric: W2 + W2^T, W2 upper-triangular c2 (float64)
+    const T* S2p;       // [L+1][n][np] the same, rows zero padded (float)
     const unsigned char* tiles;  // the ntau l-triple tiles, back to back
     const int* tile_off;         // [ntau + 1] byte offset of each tile, then the end
     const T* ylmk;      // [nlm] normalisation of Y_lm times sqrt2 for m != 0

@@ -13,17 +13,13 @@ void launch_build(const Dev& d, cudaStream_t s);
 void launch_sets(const Dev& d, const Regions& r, const SeedRule& sr, cudaStream_t s);
 int sets_launches(const SeedRule& sr);   // kernels launch_sets enqueues
 
-// expensive potential (k_ace.cuh, k_ace_f32.cu, k_ace_f64.cu); returns cudaSuccess or the launch error;
+// expensive potential (k_ace.cuh, k_ace_f32_n*.cu, k_ace_f64.cu); returns cudaSuccess or the launch error;
 // wn: warps (atoms) a CTA, ACE_GROUP or ACE_MAX_WARPS
 cudaError_t ace_configure(int precision, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid,
                           int wn);
 void launch_ace(const Dev& d, const void* tab, int precision, int L, size_t smem, int grid, int wn, cudaStream_t s);
-cudaError_t ace_configure_f32(int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid, int wn);
-cudaError_t ace_configure_f64(int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid, int wn);
-void launch_ace_f32(const Dev& d, const void* tab, int L, size_t smem, int grid, int wn, cudaStream_t s);
-void launch_ace_f64(const Dev& d, const void* tab, int L, size_t smem, int grid, int wn, cudaStream_t s);
 
-// expensive potential with the tensor-core readout (k_ace_tc.cu; float tables
+// expensive potential with the tensor-core readout (k_ace_tc.cuh, k_ace_tc*_n*.cu; float tables
 // with the bf16 operand sections): tcm 1 bf16, 2 bf16 hi/lo.  *nbuf: tile
 // buffers that fit shared memory (2, else 1); cudaErrorInvalidValue when even
 // one does not fit
@@ -31,12 +27,9 @@ cudaError_t ace_tc_configure(int tcm, int L, int n, int cap, int tile_max, int q
                              int* nbuf);
 void launch_ace_tc(const Dev& d, const void* tab, int tcm, int L, size_t smem, int grid, int nbuf, cudaStream_t s);
 
-// the Gaunt table of the float expensive kernels into the constant memory of
-// every module that holds them, on the current device (k_ace_f64.cu dispatches)
-cudaError_t ace_gaunt_upload(const void* ent_f, int n_ent, const int* rows, int n_rows);
-cudaError_t ace_gaunt_upload_f32(const void* ent_f, int n_ent, const int* rows, int n_rows);
-cudaError_t ace_gaunt_upload_tc1(const void* ent_f, int n_ent, const int* rows, int n_rows);
-cudaError_t ace_gaunt_upload_tc2(const void* ent_f, int n_ent, const int* rows, int n_rows);
+// the Gaunt coefficients into the constant memory of the module that holds the
+// float expensive kernels of tcm and n_rad, on the current device
+cudaError_t ace_gaunt_upload(int tcm, int n_rad, const float* g, int n);
 
 // tensor-core building block check (k_tc.cu)
 cudaError_t tc_selftest(const uint16_t* a, const uint16_t* b, int m, int n, int k, float* d, int* status,
@@ -91,14 +84,8 @@ void launch_disp_batch(const BatchPlan& p, cudaStream_t s, int integrate, double
 void launch_build_batch(const BatchPlan& p, cudaStream_t s);
 void launch_sets_batch(const BatchPlan& p, cudaStream_t s);
 cudaError_t ace_batch_configure(int precision, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid);
-cudaError_t ace_batch_configure_f32(int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid);
-cudaError_t ace_batch_configure_f64(int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid);
 void launch_ace_batch(int precision, const Dev* devs, const void* tabs, const int2* list, const int* count, int n,
                       int L, size_t smem, int grid, cudaStream_t s);
-void launch_ace_batch_f32(const Dev* devs, const void* tabs, const int2* list, const int* count, int n, int L,
-                          size_t smem, int grid, cudaStream_t s);
-void launch_ace_batch_f64(const Dev* devs, const void* tabs, const int2* list, const int* count, int n, int L,
-                          size_t smem, int grid, cudaStream_t s);
 cudaError_t spline_batch_configure(int precision, int lpa, size_t* smem, int* grid);
 void launch_spline_batch(int precision, int lpa, const Dev* devs, const void* tabs, const int2* list,
                          const int* count, int uniform, size_t smem, int grid, cudaStream_t s);
