@@ -13,7 +13,10 @@
  *  - Return value: MIX_OK (0) or a negative MIX_E* code; no exceptions cross
  *    the boundary.  mix_strerror() names a code; mix_last_error() gives the
  *    context's last message.
- *  - Device work is enqueued asynchronously on the context's stream.  Errors
+ *  - Device work is enqueued asynchronously on the context's stream.  The kernel
+ *    that opens an evaluation is a cooperative launch (its blocks meet at grid
+ *    barriers; every wait is bounded and reports MIX_ETIMEOUT, after which the
+ *    context's kernels do nothing).  Errors
  *    detected by kernels (capacity overflow, non-finite values, an atom leaving
  *    a non-periodic box) surface at the next synchronising call: mix_sync(),
  *    the mix_get_* exports, mix_get_state() and the *_host entry points.
@@ -292,9 +295,10 @@ const char* mix_last_error(const mix_ctx* ctx);
 /* kernels and to state roofline fractions.                                   */
 
 /* Kernel groups of one force evaluation, in launch order. */
-#define MIX_PHASE_DISP 0     /* first half-kick, drift, skin test */
-#define MIX_PHASE_LISTS 1    /* cell list and neighbour list (no-ops unless rebuilding) */
-#define MIX_PHASE_SETS 2     /* weights, buffers, compaction */
+#define MIX_PHASE_DISP 0     /* first half-kick, drift, skin test; the lists when they are
+                                rebuilt; weights, buffers, compaction (one kernel) */
+#define MIX_PHASE_LISTS 1    /* empty: part of the kernel above */
+#define MIX_PHASE_SETS 2     /* empty: part of the kernel above */
 #define MIX_PHASE_EXP 3      /* expensive potential (one kernel) */
 #define MIX_PHASE_CHEAP 4    /* cheap potential (one kernel) */
 #define MIX_PHASE_GATHER 5   /* gather, blend, second half-kick (one kernel) */
@@ -321,8 +325,9 @@ typedef struct {
     int launches_per_evaluation;
     int64_t launches;       /* kernels enqueued since mix_bind */
     int gather_grid;        /* CTAs of the gather kernel */
-    int build_grid;         /* CTAs of the neighbour-list kernel */
-    int buffer_grid;        /* CTAs of the buffer-scan kernel */
+    int build_grid;         /* 0: the lists are built by the kernel of buffer_grid */
+    int buffer_grid;        /* limit on the CTAs of the kernel that moves the atoms, builds the
+                               lists and forms the sets (0: as many as are resident) */
     int exp_tensor_cores;   /* 1: the nu = 3 readout runs on the tensor cores (bf16 modes) */
     double tc_flops_per_atom;  /* algorithmic flops of that readout, V = Z W: sum over
                                   l-triples of 2 (2 l3 + 1) n^3 per evaluated atom */
@@ -382,7 +387,7 @@ int mix_tc_selftest(const void* a_dev, const void* b_dev, int m, int n, int k, f
  * neighbour count measured so far fills at most two thirds of its on-chip
  * slots; a later overflow reports MIX_EOVERFLOW and widens the groups again),
  * the persistent grid of each potential kernel and the grids of the gather and
- * buffer kernels, and keeps the fastest (reported by mix_get_info); the
+ * of the kernel that forms the sets, and keeps the fastest (reported by mix_get_info); the
  * forces do not depend on any of them.
  * reps: timed evaluations per candidate (median). */
 int mix_tune(mix_ctx* ctx, int reps);

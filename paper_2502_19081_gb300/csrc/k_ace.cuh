@@ -959,7 +959,7 @@ __global__ void __launch_bounds__(ACE_MAX_WARPS * 32, ace_min_ctas_max<T>()) k_a
     const int WN = (int)(blockDim.x >> 5);   // ACE_GROUP or ACE_MAX_WARPS atoms a CTA
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_g;
-    const int count = d.status[SW_NEXP];
+    const int count = list_ok(d) ? d.status[SW_NEXP] : 0;
     const int ng = (count + WN - 1) / WN;
     for (int g = ace_next_group(d, &s_g); g < ng; g = ace_next_group(d, &s_g))
         ace_group<T, L, NP, QB>(d, tab, g * WN, count, smem_raw, nullptr, WN);

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(TC_ACE_WARPS * 32, TC_MIN_CTAS) k_ace_tc(Dev d
     tc_fence_after();
     tc.tmem = s_tmem;
     tc.bar = smem_u32(&s_bar);
-    const int count = d.status[SW_NEXP];
+    const int count = list_ok(d) ? d.status[SW_NEXP] : 0;
     const int ng = (count + TC_ACE_WARPS - 1) / TC_ACE_WARPS;
     __shared__ int s_g;
     for (int g = ace_next_group(d, &s_g); g < ng; g = ace_next_group(d, &s_g))

@@ -194,6 +194,7 @@ __device__ __forceinline__ void gather_body(const Dev& d, int bx, int gx, int in
 template <typename T, int LPA>
 __global__ void __launch_bounds__(G_WARPS * 32, sizeof(T) == 4 ? 4 : 2) k_gather(Dev d, int integrate, double h, int ga) {
     __shared__ GSum<T> park[G_WARPS * G_ATOMS * 6];
+    if (!list_ok(d)) return;
     gather_body<T, LPA>(d, blockIdx.x, gridDim.x, integrate, h, ga, park);
 }
 

@@ -33,7 +33,8 @@ constexpr size_t NA_O_CELL_ATOMS = na_al(NA_O_CELL_OF + NA_MAX_ATOMS * sizeof(in
 constexpr size_t NA_O_CELL_COUNT = na_al(NA_O_CELL_ATOMS + NA_MAX_ATOMS * sizeof(int));
 constexpr size_t NA_O_CELL_FILL = na_al(NA_O_CELL_COUNT + NA_MAX_CELLS * sizeof(int));
 constexpr size_t NA_O_CELL_START = na_al(NA_O_CELL_FILL + NA_MAX_CELLS * sizeof(int));
-constexpr size_t NA_BYTES = na_al(NA_O_CELL_START + (NA_MAX_CELLS + 1) * sizeof(int));
+constexpr size_t NA_O_BLK = na_al(NA_O_CELL_START + (NA_MAX_CELLS + 1) * sizeof(int));
+constexpr size_t NA_BYTES = na_al(NA_O_BLK + FRONT_MAX_CTAS * sizeof(int));
 
 // the scratch; every GPU that loads the library holds it until exit
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
@@ -41,30 +42,6 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 constexpr int NA_MAX_DEVICES = 64;
 std::mutex g_na_mutex;
 unsigned char* g_na_ptr[NA_MAX_DEVICES] = {};
-
-// Zero what must start at zero (status words, cell counts) and request a build.
-__global__ void k_noalloc_init(int* status, int* cell_count, int ncell) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < SW_COUNT) status[t] = (t == SW_REBUILD) ? 1 : 0;
-    for (int k = t; k < ncell; k += gridDim.x * blockDim.x) cell_count[k] = 0;
-}
-
-// The position checks the context path makes before a build: a non-finite
-// coordinate, or one outside a non-periodic dimension of the box, sets its
-// status bit (the build still runs; every cell index it forms is clamped).
-__global__ void k_noalloc_check(Dev d) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double4 x = d.x[i];
-        if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z))) {
-            set_status(d.status, ST_NONFINITE);
-            continue;
-        }
-        const double xs[3] = {x.x, x.y, x.z};
-        for (int k = 0; k < 3; ++k)
-            if (!d.box.per[k] && (xs[k] < d.box.lo[k] || xs[k] >= d.box.lo[k] + d.box.L[k]))
-                set_status(d.status, ST_OUT_OF_BOX);
-    }
-}
 
 // Device address of the scratch on the current device, looked up once per device.
 int scratch_address(unsigned char** out) {
@@ -122,11 +99,13 @@ extern "C" int mix_neighbours_noalloc(int64_t n_atoms, const double* x_dev, cons
     if (ncell > NA_MAX_CELLS) return MIX_EINVAL;
     d.cells.ncell = (int)ncell;
     d.rlist2 = r_list * r_list;
+    d.nbs = nb_screen(d.rlist2, d.box);
     unsigned char* base = nullptr;
     int st = scratch_address(&base);
     if (st) return st;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     d.status = reinterpret_cast<int*>(base + NA_O_STATUS);
+    d.blk_e = reinterpret_cast<int*>(base + NA_O_BLK);
     d.x = reinterpret_cast<double4*>(base + NA_O_X);
     d.xb = reinterpret_cast<double4*>(base + NA_O_XB);
     d.xf = reinterpret_cast<float4*>(base + NA_O_XF);
@@ -143,16 +122,13 @@ extern "C" int mix_neighbours_noalloc(int64_t n_atoms, const double* x_dev, cons
     d.nnb = nnb_dev;
     d.nbr = nbr_dev;
     d.rev = rev_dev;
-    if (n_atoms > 0 &&
-        cudaMemcpyAsync(d.x, x_dev, (size_t)n_atoms * sizeof(double4), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return MIX_ECUDA;
-    k_noalloc_init<<<64, 256, 0, s>>>(d.status, d.cell_count, d.cells.ncell);
-    if (n_atoms > 0) k_noalloc_check<<<(int)((n_atoms + 255) / 256), 256, 0, s>>>(d);
-    launch_build(d, s);
-    if (cudaGetLastError() != cudaSuccess) return MIX_ECUDA;
+    // status words (the grid barrier's among them) start at zero; the kernel clears the cell counts
+    if (cudaMemsetAsync(d.status, 0, SW_COUNT * sizeof(int), s) != cudaSuccess) return MIX_ECUDA;
+    if (n_atoms > 0 && launch_front_lists(d, reinterpret_cast<const double4*>(x_dev), s) != cudaSuccess) return MIX_ECUDA;
     int status[SW_COUNT];
     if (cudaMemcpyAsync(status, d.status, sizeof status, cudaMemcpyDeviceToHost, s) != cudaSuccess) return MIX_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return MIX_ECUDA;
+    if (status[SW_STATUS] & ST_GRID_TIMEOUT) return MIX_ETIMEOUT;
     if (status[SW_STATUS] & ST_NONFINITE) return MIX_ENUMERIC;
     if (status[SW_STATUS] & ST_OUT_OF_BOX) return MIX_EBOX;
     if (status[SW_STATUS] & ST_NBR_OVERFLOW) return MIX_EOVERFLOW;

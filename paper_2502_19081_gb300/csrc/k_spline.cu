@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 1) k_spli
     spl_stage<T>(c3s, tab.c3w, tab.c2w);
     spl_fill_tq<NB>(tq);
     __syncthreads();
-    const int count = d.status[SW_NCHEAP];
+    const int count = list_ok(d) ? d.status[SW_NCHEAP] : 0;
     const int stride = gridDim.x * SPL_WARPS * G;
     int a = (blockIdx.x * SPL_WARPS + warp) * G + grp;
     const int sub = threadIdx.x & (LPA - 1), cap = d.cap;

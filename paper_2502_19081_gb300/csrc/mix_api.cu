@@ -19,9 +19,8 @@ using namespace mixd;
 
 namespace {
 
-// kernels per evaluation: displacement 1, lists 5, sets 4, expensive 1, cheap 1, gather 1
-// (13 with geometric regions; the seed-atom modes add one or two)
-constexpr int LAUNCHES_PER_EVAL = 13;
+// kernels per evaluation: front (displacement, lists, weights, sets) 1, expensive 1, cheap 1, gather 1
+constexpr int LAUNCHES_PER_EVAL = 4;
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -696,8 +695,8 @@ void layout(mix_ctx* c) {
     c->o_act_c = take(N * 4);
     c->o_pos_e = take(N * 4);
     c->o_pos_c = take(N * 4);
-    c->o_blk_e = take((size_t)c->dev.nblk * 4);
-    c->o_blk_c = take((size_t)c->dev.nblk * 4);
+    c->o_blk_e = take(std::max<size_t>(c->dev.nblk, FRONT_MAX_CTAS) * 4);
+    c->o_blk_c = take(std::max<size_t>(c->dev.nblk, FRONT_MAX_CTAS) * 4);
     c->o_ge = take(N * cap * v4);
     c->o_gc = take(N * cap * v4);
     c->o_gei = take(N * cap * v4);
@@ -719,7 +718,7 @@ int check_stream_error(mix_ctx* c, const char* what) {
     return MIX_OK;
 }
 
-int evals_launches(const mix_ctx* c) { return LAUNCHES_PER_EVAL - 4 + sets_launches(c->seedrule); }
+int evals_launches(const mix_ctx*) { return LAUNCHES_PER_EVAL; }
 
 // the kernels of one evaluation, in order, on stream s (events between the
 // phases when profiling)
@@ -729,11 +728,10 @@ void enqueue_evaluation(mix_ctx* c, cudaStream_t s, int integrate, double dt, in
     const double h = half_kick(dt, c->sys.mass);
     const unsigned ef = captured ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (prof) cudaEventRecordWithFlags(c->ev[0], s, ef);
-    launch_disp(c->dev, s, integrate, dt, h, force_rebuild);
+    launch_front(c->dev, c->regions, c->seedrule, s, integrate, dt, h, force_rebuild);
+    // one kernel: its time is the first phase's, the list and set phases are empty
     if (prof) cudaEventRecordWithFlags(c->ev[1], s, ef);
-    launch_build(c->dev, s);
     if (prof) cudaEventRecordWithFlags(c->ev[2], s, ef);
-    launch_sets(c->dev, c->regions, c->seedrule, s);
     if (prof) cudaEventRecordWithFlags(c->ev[3], s, ef);
     const void* at = c->precision == MIX_FP64 ? (const void*)&c->ace64 : (const void*)&c->ace32;
     const void* st = c->precision == MIX_FP64 ? (const void*)&c->spl64 : (const void*)&c->spl32;
@@ -870,6 +868,7 @@ int read_status(mix_ctx* c) {
     if (st & ST_NONFINITE) return fail(c, MIX_ENUMERIC, "non-finite position or force");
     if (st & ST_OUT_OF_BOX) return fail(c, MIX_EBOX, "an atom left the box in a non-periodic dimension");
     if (st & ST_REV_MISSING) return fail(c, MIX_EINVAL, "asymmetric neighbour list");
+    if (st & ST_GRID_TIMEOUT) return fail(c, MIX_ETIMEOUT, "a wait at a grid barrier gave up");
     if (st & ST_TC_TIMEOUT) return fail(c, MIX_ETIMEOUT, "a wait for the tensor-core readout gave up");
     // The uniform-density estimate behind the initial lane groups overstates
     // open lattices (diamond holds half of it inside 3.4 A).  Once an
@@ -1002,6 +1001,7 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
     if (c->cap < 1) return bad("nbr_cap");
     d.cap = c->cap;
     d.rlist2 = c->rlist * c->rlist;
+    d.nbs = nb_screen(d.rlist2, d.box);
     d.half_skin2 = 0.25 * opt->skin * opt->skin;
     d.rce = a->r_cut;
     d.rce2 = a->r_cut * a->r_cut;
@@ -1056,6 +1056,7 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
         c->spl_bulk = bulk;
     }
     e = spline_configure(c->precision, c->spl_lpa, &c->spl_smem, &c->spl_grid);
+    if (e == cudaSuccess) e = front_configure(c->dev);
     c->ace_grid_max = c->ace_grid;
     c->spl_grid_max = c->spl_grid;
     if (e != cudaSuccess) {
@@ -1387,7 +1388,7 @@ int mix_get_info(const mix_ctx* c, mix_info* info) {
     info->launches_per_evaluation = evals_launches(c);
     info->launches = c->launches;
     info->gather_grid = c->dev.grid_gather;
-    info->build_grid = c->dev.grid_build;
+    info->build_grid = 0;
     info->buffer_grid = c->dev.grid_buffer;
     info->exp_tensor_cores = c->ace_tcm ? 1 : 0;
     info->tc_flops_per_atom = c->ace_tcm ? 2.0 * (double)c->tau_d3_sum * c->n * c->n * c->n : 0.0;
@@ -1961,6 +1962,7 @@ int fused_graph(mix_batch* b, int integrate, double dt, cudaGraph_t* graph, cuda
 
 // evaluate members whose forces or lists are not current, one by one
 int batch_prepare(mix_batch* b) {
+    std::vector<size_t> fresh;
     for (size_t k = 0; k < b->m.size(); ++k) {
         mix_ctx* c = b->m[k];
         if (!c->bound) return bfail(b, MIX_ESTATE, "member " + std::to_string(k) + " is not bound");
@@ -1968,8 +1970,20 @@ int batch_prepare(mix_batch* b) {
             int st = evaluate(c, 0, 0.0);
             if (st) return bfail(b, st, "member " + std::to_string(k) + ": " + c->err);
             c->forces_valid = true;
+            fresh.push_back(k);
         }
     }
+    // the batched kernels walk these members' lists: they must be whole (other
+    // device errors surface at the next synchronising call)
+    cudaError_t e = cudaSuccess;
+    for (size_t k : fresh)
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(b->m[k]->pinned, b->m[k]->dev.status, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess && !fresh.empty()) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return bfail(b, MIX_ECUDA, std::string("member status: ") + cudaGetErrorString(e));
+    for (size_t k : fresh)
+        if (b->m[k]->pinned[SW_STATUS] & ST_GRID_TIMEOUT)
+            return bfail(b, MIX_ETIMEOUT, "member " + std::to_string(k) + ": a wait at a grid barrier gave up");
     return MIX_OK;
 }
 
@@ -1984,6 +1998,7 @@ int mix_tune(mix_ctx* c, int reps) {
     const int sms = sm_count();
     std::vector<int> ga = {c->ace_grid_max, c->ace_grid_max * 3 / 4, c->ace_grid_max / 2, c->ace_grid_max / 4};
     std::vector<int> gg = {sms * 2, sms * 4, sms * 8, sms * 16};
+    std::vector<int> gf = {sms * 2, sms, sms / 2};
     SeedSave saved;
     const std::vector<int> orders = {MIX_ORDER_CHEAP_FIRST, MIX_ORDER_EXP_FIRST, MIX_ORDER_SERIAL};
     int st = seed_save(c, &saved);
@@ -1993,7 +2008,7 @@ int mix_tune(mix_ctx* c, int reps) {
     if (!st) st = tune_param(c, reps, &c->ace_grid, ga);
     if (!st) st = tune_param(c, reps, &c->spl_grid, gs);
     if (!st) st = tune_param(c, reps, &c->dev.grid_gather, gg);
-    if (!st) st = tune_param(c, reps, &c->dev.grid_buffer, gg);
+    if (!st) st = tune_param(c, reps, &c->dev.grid_buffer, gf);
     if (!st) st = tune_param(c, reps, &c->order, orders);   // again, at the shapes chosen
     drop_graph(c);
     const int st2 = seed_restore(c, saved);
@@ -2216,6 +2231,8 @@ int mix_set_seed_rule(mix_ctx* c, double r_coord, double z_lo, double z_hi, int 
     r.rblend2 = r_blend * r_blend;
     r.rblend = r_blend;
     r.rz2 = r_coord * r_coord;
+    r.rz2_lo = (float)(r.rz2 - 1e-3);
+    r.rz2_hi = (float)(r.rz2 + 1e-3);
     r.zlo = z_lo;
     r.zhi = z_hi;
     r.period = period;

@@ -18,6 +18,7 @@ enum StatusBits : int {
     ST_NONFINITE = 8,        // non-finite position or force
     ST_OUT_OF_BOX = 16,      // atom outside a non-periodic dimension
     ST_TC_TIMEOUT = 32,      // a bounded wait for tensor-core MMAs gave up
+    ST_GRID_TIMEOUT = 64,    // a bounded wait at a grid barrier gave up
 };
 enum StatusWord : int {
     SW_STATUS = 0,
@@ -36,12 +37,16 @@ enum StatusWord : int {
     SW_EPOCH = 13,      // force evaluations since binding (stamps the incoming gradient rows)
     SW_ACE_NEXT = 14,   // next group of expensive atoms to hand out (0 between launches)
     SW_ACE_DONE = 15,   // CTAs of the expensive kernel that have finished (0 between launches)
+    SW_GRID_COUNT = 32, // arrivals at the grid barriers of the running front kernel (0 between launches;
+                        // a 128-byte line of its own)
+    SW_GRID_DONE = 16,  // CTAs of the front kernel that have left (0 between launches)
     SW_COUNT = 64,
 };
 
 constexpr int NB3MAX = 32;          // three-body neighbours per atom handled on chip
 constexpr int MAX_CAP = 256;        // neighbour slots per atom
-constexpr int SCAN_BLOCK = 1024;    // atoms per block in the set compaction
+constexpr int SCAN_BLOCK = 1024;    // atoms per block in the batched set compaction
+constexpr int FRONT_MAX_CTAS = 1024;   // most CTAs of the front kernel (its block counts)
 
 struct Box {
     double lo[3], L[3], invL[3];
@@ -86,6 +91,7 @@ struct SeedRule {
     int blend;         // MIX_BLEND_*
     double rcore2, rblend2, rblend;
     double rz2;        // coordination radius squared
+    float rz2_lo, rz2_hi;   // float screen of the count: rz2 -+ 1e-3 A^2 (see Dev::bufe2_lo)
     double zlo, zhi;   // seed when the averaged coordination lies in [zlo, zhi]
     int period;        // evaluations averaged per seed refresh
 };
@@ -99,6 +105,30 @@ __host__ __device__ __forceinline__ double half_kick(double dt, double mass) {
     return 0.5 * dt * MIX_KAPPA / mass;
 }
 
+// Float screen of the list build, formed on the host: squared list radius less and
+// plus 2e-4 of it (the float distance is within 2e-5 relative of the float64 one
+// for boxes up to a few thousand Angstrom, so only candidates in between take the
+// exact float64 test), box lengths, their inverses and origin.  Formed in the kernel from
+// the float64 fields, the conversions were repeated for every pass over
+// candidates: ten float64-pipe instructions a pass and warp, 16 cycles of the SM
+// each, which made them the whole build (a warp's row 31 us with 16 warps an SM).
+struct NbScreen {
+    float lo2, hi2;
+    float L[3], iL[3], lo[3];
+    float pad;   // a multiple of 8 bytes
+};
+inline NbScreen nb_screen(double rlist2, const Box& b) {
+    NbScreen s{};
+    s.lo2 = (float)(rlist2 * (1.0 - 2e-4));
+    s.hi2 = (float)(rlist2 * (1.0 + 2e-4));
+    for (int k = 0; k < 3; ++k) {
+        s.L[k] = (float)b.L[k];
+        s.iL[k] = (float)b.invL[k];
+        s.lo[k] = (float)b.lo[k];
+    }
+    return s;
+}
+
 struct Dev {
     int64_t n;
     int cap;
@@ -106,6 +136,7 @@ struct Dev {
     Box box;
     Cells cells;
     double rlist2;       // (rc_max + skin)^2
+    NbScreen nbs;        // float screen of the list build
     double half_skin2;   // (skin / 2)^2
     double rce, rce2;    // expensive cutoff
     double rcc, rcc2;    // cheap 2-body cutoff
@@ -160,8 +191,8 @@ struct Dev {
     int* zsum;           // [N] coordination summed over the current averaging period
     int nblk;            // blocks of the compaction kernels
     // launch shapes chosen by the autotuner (0: default)
-    int grid_build;      // CTAs of the neighbour-list build (4 warps each)
-    int grid_buffer;     // CTAs of the buffer scan (8 warps each)
+    int grid_front_max;  // CTAs of the front kernel that are resident together
+    int grid_buffer;     // most CTAs of the front kernel (16 warps each)
     int grid_gather;     // CTAs of the gather (8 warps each)
 };
 
@@ -353,6 +384,10 @@ __device__ __forceinline__ int cell_coord(const Box& b, const Cells& c, double x
 }
 
 __device__ __forceinline__ void set_status(int* st, int bits) { atomicOr(st + SW_STATUS, bits); }
+
+// false once a front kernel of the context gave up at a grid barrier: its lists
+// and sets may then be half written, and no kernel may walk them
+__device__ __forceinline__ bool list_ok(const Dev& d) { return (d.status[SW_STATUS] & ST_GRID_TIMEOUT) == 0; }
 
 // Warp-wide sum delivered to lane 0 as float64, lanes combined in a fixed
 // order.  float64 inputs are summed in float64; float inputs are summed in

@@ -5,13 +5,13 @@
 
 namespace mixd {
 
-// lists (k_lists.cu)
-void launch_disp(const Dev& d, cudaStream_t s, int integrate, double dt, double h, int force_rebuild);
-void launch_build(const Dev& d, cudaStream_t s);
-
-// weights, sets, compaction (k_sets.cu)
-void launch_sets(const Dev& d, const Regions& r, const SeedRule& sr, cudaStream_t s);
-int sets_launches(const SeedRule& sr);   // kernels launch_sets enqueues
+// displacement, lists, weights, sets and their compaction in one cooperative
+// launch (k_front.cu).  front_configure fills d.grid_front_max.
+cudaError_t front_configure(Dev& d);
+cudaError_t launch_front(const Dev& d, const Regions& r, const SeedRule& sr, cudaStream_t s, int integrate, double dt,
+                         double h, int force_rebuild);
+// the lists alone, of the positions x_in (copied to d.x and folded there)
+cudaError_t launch_front_lists(const Dev& d, const double4* x_in, cudaStream_t s);
 
 // expensive potential (k_ace.cuh, k_ace_f32_n*.cu, k_ace_f64.cu); returns cudaSuccess or the launch error;
 // wn: warps (atoms) a CTA, ACE_GROUP or ACE_MAX_WARPS
