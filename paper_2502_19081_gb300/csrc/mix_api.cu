@@ -371,6 +371,7 @@ struct mix_ctx {
     int ace_tcm;                      // 0: CUDA-core nu = 3; 1, 2: tensor-core readout (bf16, bf16 hi/lo)
     int ace_nbuf;                     // tile buffers of the tensor-core kernel
     int spl_lpa;                      // lanes per atom of the cheap kernel (32, 16 or 8)
+    int spl_na;                       // SplTab::na
     bool spl_bulk;                    // periodic in every dimension (narrow lane groups allowed)
     bool spl_lpa_settled;             // the lane groups were narrowed or widened once
     int ace_grid_max, spl_grid_max;   // resident CTAs at full occupancy
@@ -603,6 +604,9 @@ int build_tables(mix_ctx* c, const mix_ace* a, const mix_spline* sp) {
     std::vector<double> sc2(SPL_W2 * 4), sc3(64 * SPL_W3 * 4);
     for (int q = 0; q < SPL_W2; ++q)
         for (int k = 0; k < 4; ++k) sc2[q * 4 + k] = sp->c2[q + k];
+    c->spl_na = 0;
+    for (int abc = 0; abc < 512; ++abc)
+        if (sp->c3[abc] != 0.0) c->spl_na = std::max(c->spl_na, abc / 64 + 1);
     for (int ab = 0; ab < 64; ++ab)
         for (int z = 0; z < SPL_W3; ++z)
             for (int k = 0; k < 4; ++k) sc3[(ab * SPL_W3 + z) * 4 + k] = sp->c3[ab * 8 + z + k];
@@ -664,6 +668,8 @@ void fill_tabs(mix_ctx* c, unsigned char* base, AceTab<T>& at, SplTab<T>& st) {
     st.invh2 = (T)(13.0 / c->spl_rc);
     st.invh3 = (T)(5.0 / c->spl_rc3);
     st.invhc = (T)(5.0 / (2.0 * c->spl_rc3));
+    st.na = c->spl_na;
+    st.pad = 0;
 }
 
 void layout(mix_ctx* c) {

@@ -354,6 +354,8 @@ struct SplTab {
     // (no float64 division per atom on the device)
     T rc2, rc32;            // rc^2 (2-body), rc3^2
     T invh2, invh3, invhc;  // 13/rc, 5/rc3, 5/(2 rc3)
+    int na;                 // 1 + the largest a with a non-zero c3[a][b][c] (and, by symmetry, b)
+    int pad;
 };
 
 // ---------------------------------------------------------------------------
