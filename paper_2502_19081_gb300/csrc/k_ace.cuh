@@ -974,7 +974,7 @@ __global__ void __launch_bounds__(ace_warps<T>() * 32, ace_min_ctas<T>()) kb_ace
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Dev s_dev;
     __shared__ AceTab<T> s_tab;
-    const int count = *b.count;
+    const int count = list_ok(b.words) ? *b.count : 0;
     int cur = -1;
     for (int g = blockIdx.x; g < count; g += gridDim.x) {
         const int2 e = b.list[g];

@@ -17,6 +17,7 @@ struct AceBatch {
     const AceTab<T>* tabs;
     const int2* list;
     const int* count;
+    const int* words;   // the plan's status words (list_ok)
 };
 
 template <typename T>

@@ -202,21 +202,22 @@ __global__ void __launch_bounds__(G_WARPS * 32, sizeof(T) == 4 ? 4 : 2) k_gather
 // Each block belongs to one system and gathers with that system's own lane
 // groups, so a system's forces are bit for bit those it gets alone.
 template <typename T>
-__global__ void __launch_bounds__(G_WARPS * 32) kb_gather(BatchArgs ba, int integrate, double dt) {
+__global__ void __launch_bounds__(G_WARPS * 32) kb_gather(BatchArgs ba, const double* __restrict__ hk, int integrate) {
     __shared__ GSum<T> park[G_WARPS * G_ATOMS * 6];
     MIX_BATCH_BLOCK(ba)
-    const double h = half_kick(dt, s_dev.mass);
+    if (!list_ok(s_dev)) return;
+    const double h = hk[s_ent.x];
     const int lpa = gather_lpa(s_dev);
     if (lpa == 8) gather_body<T, 8>(s_dev, s_ent.y, s_ent.z, integrate, h, G_ATOMS, park);
     else if (lpa == 16) gather_body<T, 16>(s_dev, s_ent.y, s_ent.z, integrate, h, G_ATOMS, park);
     else gather_body<T, 32>(s_dev, s_ent.y, s_ent.z, integrate, h, G_ATOMS, park);
 }
 
-void launch_gather_batch(const BatchPlan& p, int precision, int integrate, double dt, cudaStream_t s) {
+void launch_gather_batch(const BatchPlan& p, int precision, int integrate, cudaStream_t s) {
     if (precision == MIX_FP64)
-        kb_gather<double><<<p.nblk[BT_GATHER], G_WARPS * 32, 0, s>>>(p.ba[BT_GATHER], integrate, dt);
+        kb_gather<double><<<p.nblk[BT_GATHER], G_WARPS * 32, 0, s>>>(p.ba[BT_GATHER], p.hk, integrate);
     else
-        kb_gather<float><<<p.nblk[BT_GATHER], G_WARPS * 32, 0, s>>>(p.ba[BT_GATHER], integrate, dt);
+        kb_gather<float><<<p.nblk[BT_GATHER], G_WARPS * 32, 0, s>>>(p.ba[BT_GATHER], p.hk, integrate);
 }
 
 void launch_gather(const Dev& d, int precision, int integrate, double h, cudaStream_t s) {

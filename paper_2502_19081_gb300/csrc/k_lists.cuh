@@ -26,8 +26,8 @@ __device__ __forceinline__ void disp_reset(const Dev& d, int force_rebuild) {
 }
 
 // v += h F; x += dt v (when integrating); then flag a rebuild if the atom moved
-// more than skin/2 since the last build.
-__device__ __forceinline__ void disp_atom(const Dev& d, int64_t i, int integrate, double dt, double h,
+// more than skin/2 since the last build (returned as well).
+__device__ __forceinline__ bool disp_atom(const Dev& d, int64_t i, int integrate, double dt, double h,
                                           int force_rebuild) {
     // every load first, so that one memory latency covers them all (the
     // arrays never overlap, which the compiler cannot know)
@@ -55,31 +55,25 @@ __device__ __forceinline__ void disp_atom(const Dev& d, int64_t i, int integrate
     const bool finite = isfinite(x.x) && isfinite(x.y) && isfinite(x.z);
     if (!finite) {
         set_status(d.status, ST_NONFINITE);
-        return;
+        return false;
     }
+    bool moved = false;
     const double xs[3] = {x.x, x.y, x.z};
     for (int k = 0; k < 3; ++k)
         if (!d.box.per[k] && (xs[k] < d.box.lo[k] || xs[k] >= d.box.lo[k] + d.box.L[k]))
             set_status(d.status, ST_OUT_OF_BOX);
     if (!force_rebuild) {
         const double dx = x.x - xb.x, dy = x.y - xb.y, dz = x.z - xb.z;
-        if (dx * dx + dy * dy + dz * dz > d.half_skin2) d.status[SW_REBUILD] = 1;
+        moved = dx * dx + dy * dy + dz * dz > d.half_skin2;
+        if (moved) d.status[SW_REBUILD] = 1;
         // relative to the cell of the last build (recomputed by the binning on rebuilds)
         if (d.xr) d.xr[i] = cell_relative(d.box, d.cells, x, c3);
     }
+    return moved;
 }
 
 // (Bodies take the system d, this block's index bx among the gx blocks working
 // on d, and stride over d's atoms.)
-__device__ __forceinline__ void disp_body(const Dev& d, int bx, int gx, int integrate, double dt, double h,
-                                          int force_rebuild) {
-    const int64_t stride = (int64_t)gx * blockDim.x;
-    for (int64_t i = bx * (int64_t)blockDim.x + threadIdx.x;; i += stride) {
-        if (i == 0) disp_reset(d, force_rebuild);
-        if (i >= d.n) return;
-        disp_atom(d, i, integrate, dt, h, force_rebuild);
-    }
-}
 
 // Fold periodic coordinates into [0, L), bin into cells, count per cell.
 __device__ __forceinline__ void cell_bin_atom(const Dev& d, int64_t i) {
@@ -103,10 +97,6 @@ __device__ __forceinline__ void cell_bin_atom(const Dev& d, int64_t i) {
     atomicAdd(d.cell_count + c, 1);
 }
 
-__device__ __forceinline__ void cell_bin_body(const Dev& d, int bx, int gx) {
-    for (int64_t i = bx * (int64_t)blockDim.x + threadIdx.x; i < d.n; i += (int64_t)gx * blockDim.x)
-        cell_bin_atom(d, i);
-}
 // Exclusive scan of the cell counts (one block), zeroing counts and fill slots.
 __device__ __forceinline__ void cell_scan_body(const Dev& d) {
     __shared__ int wsum[32];
@@ -157,8 +147,6 @@ __device__ __forceinline__ void cell_fill_body(const Dev& d, int bx, int gx) {
         d.cell_atoms[slot] = (int)i;
     }
 }
-constexpr int NB_WARPS = 4;
-
 // One warp per atom: the 27-cell stencil is up to 18 contiguous runs of cells
 // (9 rows (dz, dy), one or two runs along x each); lane r < 18 finds run r, a
 // warp prefix sum numbers all candidates of all runs, and the lanes take 32
@@ -261,9 +249,7 @@ __device__ __forceinline__ void nb_write_row(const Dev& d, int64_t i, const doub
     __syncwarp();
 }
 
-// AHEAD2: also load the float positions a pass ahead (the batched kernel; the
-// single-context one, on longer candidate runs, measured faster without)
-template <bool AHEAD2, int NBW>
+template <int NBW>
 __device__ __forceinline__ void neigh_build_body(const Dev& d, int bx, int gx, int capp2, int* sbuf) {
     __shared__ int s_runx[NBW][NB_RUNS];   // cell_atoms index of a run's first candidate, less its number
     __shared__ int s_runi[NBW][NB_RUNS];   // candidates in runs 0..r
@@ -293,42 +279,23 @@ __device__ __forceinline__ void neigh_build_body(const Dev& d, int bx, int gx, i
             runx[lane] = t0 - (inc - len);
         }
         __syncwarp();
-        // AHEAD2: the atom two passes ahead and the position one pass ahead are
-        // loaded before this pass is tested; else the atom one pass ahead
-        // (r: run of the furthest candidate loaded)
+        // the atom one pass ahead is loaded before this pass is tested (r: run of the
+        // furthest candidate loaded)
         int r = 0;
-        int jn = -1, jnn = -1;
-        float4 xn = make_float4(0.f, 0.f, 0.f, 0.f);
+        int jn = -1;
         if (lane < total) {
             while (lane >= runi[r]) ++r;
             jn = d.cell_atoms[runx[r] + lane];
-            if (AHEAD2) xn = d.xf[jn];
-        }
-        if (AHEAD2 && lane + 32 < total) {
-            while (lane + 32 >= runi[r]) ++r;
-            jnn = d.cell_atoms[runx[r] + lane + 32];
         }
         int cnt = 0;
         for (int u = lane; u - lane < total; u += 32) {
             const int j = jn;
-            float4 xjf;
-            if (AHEAD2) {
-                xjf = xn;
-                jn = jnn;
-                if (u + 32 < total) xn = d.xf[jnn];
-                if (u + 64 < total) {
-                    while (u + 64 >= runi[r]) ++r;
-                    jnn = d.cell_atoms[runx[r] + u + 64];
-                }
-            } else if (u + 32 < total) {
+            if (u + 32 < total) {
                 while (u + 32 >= runi[r]) ++r;
                 jn = d.cell_atoms[runx[r] + u + 32];
             }
             bool ok = false;
-            if (u < total && j != (int)i) {
-                if (!AHEAD2) xjf = d.xf[j];
-                ok = nb_accept(d, xi, xif, xjf, j);
-            }
+            if (u < total && j != (int)i) ok = nb_accept(d, xi, xif, d.xf[j], j);
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             if (ok) {
                 const int p = cnt + __popc(m & lt);
@@ -355,7 +322,7 @@ __device__ __forceinline__ void neigh_build_body(const Dev& d, int bx, int gx, i
 // at those images and any other pair only reads as farther away): the minimum image
 // per pair and component was half the instructions of this issue-bound kernel.
 // The float screen only decides away from the threshold, so the rows are those of
-// the batched build (neigh_build_body).  A stencil with more than NB_TILE
+// the warp-per-atom build (neigh_build_body).  A stencil with more than NB_TILE
 // candidates (a dense spot) is tested from global memory instead.
 constexpr int NB_TILE = 1024;
 

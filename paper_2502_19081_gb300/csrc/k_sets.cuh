@@ -14,19 +14,6 @@
 
 namespace mixd {
 
-__device__ __forceinline__ void lambda_atom(const Dev& d, const Regions& r, int64_t i);
-
-__device__ __forceinline__ void lambda_body(const Dev& d, const Regions& r, int bx, int gx) {
-    for (int64_t i = bx * (int64_t)blockDim.x + threadIdx.x;; i += (int64_t)gx * blockDim.x) {
-        if (i == 0 && d.status[SW_REBUILD]) {
-            d.status[SW_REBUILDS] += 1;
-            d.status[SW_REBUILD] = 0;
-        }
-        if (i >= d.n) return;
-        lambda_atom(d, r, i);
-    }
-}
-
 __device__ __forceinline__ void lambda_atom(const Dev& d, const Regions& r, int64_t i) {
     double4 x = make_double4(0.0, 0.0, 0.0, 0.0);   // read once some region is not screened out
     bool have_x = false;

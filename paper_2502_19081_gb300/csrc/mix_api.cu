@@ -701,8 +701,8 @@ void layout(mix_ctx* c) {
     c->o_act_c = take(N * 4);
     c->o_pos_e = take(N * 4);
     c->o_pos_c = take(N * 4);
-    c->o_blk_e = take(std::max<size_t>(c->dev.nblk, FRONT_MAX_CTAS) * 4);
-    c->o_blk_c = take(std::max<size_t>(c->dev.nblk, FRONT_MAX_CTAS) * 4);
+    c->o_blk_e = take((size_t)c->dev.nblk * 4);
+    c->o_blk_c = take((size_t)c->dev.nblk * 4);
     c->o_ge = take(N * cap * v4);
     c->o_gc = take(N * cap * v4);
     c->o_gei = take(N * cap * v4);
@@ -1025,8 +1025,7 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
     double extent = 0.0;
     for (int k = 0; k < 3; ++k) extent = std::max(extent, std::fabs(sys->box_lo[k]) + sys->box_len[k]);
     d.exact_lists = extent > 2000.0 ? 1 : 0;
-    const int64_t nblk = (sys->n_atoms + SCAN_BLOCK - 1) / SCAN_BLOCK;
-    d.nblk = (int)(nblk > 0 ? nblk : 1);
+    d.nblk = (int)std::max<int64_t>(FRONT_MAX_CTAS, (sys->n_atoms + FRONT_ATOMS - 1) / FRONT_ATOMS);
     std::memset(&c->regions, 0, sizeof c->regions);
     c->regions.blend = opt->blend;
     int st = build_tables(c, a, sp);
@@ -1769,7 +1768,7 @@ void fused_free(mix_batch* b) {
 // Host-built plan: per-system parameter arrays, one block table per launch
 // granularity, the expensive groups (systems sharing L and the padded radial
 // count) and the flattened work lists, all in one device allocation.
-int fused_build(mix_batch* b) {
+int fused_build(mix_batch* b, double dt) {
     const int ns = (int)b->m.size();
     b->precision = b->m[0]->precision;
     const bool f64 = b->precision == MIX_FP64;
@@ -1823,8 +1822,7 @@ int fused_build(mix_batch* b) {
         const Dev& d = devs[s];
         const int64_t n = d.n;
         auto blocks = [](int64_t units, int64_t per) { return (int)std::max<int64_t>(1, (units + per - 1) / per); };
-        const int gx[BT_COUNT] = {blocks(n, 1024), 1, blocks(n, 32), blocks(n, 64),
-                                  blocks(n, 256), std::max(1, d.nblk), blocks(n, 256)};
+        const int gx[BT_COUNT] = {blocks(n, FRONT_ATOMS), blocks(n, 256)};
         for (int k = 0; k < BT_COUNT; ++k)
             for (int bx = 0; bx < gx[k]; ++bx) tabs[k].push_back(make_int4(s, bx, gx[k], 0));
         while (capp2 < d.cap) capp2 <<= 1;
@@ -1840,7 +1838,8 @@ int fused_build(mix_batch* b) {
     };
     const size_t o_devs = take(ns * sizeof(Dev)), o_regs = take(ns * sizeof(Regions)), o_ace = take(ns * tsz),
                  o_spl = take(ns * ssz), o_eg = take(ns * 4), o_el = take(ns * 4), o_eb = take(ng * 4),
-                 o_cnt = take((ng + 1) * 4), o_le = take(tot * sizeof(int2)), o_lc = take(tot * sizeof(int2));
+                 o_cnt = take((ng + 1) * 4), o_hk = take(ns * sizeof(double)), o_words = take(SW_COUNT * 4),
+                 o_le = take(tot * sizeof(int2)), o_lc = take(tot * sizeof(int2));
     size_t o_tab[BT_COUNT];
     for (int k = 0; k < BT_COUNT; ++k) o_tab[k] = take(tabs[k].size() * sizeof(int4));
     fused_free(b);
@@ -1868,6 +1867,9 @@ int fused_build(mix_batch* b) {
     put(o_eg, egroup.data(), ns * 4);
     put(o_el, elast.data(), ns * 4);
     put(o_eb, ebase.data(), ng * 4);
+    std::vector<double> hk(ns);
+    for (int s = 0; s < ns; ++s) hk[s] = half_kick(dt, b->m[s]->sys.mass);
+    put(o_hk, hk.data(), ns * sizeof(double));
     for (int k = 0; k < BT_COUNT; ++k) put(o_tab[k], tabs[k].data(), tabs[k].size() * sizeof(int4));
     e = cudaMemcpy(b->dmem, host.data(), off, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return bfail(b, MIX_ECUDA, std::string("fused batch upload: ") + cudaGetErrorString(e));
@@ -1883,6 +1885,8 @@ int fused_build(mix_batch* b) {
     }
     P.regions = reinterpret_cast<const Regions*>(base + o_regs);
     P.capp2 = capp2;
+    P.hk = reinterpret_cast<const double*>(base + o_hk);
+    P.words = reinterpret_cast<int*>(base + o_words);   // zero, as the whole upload's gaps are
     FlatArgs& F = P.flat;
     F.devs = b->ddevs;
     F.nsys = ns;
@@ -1920,7 +1924,7 @@ int fused_build(mix_batch* b) {
     return MIX_OK;
 }
 
-int fused_launches(const mix_batch* b) { return 15 + (int)b->groups.size(); }
+int fused_launches(const mix_batch* b) { return 3 + (int)b->groups.size(); }   // front, cheap, gather
 
 // one fused step (or force evaluation) captured on the batch's private stream
 int fused_graph(mix_batch* b, int integrate, double dt, cudaGraph_t* graph, cudaGraphExec_t* exec) {
@@ -1938,25 +1942,27 @@ int fused_graph(mix_batch* b, int integrate, double dt, cudaGraph_t* graph, cuda
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return bfail(b, MIX_ECUDA, std::string("cudaStreamBeginCapture: ") + cudaGetErrorString(e));
     const BatchPlan& P = b->plan;
-    launch_disp_batch(P, s, integrate, dt, 0);
-    launch_build_batch(P, s);
-    launch_sets_batch(P, s);
+    const cudaError_t ef = launch_front_batch(P, s, integrate, dt);
     // cheap potential on a second branch, concurrent with the expensive groups
     cudaEventRecord(b->ev_fork, s);
     cudaStreamWaitEvent(b->aux, b->ev_fork, 0);
     launch_spline_batch(b->precision, b->spl_lpa, b->ddevs, b->dspl, P.flat.list_c, P.flat.counts + b->groups.size(),
-                        b->spl_uniform, b->spl_smem, b->spl_grid, b->aux);
+                        P.words, b->spl_uniform, b->spl_smem, b->spl_grid, b->aux);
     cudaEventRecord(b->ev_join, b->aux);
     for (size_t g = 0; g < b->groups.size(); ++g) {
         const mix_batch::Group& G = b->groups[g];
-        launch_ace_batch(b->precision, b->ddevs, b->dace, P.flat.list_e + G.base, P.flat.counts + g, G.n, G.L, G.smem,
+        launch_ace_batch(b->precision, b->ddevs, b->dace, P.flat.list_e + G.base, P.flat.counts + g, P.words, G.n, G.L, G.smem,
                          G.grid, s);
     }
     cudaStreamWaitEvent(s, b->ev_join, 0);
-    launch_gather_batch(P, b->precision, integrate, dt, s);
+    launch_gather_batch(P, b->precision, integrate, s);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(s, &g);
-    if (e != cudaSuccess) return bfail(b, MIX_ECUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(e));
+    if (e == cudaSuccess && ef != cudaSuccess) {
+        cudaGraphDestroy(g);
+        e = ef;
+    }
+    if (e != cudaSuccess) return bfail(b, MIX_ECUDA, std::string("fused step capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(exec, g, 0);
     if (e != cudaSuccess) {
         cudaGraphDestroy(g);
@@ -2053,7 +2059,7 @@ int mix_batch_step(mix_batch* b, double dt, int nsteps) {
         batch_drop(b);
         if (fused) {
             // the plan snapshots the members' device descriptors: rebuilt with the graph
-            st = fused_build(b);
+            st = fused_build(b, dt);
             if (!st) st = fused_graph(b, 1, dt, &b->graph, &b->exec);
         } else {
             st = batch_graph(b, 1, dt, &b->graph, &b->exec);

@@ -40,12 +40,13 @@ enum StatusWord : int {
     SW_GRID_COUNT = 32, // arrivals at the grid barriers of the running front kernel (0 between launches;
                         // a 128-byte line of its own)
     SW_GRID_DONE = 16,  // CTAs of the front kernel that have left (0 between launches)
+    SW_ANY = 1,         // batch plan words: some system rebuilds its lists in this step (word 0: status bits)
     SW_COUNT = 64,
 };
 
 constexpr int NB3MAX = 32;          // three-body neighbours per atom handled on chip
 constexpr int MAX_CAP = 256;        // neighbour slots per atom
-constexpr int SCAN_BLOCK = 1024;    // atoms per block in the batched set compaction
+constexpr int FRONT_ATOMS = 512;       // atoms of a block-table entry of the batched front (a thread each)
 constexpr int FRONT_MAX_CTAS = 1024;   // most CTAs of the front kernel (its block counts)
 
 struct Box {
@@ -189,7 +190,7 @@ struct Dev {
     uint8_t* seed;       // [N] seed atoms (seed-atom weights)
     uint8_t* core;       // [N] core atoms
     int* zsum;           // [N] coordination summed over the current averaging period
-    int nblk;            // blocks of the compaction kernels
+    int nblk;            // entries of blk_e and blk_c
     // launch shapes chosen by the autotuner (0: default)
     int grid_front_max;  // CTAs of the front kernel that are resident together
     int grid_buffer;     // most CTAs of the front kernel (16 warps each)
@@ -227,21 +228,6 @@ __device__ __forceinline__ void load_dev(Dev* dst, const Dev* src) { copy_shared
     if (threadIdx.x == 0) s_ent = (ba).tab[blockIdx.x];      \
     __syncthreads();                                         \
     load_dev(&s_dev, (ba).devs + s_ent.x);                   \
-    __syncthreads();
-
-// The same for kernels that only work on list rebuilds: the block returns
-// before loading anything when its system keeps its lists.
-#define MIX_BATCH_BLOCK_REBUILD(ba)                                       \
-    __shared__ Dev s_dev;                                                 \
-    __shared__ int4 s_ent;                                                \
-    __shared__ int s_go;                                                  \
-    if (threadIdx.x == 0) {                                               \
-        s_ent = (ba).tab[blockIdx.x];                                     \
-        s_go = (ba).devs[s_ent.x].status[SW_REBUILD];                     \
-    }                                                                     \
-    __syncthreads();                                                      \
-    if (s_go == 0) return;                                                \
-    load_dev(&s_dev, (ba).devs + s_ent.x);                                \
     __syncthreads();
 
 template <typename T> struct Vec4;
@@ -389,7 +375,8 @@ __device__ __forceinline__ void set_status(int* st, int bits) { atomicOr(st + SW
 
 // false once a front kernel of the context gave up at a grid barrier: its lists
 // and sets may then be half written, and no kernel may walk them
-__device__ __forceinline__ bool list_ok(const Dev& d) { return (d.status[SW_STATUS] & ST_GRID_TIMEOUT) == 0; }
+__device__ __forceinline__ bool list_ok(const int* status) { return (status[SW_STATUS] & ST_GRID_TIMEOUT) == 0; }
+__device__ __forceinline__ bool list_ok(const Dev& d) { return list_ok(d.status); }
 
 // Warp-wide sum delivered to lane 0 as float64, lanes combined in a fixed
 // order.  float64 inputs are summed in float64; float inputs are summed in

@@ -50,12 +50,7 @@ void launch_gather(const Dev& d, int precision, int integrate, double h, cudaStr
 
 // Block-table classes: every batched launch uses the table of its granularity.
 enum BatchTabClass : int {
-    BT_ATOM = 0,   // 256 threads, a thread per atom (grid-stride)
-    BT_ONE,        // one block per system
-    BT_NB,         // 4 warps, a warp per atom (list build)
-    BT_REV,        // 8 warps, a warp per atom (reverse map)
-    BT_WARP8,      // 8 warps of 32 atoms each (buffer scan)
-    BT_SCAN,       // SCAN_BLOCK atoms per block, the system's own block count
+    BT_FRONT = 0,  // FRONT_ATOMS atoms (front)
     BT_GATHER,     // 8 warps of 32 atoms each (gather)
     BT_COUNT
 };
@@ -67,7 +62,7 @@ struct FlatArgs {
     const int* egroup;   // [nsys] expensive group (systems sharing T, L, NP)
     const int* elast;    // [nsys] 1 for the last system of its group
     const int* ebase;    // [ngrp] start of each group in list_e
-    int2* list_e;        // {system, index in its expensive list}
+    int2* list_e;        // {system, first index of a group of ACE_GROUP in its expensive list}
     int2* list_c;        // {system, atom} for each entry of the systems' cheap lists
     int* counts;         // [ngrp + 1] expensive totals per group, cheap total
 };
@@ -76,20 +71,22 @@ struct BatchPlan {
     BatchArgs ba[BT_COUNT];
     int nblk[BT_COUNT];
     const Regions* regions;   // [nsys]
+    const double* hk;         // [nsys] half-kick factors of the plan's time step
+    int* words;               // [SW_COUNT] status bits, grid barrier and rebuild flag of the front
     int capp2;                // largest power-of-two list capacity (build scratch)
     FlatArgs flat;
 };
 
-void launch_disp_batch(const BatchPlan& p, cudaStream_t s, int integrate, double dt, int force_rebuild);
-void launch_build_batch(const BatchPlan& p, cudaStream_t s);
-void launch_sets_batch(const BatchPlan& p, cudaStream_t s);
+// displacement, lists, weights, sets and their flattened lists of every system in
+// one cooperative launch (k_front.cu)
+cudaError_t launch_front_batch(const BatchPlan& p, cudaStream_t s, int integrate, double dt);
 cudaError_t ace_batch_configure(int precision, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid);
-void launch_ace_batch(int precision, const Dev* devs, const void* tabs, const int2* list, const int* count, int n,
-                      int L, size_t smem, int grid, cudaStream_t s);
+void launch_ace_batch(int precision, const Dev* devs, const void* tabs, const int2* list, const int* count,
+                      const int* words, int n, int L, size_t smem, int grid, cudaStream_t s);
 cudaError_t spline_batch_configure(int precision, int lpa, size_t* smem, int* grid);
 void launch_spline_batch(int precision, int lpa, const Dev* devs, const void* tabs, const int2* list,
-                         const int* count, int uniform, size_t smem, int grid, cudaStream_t s);
-void launch_gather_batch(const BatchPlan& p, int precision, int integrate, double dt, cudaStream_t s);
+                         const int* count, const int* words, int uniform, size_t smem, int grid, cudaStream_t s);
+void launch_gather_batch(const BatchPlan& p, int precision, int integrate, cudaStream_t s);
 
 int sm_count();
 
