@@ -875,7 +875,7 @@ int read_status(mix_ctx* c) {
     if (st & ST_OUT_OF_BOX) return fail(c, MIX_EBOX, "an atom left the box in a non-periodic dimension");
     if (st & ST_REV_MISSING) return fail(c, MIX_EINVAL, "asymmetric neighbour list");
     if (st & ST_GRID_TIMEOUT) return fail(c, MIX_ETIMEOUT, "a wait at a grid barrier gave up");
-    if (st & ST_TC_TIMEOUT) return fail(c, MIX_ETIMEOUT, "a wait for the tensor-core readout gave up");
+    if (st & ST_TC_TIMEOUT) return fail(c, MIX_ETIMEOUT, "a wait for a coefficient tile or the tensor-core readout gave up");
     // The uniform-density estimate behind the initial lane groups overstates
     // open lattices (diamond holds half of it inside 3.4 A).  Once an
     // evaluation has measured the largest 3-body count, a periodic bulk moves
@@ -1822,7 +1822,7 @@ int fused_build(mix_batch* b, double dt) {
         const Dev& d = devs[s];
         const int64_t n = d.n;
         auto blocks = [](int64_t units, int64_t per) { return (int)std::max<int64_t>(1, (units + per - 1) / per); };
-        const int gx[BT_COUNT] = {blocks(n, FRONT_ATOMS), blocks(n, 256)};
+        const int gx[BT_COUNT] = {blocks(n, FRONT_ATOMS), blocks(n, 8 * GB_ATOMS)};
         for (int k = 0; k < BT_COUNT; ++k)
             for (int bx = 0; bx < gx[k]; ++bx) tabs[k].push_back(make_int4(s, bx, gx[k], 0));
         while (capp2 < d.cap) capp2 <<= 1;

@@ -48,10 +48,12 @@ void launch_gather(const Dev& d, int precision, int integrate, double h, cudaStr
 // ---------------------------------------------------------------------------
 // multi-system step (batches of contexts sharing one stream)
 
+constexpr int GB_ATOMS = 8;   // atoms a warp of the batched gather
+
 // Block-table classes: every batched launch uses the table of its granularity.
 enum BatchTabClass : int {
     BT_FRONT = 0,  // FRONT_ATOMS atoms (front)
-    BT_GATHER,     // 8 warps of 32 atoms each (gather)
+    BT_GATHER,     // 8 warps of GB_ATOMS atoms each (gather)
     BT_COUNT
 };
 
