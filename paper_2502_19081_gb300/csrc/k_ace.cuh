@@ -520,6 +520,88 @@ __device__ __forceinline__ void nu2_float(const AceTab<float>& tab, const float*
     }
 }
 
+// polls of an mbarrier before a copy or a readout MMA is declared lost (status
+// bit ST_TC_TIMEOUT, reported as MIX_ETIMEOUT)
+constexpr int TC_WAIT_POLLS = 1 << 20;
+
+// The CUDA-core kernels' tile ring: two buffers filled by bulk copies (one thread
+// issues a whole tile) that complete on an mbarrier each; two tiles are on their
+// way before the atom's density is formed.  A warp counts itself done with a tile,
+// and the last of the CTA's warps to finish it issues the copy of the next but one
+// into its place.  (n = 10, lmax = 4, 1,394 atoms in a step: 87 -> 75 us with the
+// next 32 slots' partners loaded ahead in the density, against copies by every
+// thread a triple ahead.)
+struct TileRing {
+    uint32_t full;       // two mbarriers, 8 bytes apart (shared address)
+    int* left;           // [2] warps still to finish the buffer's tile
+    uint32_t phase;      // bit b: parity of buffer b's next completion
+    int abort;           // a wait ran out: no further waits
+};
+
+__device__ __forceinline__ void bulk_fetch(void* dst, const void* src, int bytes, uint32_t bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
+// one thread: tile t into buf
+__device__ __forceinline__ void ring_fetch(const TileRing& ring, const unsigned char* tiles, const int* off, int t,
+                                           unsigned char* buf, int warps) {
+    const int b0 = __ldg(off + t), nb = __ldg(off + t + 1) - b0;
+    ring.left[t & 1] = warps;
+    __threadfence_block();
+    bulk_fetch(buf, tiles + b0, nb, ring.full + 8 * (t & 1));
+}
+
+// every thread of the CTA, once per launch
+__device__ __forceinline__ void ring_init(TileRing& ring, unsigned long long* bars, int* left) {
+    ring.full = smem_u32(bars);
+    ring.left = left;
+    ring.phase = 0u;
+    ring.abort = 0;
+    if (threadIdx.x == 0) {
+        mbar_init(ring.full, 1u);
+        mbar_init(ring.full + 8, 1u);
+    }
+    __syncthreads();
+}
+
+// rho = omega . R and sig = omega . R' of one row (q padded to NP with zeros):
+// float on packed pairs of even and odd q, float64 over the n real ones in two
+// chains each
+template <typename T, int NP>
+__device__ __forceinline__ void grad_dots(const T* orow, const T* R, const T* dR, int n, T& rho, T& sig) {
+    if constexpr (sizeof(T) == 4) {
+        float2 rr = make_float2(0.f, 0.f), ss = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int p = 0; p < NP; p += 4) {
+            const V4<T> o4 = ld4<T>(orow + p);
+            const float2 olo = make_float2(o4.x, o4.y), ohi = make_float2(o4.z, o4.w);
+            rr = __ffma2_rn(olo, make_float2(R[p], R[p + 1]), rr);
+            rr = __ffma2_rn(ohi, make_float2(R[p + 2], R[p + 3]), rr);
+            ss = __ffma2_rn(olo, make_float2(dR[p], dR[p + 1]), ss);
+            ss = __ffma2_rn(ohi, make_float2(dR[p + 2], dR[p + 3]), ss);
+        }
+        rho = rr.x + rr.y;
+        sig = ss.x + ss.y;
+    } else {
+        T r0 = T(0), r1 = T(0), s0 = T(0), s1 = T(0);
+#pragma unroll
+        for (int p = 0; p < NP; p += 2) {
+            if (p < n) {   // uniform
+                const double2 o2 = *reinterpret_cast<const double2*>(orow + p);
+                r0 += o2.x * R[p];
+                s0 += o2.x * dR[p];
+                r1 += o2.y * R[p + 1];
+                s1 += o2.y * dR[p + 1];
+            }
+        }
+        rho = r0 + r1;
+        sig = s0 + s1;
+    }
+}
+
 // State of the tensor-core readout of one thread (TCM != 0).
 struct TcState {
     unsigned char* zhi;   // A operand: Z rows of the CTA's atoms (bf16)
@@ -532,17 +614,13 @@ struct TcState {
     int abort;            // a completion wait ran out: no further waits
 };
 
-// polls of an mbarrier before a readout MMA is declared lost (status bit
-// ST_TC_TIMEOUT, reported as MIX_ETIMEOUT)
-constexpr int TC_WAIT_POLLS = 1 << 20;
-
 // One group of atoms a0 .. a0 + WN - 1 of the system's expensive list (those
 // below nexp), warp w on atom a0 + w; every thread of the CTA calls it.
 // TCM != 0 (float only): the nu = 3 readout V = Z W runs on the tensor cores
 // for the CTA's TC_ACE_WARPS atoms at once (16 rows (atom, m3) per atom).
 template <typename T, int L, int NP, int QB, int TCM = 0>
 __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, int a0, int nexp, unsigned char* smem,
-                                          TcState* tc = nullptr, int wn = ACE_GROUP) {
+                                          TcState* tc = nullptr, int wn = ACE_GROUP, TileRing* ring = nullptr) {
     const int WN = TCM != 0 ? TC_ACE_WARPS : wn;   // warps (atoms) of the CTA
     constexpr int NLM = (L + 1) * (L + 1);
     constexpr int D = 2 * L + 1;
@@ -554,8 +632,13 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
     const int n = tab.n, cap = d.cap, ntau = tab.ntau;
     constexpr int ROWS = nu3_rows(L);
     const AceLay lay(tab.tile_max, cap, n, tab.qb, L, ROWS, NP, (int)sizeof(T), WN, TCM != 0 ? tc->nbuf : 2);
-    // the first tile lands while the warps run steps 1-3
-    if (ntau > 0) tile_fetch(tab.tiles, tab.tile_off, 0, smem);
+    // the first tile (the ring: two) lands while the warps run steps 1-3
+    if constexpr (TCM != 0) {
+        if (ntau > 0) tile_fetch(tab.tiles, tab.tile_off, 0, smem);
+    } else {
+        if (tid == 0 && !ring->abort)
+            for (int t = 0; t < 2 && t < ntau; ++t) ring_fetch(*ring, tab.tiles, tab.tile_off, t, smem + t * lay.tile, WN);
+    }
 
     unsigned char* wreg = smem + lay.o_w + warp * lay.wb;
     T* At = reinterpret_cast<T*>(wreg + lay.o_at);
@@ -593,14 +676,25 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
         T acc[NUL][4];
 #pragma unroll
         for (int j = 0; j < NUL; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = T(0);
+        // this lane's units (clamped: what the surplus lanes sum is not stored)
+        int ulm[NUL], uq4[NUL];
+#pragma unroll
+        for (int j = 0; j < NUL; ++j) {
+            const int u = lane + 32 * j < NU ? lane + 32 * j : 0;
+            ulm[j] = u / NQ4;
+            uq4[j] = (u - ulm[j] * NQ4) * 4;
+        }
+        typename PairFrame<T>::Pt ptn{};   // the next 32 slots' partners are loaded ahead
+        if (lane < m) ptn = PairFrame<T>::load(d, row[lane]);
         for (int b0 = 0; b0 < m; b0 += 32) {
             const int s = b0 + lane;
             bool ok = false;
             T dv[3] = {T(0), T(0), T(0)}, r2 = T(0);
             if (s < m) {
-                pf.vec(d, row[s], dv, r2);
+                pf.vec(d, ptn, dv, r2);
                 ok = r2 < rc2;
             }
+            if (s + 32 < m) ptn = PairFrame<T>::load(d, row[s + 32]);
             const unsigned bal = __ballot_sync(0xffffffffu, ok);
             const int kc = __popc(bal);
             if (ok) {
@@ -618,28 +712,27 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
                 }
             }
             __syncwarp();
+            // neighbours outermost and unrolled: every unit's loads of several
+            // neighbours are in flight at once
+#pragma unroll 4
+            for (int kl = 0; kl < kc; ++kl) {
 #pragma unroll
-            for (int j = 0; j < NUL; ++j) {
-                const int u = lane + 32 * j;
-                if (u < NU) {
-                    const int lm = u / NQ4, q4 = (u - lm * NQ4) * 4;
-                    for (int kl = 0; kl < kc; ++kl) {
-                        const T y = cY[kl * NLM + lm];
-                        const V4<T> r4 = ld4<T>(cR + kl * NP + q4);
-                        if constexpr (sizeof(T) == 4) {
-                            const float2 yy = make_float2(y, y);
-                            const float2 lo = __ffma2_rn(yy, make_float2(r4.x, r4.y), make_float2(acc[j][0], acc[j][1]));
-                            const float2 hi = __ffma2_rn(yy, make_float2(r4.z, r4.w), make_float2(acc[j][2], acc[j][3]));
-                            acc[j][0] = lo.x;
-                            acc[j][1] = lo.y;
-                            acc[j][2] = hi.x;
-                            acc[j][3] = hi.y;
-                        } else {
-                            acc[j][0] += y * r4.x;
-                            acc[j][1] += y * r4.y;
-                            acc[j][2] += y * r4.z;
-                            acc[j][3] += y * r4.w;
-                        }
+                for (int j = 0; j < NUL; ++j) {
+                    const T y = cY[kl * NLM + ulm[j]];
+                    const V4<T> r4 = ld4<T>(cR + kl * NP + uq4[j]);
+                    if constexpr (sizeof(T) == 4) {
+                        const float2 yy = make_float2(y, y);
+                        const float2 lo = __ffma2_rn(yy, make_float2(r4.x, r4.y), make_float2(acc[j][0], acc[j][1]));
+                        const float2 hi = __ffma2_rn(yy, make_float2(r4.z, r4.w), make_float2(acc[j][2], acc[j][3]));
+                        acc[j][0] = lo.x;
+                        acc[j][1] = lo.y;
+                        acc[j][2] = hi.x;
+                        acc[j][3] = hi.y;
+                    } else {
+                        acc[j][0] += y * r4.x;
+                        acc[j][1] += y * r4.y;
+                        acc[j][2] += y * r4.z;
+                        acc[j][3] += y * r4.w;
                     }
                 }
             }
@@ -698,13 +791,21 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
         __syncwarp();
     }
 
-    // 4. nu = 3, tile by tile (every thread takes part in the copies and barriers)
+    // 4. nu = 3, tile by tile
     if constexpr (TCM == 0) {
         for (int t = 0; t < ntau; ++t) {
-            cp_async_wait_all();
-            __syncthreads();   // tile t visible; every warp is done with the other buffer
-            if (t + 1 < ntau) tile_fetch(tab.tiles, tab.tile_off, t + 1, smem + ((t + 1) & 1) * lay.tile);
-            const unsigned char* tile = smem + (t & 1) * lay.tile;
+            // the CTA's warps start a triple together: each triple is code of its own
+            // (some 10 KB), and warps a triple apart fetch it one after the other (n =
+            // 12, lmax = 5: 1.26 ms without this barrier, 1.05 with it)
+            __syncthreads();
+            const int bsel = t & 1;
+            unsigned char* tile = smem + bsel * lay.tile;
+            if (!ring->abort && !mbar_wait(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, TC_WAIT_POLLS)) {
+                ring->abort = 1;
+                set_status(d.status, ST_TC_TIMEOUT);
+            }
+            if (ring->abort) continue;   // no tile: the barrier above is all that is left to do
+            ring->phase ^= 1u << bsel;
             if constexpr (sizeof(T) == 8) {
                 if (has) nu3_tile<NP>(tile, tab, At, om, U1, P1, lane, ep);
             } else if (has) {
@@ -714,6 +815,12 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
                 if (h.mode != 3) nu3_dense_u<NP, QB>(W, At + o3, n, d3, lane, U1);
                 nu3_mid_of<L, NP, QB, 0>(h.tri, At, om, U1, n, lane, Nu3Op{});
                 nu3_dense_w<NP, QB>(W, At + o3, n, d3, U1, om + o3, nu3_mult3(h), lane, ep);
+            }
+            __syncwarp();   // every lane is done with the tile
+            if (lane == 0) {
+                __threadfence_block();
+                if (atomicSub(ring->left + bsel, 1) == 1 && t + 2 < ntau)
+                    ring_fetch(*ring, tab.tiles, tab.tile_off, t + 2, tile, WN);
             }
         }
     } else {
@@ -843,64 +950,35 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
             radial<T, NP>(r, invrc, n, R, dR);
             T Pi[(L + 1) * (L + 2) / 2], C[L + 1], S[L + 1];
             legendre_tables<T, L>(x, y, z, Pi, C, S);
+            // Y_l,m and Y_l,-m share their polynomial and norm, so the two are taken
+            // together: with rho, sig of both,
+            //   sum sig Y = K Pi (sig+ C_m + sig- S_m),
+            //   sum rho grad Y = K m Pi (rho+ C_m-1 + rho- S_m-1, rho- C_m-1 - rho+ S_m-1, 0)
+            //                    + K Pi' (0, 0, rho+ C_m + rho- S_m);
+            // half the products of one m at a time, and four independent dot
+            // products in flight (float64: the latency of a single warp)
             T sy = T(0), Gx = T(0), Gy = T(0), Gz = T(0);
 #pragma unroll
             for (int l = 0; l <= L; ++l) {
-                const int pl = l * (l + 1) / 2;
+                const int pl = l * (l + 1) / 2, o = l * l + l;
+                {
+                    T rho, sig;
+                    grad_dots<T, NP>(om + o * NP, R, dR, n, rho, sig);
+                    const T kk = __ldg(K + o);
+                    sy += sig * (kk * Pi[pl]);
+                    if (l > 0) Gz += rho * (kk * Pi[pl + 1]);
+                }
 #pragma unroll
-                for (int mm = -l; mm <= l; ++mm) {
-                    const int lm = l * l + l + mm;
-                    const T* orow = om + lm * NP;
-                    T rho = T(0), sig = T(0);
-                    if constexpr (sizeof(T) == 4) {
-                        // even and odd q in packed pairs, added at the end
-                        float2 rr = make_float2(0.f, 0.f), ss = make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int p = 0; p < NP; p += 4) {
-                            const V4<T> o4 = ld4<T>(orow + p);
-                            const float2 olo = make_float2(o4.x, o4.y), ohi = make_float2(o4.z, o4.w);
-                            rr = __ffma2_rn(olo, make_float2(R[p], R[p + 1]), rr);
-                            rr = __ffma2_rn(ohi, make_float2(R[p + 2], R[p + 3]), rr);
-                            ss = __ffma2_rn(olo, make_float2(dR[p], dR[p + 1]), ss);
-                            ss = __ffma2_rn(ohi, make_float2(dR[p + 2], dR[p + 3]), ss);
-                        }
-                        rho = rr.x + rr.y;
-                        sig = ss.x + ss.y;
-                    } else {
-#pragma unroll
-                        for (int p = 0; p < NP; p += 4) {
-                            const V4<T> o4 = ld4<T>(orow + p);
-                            rho += o4.x * R[p] + o4.y * R[p + 1] + o4.z * R[p + 2] + o4.w * R[p + 3];
-                            sig += o4.x * dR[p] + o4.y * dR[p + 1] + o4.z * dR[p + 2] + o4.w * dR[p + 3];
-                        }
-                    }
-                    const int mu = mm < 0 ? -mm : mm;
-                    const T kk = __ldg(K + lm);
-                    const T p = Pi[pl + mu];
-                    const T pz = (mu < l) ? Pi[pl + mu + 1] : T(0);
-                    T yv, gx, gy, gz;
-                    if (mm == 0) {
-                        yv = kk * p;
-                        gx = T(0);
-                        gy = T(0);
-                        gz = kk * pz;
-                    } else if (mm > 0) {
-                        // p_{l,m} = K Pi C_m
-                        yv = kk * p * C[mu];
-                        gx = kk * p * T(mu) * C[mu - 1];
-                        gy = -kk * p * T(mu) * S[mu - 1];
-                        gz = kk * pz * C[mu];
-                    } else {
-                        // p_{l,-m} = K Pi S_m
-                        yv = kk * p * S[mu];
-                        gx = kk * p * T(mu) * S[mu - 1];
-                        gy = kk * p * T(mu) * C[mu - 1];
-                        gz = kk * pz * S[mu];
-                    }
-                    sy += sig * yv;
-                    Gx += rho * gx;
-                    Gy += rho * gy;
-                    Gz += rho * gz;
+                for (int mu = 1; mu <= l; ++mu) {
+                    T rp, sp, rm, sm;
+                    grad_dots<T, NP>(om + (o + mu) * NP, R, dR, n, rp, sp);
+                    grad_dots<T, NP>(om + (o - mu) * NP, R, dR, n, rm, sm);
+                    const T kk = __ldg(K + o + mu);
+                    const T kp = kk * Pi[pl + mu], km = kp * T(mu);
+                    sy += kp * (sp * C[mu] + sm * S[mu]);
+                    Gx += km * (rp * C[mu - 1] + rm * S[mu - 1]);
+                    Gy += km * (rm * C[mu - 1] - rp * S[mu - 1]);
+                    if (mu < l) Gz += kk * Pi[pl + mu + 1] * (rp * C[mu] + rm * S[mu]);
                 }
             }
             const T ug = x * Gx + y * Gy + z * Gz;
@@ -958,11 +1036,14 @@ template <typename T, int L, int NP, int QB>
 __global__ void __launch_bounds__(ACE_MAX_WARPS * 32, ace_min_ctas_max<T>()) k_ace(Dev d, AceTab<T> tab) {
     const int WN = (int)(blockDim.x >> 5);   // ACE_GROUP or ACE_MAX_WARPS atoms a CTA
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_g;
+    __shared__ int s_g, s_left[2];
+    __shared__ __align__(8) unsigned long long s_bar[2];
+    TileRing ring;
+    ring_init(ring, s_bar, s_left);
     const int count = list_ok(d) ? d.status[SW_NEXP] : 0;
     const int ng = (count + WN - 1) / WN;
     for (int g = ace_next_group(d, &s_g); g < ng; g = ace_next_group(d, &s_g))
-        ace_group<T, L, NP, QB>(d, tab, g * WN, count, smem_raw, nullptr, WN);
+        ace_group<T, L, NP, QB>(d, tab, g * WN, count, smem_raw, nullptr, WN, &ring);
     ace_groups_done(d);
 }
 
@@ -974,6 +1055,10 @@ __global__ void __launch_bounds__(ace_warps<T>() * 32, ace_min_ctas<T>()) kb_ace
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Dev s_dev;
     __shared__ AceTab<T> s_tab;
+    __shared__ int s_left[2];
+    __shared__ __align__(8) unsigned long long s_bar[2];
+    TileRing ring;
+    ring_init(ring, s_bar, s_left);
     const int count = list_ok(b.words) ? *b.count : 0;
     int cur = -1;
     for (int g = blockIdx.x; g < count; g += gridDim.x) {
@@ -985,7 +1070,7 @@ __global__ void __launch_bounds__(ace_warps<T>() * 32, ace_min_ctas<T>()) kb_ace
             __syncthreads();
             cur = e.x;
         }
-        ace_group<T, L, NP, QB>(s_dev, s_tab, e.y, s_dev.status[SW_NEXP], smem_raw);
+        ace_group<T, L, NP, QB>(s_dev, s_tab, e.y, s_dev.status[SW_NEXP], smem_raw, nullptr, ACE_GROUP, &ring);
     }
 }
 

@@ -295,7 +295,7 @@ __host__ __device__ constexpr int nu3_kw() {
 // spreads a 16-byte read over all banks, and all 32 lanes work.
 template <int NP, int QB>
 __device__ __forceinline__ void nu3_dense_u(const float* W, const float* A3, int n, int d3, int lane, float* uz) {
-    constexpr int NQ = nu3_nq<NP, QB>(), NH = NQ / 2, KU = nu3_ku<NP, QB>();
+    constexpr int NQ = nu3_nq<NP, QB>(), NH = NQ / 2, KU = nu3_ku<NP, QB>(), KMIN = nu3_kmin<NP, QB>();
     const int kn = n * NP;
     float2 w[KU][NH];
 #pragma unroll
@@ -304,34 +304,40 @@ __device__ __forceinline__ void nu3_dense_u(const float* W, const float* A3, int
         ld_row<NQ>(W + (k < kn ? k : 0) * NP, w[i]);
     }
     float* p = uz + lane;
-    for (int m3 = 0; m3 < d3; ++m3, A3 += NP, p += kn) {
-        float2 a[NH];
-        ld_row<NQ>(A3, a);
+    // two rows m3 at a time (independent chains), then the odd one
+    auto rows = [&](auto rc) {
+        constexpr int R = rc.value;
+        float2 a[R][NH];
+#pragma unroll
+        for (int r = 0; r < R; ++r) ld_row<NQ>(A3 + r * NP, a[r]);
 #pragma unroll
         for (int i = 0; i < KU; ++i) {
-            float2 s = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int j = 0; j < NH; ++j) s = __ffma2_rn(w[i][j], a[j], s);
-            if (lane + 32 * i < kn) p[32 * i] = s.x + s.y;
+            for (int r = 0; r < R; ++r) {
+                float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int j = 0; j < NH; ++j) s = __ffma2_rn(w[i][j], a[r][j], s);
+                if (32 * i + 31 < KMIN || lane + 32 * i < kn) p[r * kn + 32 * i] = s.x + s.y;
+            }
         }
-    }
+    };
+    int m3 = 0;
+    for (; m3 + 2 <= d3; m3 += 2, A3 += 2 * NP, p += 2 * kn) rows(std::integral_constant<int, 2>{});
+    if (m3 < d3) rows(std::integral_constant<int, 1>{});
     __syncwarp();
 }
 
 // Phase W: omega3 and the energy from the rows Z of the buffer.  Lane pair g
 // takes k = g, g + 16, .., lane t of the pair one half of the q3's, so that an
 // m3 row ends in a reduction of NP / 2 values over 16 pairs (7 shuffles for NP =
-// 12; with a lane per unit and all q3's it took 13) and no lane is idle.
+// 12; with a lane per unit and all q3's it took 13) and no lane is idle.  Two rows
+// are reduced together: the four dependent shuffle rounds are the row's critical
+// path where few warps share an SM.
 template <int NP, int QB>
 __device__ __forceinline__ void nu3_dense_w(const float* W, const float* A3, int n, int d3, const float* uz, float* o3,
                                             float mult3, int lane, float& ep) {
     constexpr int HQ = NP / 2, HP = HQ / 2, KW = nu3_kw<NP, QB>(), KMIN = nu3_kmin<NP, QB>();
     const int kn = n * NP, g = lane >> 1, t0 = (lane & 1) * HQ;
-    int q3o = 0, q3real = HQ;   // the omega3 entry this lane receives
-    bool q3w = false;
-    rs_entry<HQ, 16, 2>(lane, q3o, q3real, q3w);
-    q3o += t0;
-    q3w = q3w && q3o < n;
     float2 w[KW][HP];
 #pragma unroll
     for (int i = 0; i < KW; ++i) {
@@ -341,28 +347,43 @@ __device__ __forceinline__ void nu3_dense_w(const float* W, const float* A3, int
         for (int j = 0; j < HP; ++j) w[i][j] = k < kn ? r[j] : make_float2(0.f, 0.f);
     }
     const float* p = uz + g;
-    for (int m3 = 0; m3 < d3; ++m3, p += kn) {
-        float2 s[HP];
+    auto rows = [&](auto rc, int m3) {
+        constexpr int R = rc.value;
+        float2 s[R][HP];
 #pragma unroll
-        for (int j = 0; j < HP; ++j) s[j] = make_float2(0.f, 0.f);
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int j = 0; j < HP; ++j) s[r][j] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < KW; ++i) {
-            const float z = 16 * i + 15 < KMIN || g + 16 * i < kn ? p[16 * i] : 0.f;
 #pragma unroll
-            for (int j = 0; j < HP; ++j) s[j] = __ffma2_rn(w[i][j], make_float2(z, z), s[j]);
-        }
-        float pv[HQ];
+            for (int r = 0; r < R; ++r) {
+                const float z = 16 * i + 15 < KMIN || g + 16 * i < kn ? p[r * kn + 16 * i] : 0.f;
 #pragma unroll
-        for (int j = 0; j < HP; ++j) {
-            pv[2 * j] = s[j].x;
-            pv[2 * j + 1] = s[j].y;
+                for (int j = 0; j < HP; ++j) s[r][j] = __ffma2_rn(w[i][j], make_float2(z, z), s[r][j]);
+            }
         }
-        const float s3 = warp_rs<float, HQ, 16, 2>(pv, lane);
-        if (q3w) {
-            o3[m3 * NP + q3o] += mult3 * s3;
-            ep += A3[m3 * NP + q3o] * s3;
+        float pv[R * HQ];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int j = 0; j < HP; ++j) {
+                pv[r * HQ + 2 * j] = s[r][j].x;
+                pv[r * HQ + 2 * j + 1] = s[r][j].y;
+            }
+        int o = 0, real = R * HQ;   // the entry (row, q3) this lane receives
+        bool wr = false;
+        rs_entry<R * HQ, 16, 2>(lane, o, real, wr);
+        const float s3 = warp_rs<float, R * HQ, 16, 2>(pv, lane);
+        const int r = o >= HQ ? 1 : 0, q = o - r * HQ + t0;
+        if (wr && q < n) {
+            o3[(m3 + r) * NP + q] += mult3 * s3;
+            ep += A3[(m3 + r) * NP + q] * s3;
         }
-    }
+    };
+    int m3 = 0;
+    for (; m3 + 2 <= d3; m3 += 2, p += 2 * kn) rows(std::integral_constant<int, 2>{}, m3);
+    if (m3 < d3) rows(std::integral_constant<int, 1>{}, m3);
     __syncwarp();
 }
 

@@ -17,7 +17,7 @@ enum StatusBits : int {
     ST_NB3_OVERFLOW = 4,     // more than NB3MAX three-body neighbours
     ST_NONFINITE = 8,        // non-finite position or force
     ST_OUT_OF_BOX = 16,      // atom outside a non-periodic dimension
-    ST_TC_TIMEOUT = 32,      // a bounded wait for tensor-core MMAs gave up
+    ST_TC_TIMEOUT = 32,      // a bounded wait for tensor-core MMAs or a tile copy gave up
     ST_GRID_TIMEOUT = 64,    // a bounded wait at a grid barrier gave up
 };
 enum StatusWord : int {
