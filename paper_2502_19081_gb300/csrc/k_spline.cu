@@ -19,7 +19,7 @@ namespace mixd {
 
 constexpr int SPL_WARPS = 4;
 
-// three-body neighbours an atom may have on chip: NB3MAX with a warp per atom,
+// three-body neighbours whose pairs a group tabulates: NB3MAX with a warp per atom,
 // fewer with half or a quarter of a warp (the per-group tables grow as the square)
 template <int LPA>
 __host__ __device__ constexpr int spl_nb() {
@@ -111,6 +111,31 @@ __device__ __forceinline__ void spl_contract(const typename Vec4<T>::type* c, co
     }
 }
 
+// V3 of the pair (p, q), p < q, of three-body neighbours vp, vq (vector and
+// length) with dV3/dr_p, dV3/dr_q and (dV3/dr_pq) / r_pq
+template <typename T>
+__device__ __forceinline__ void spl_pair(const SplTab<T>& tab, const typename Vec4<T>::type& vp,
+                                         const typename Vec4<T>::type& vq, const typename Vec4<T>::type* c3w, T& val,
+                                         T& d1, T& d2, T& d3) {
+    const T wx = vq.x - vp.x, wy = vq.y - vp.y, wz = vq.z - vp.z;
+    const T w2 = wx * wx + wy * wy + wz * wz;
+    const T ri3 = w2 > T(0) ? trsqrt(w2) : T(0);
+    const T r3 = w2 * ri3;
+    int qa, qb, qc;
+    T ba[4], dba[4], bb[4], dbb[4], bc[4], dbc[4];
+    bspline4<T>(vp.w * tab.invh3, SPL_W3 - 1, qa, ba, dba);
+    bspline4<T>(vq.w * tab.invh3, SPL_W3 - 1, qb, bb, dbb);
+    bspline4<T>(r3 * tab.invhc, SPL_W3 - 1, qc, bc, dbc);
+    val = d1 = d2 = d3 = T(0);
+    if (tab.na - qa <= 2 && tab.na - qb <= 2)
+        spl_contract<T, 2>(c3w + (qa * 8 + qb) * SPL_W3 + qc, ba, dba, bb, dbb, bc, dbc, val, d1, d2, d3);
+    else
+        spl_contract<T, 4>(c3w + (qa * 8 + qb) * SPL_W3 + qc, ba, dba, bb, dbb, bc, dbc, val, d1, d2, d3);
+    d1 *= tab.invh3;
+    d2 *= tab.invh3;
+    d3 *= tab.invhc * ri3;
+}
+
 // One evaluated atom i (an entry of the system's cheap list), by the group of
 // LPA lanes that owns W; the coefficient windows c2w, c3w may sit in shared or
 // global memory.  Returns the atom's 3-body neighbour count (before any clamp
@@ -129,7 +154,7 @@ __device__ __forceinline__ int spline_atom(const Dev& d, const SplTab<T>& tab, i
     V* GIN = reinterpret_cast<V*>(d.gc_in);
     const int stamp = d.status[SW_EPOCH];
     const T rc2 = tab.rc2, rc32 = tab.rc32;
-    const T invh2 = tab.invh2, invh3 = tab.invh3, invhc = tab.invhc;
+    const T invh2 = tab.invh2;
     const unsigned lt = (1u << lane) - 1u;   // the ballots carry this group's lanes only
     const int cap = d.cap;
     int n3_all = 0;
@@ -208,7 +233,8 @@ __device__ __forceinline__ int spline_atom(const Dev& d, const SplTab<T>& tab, i
         }
         n3_all = n3;
         if (n3 > NB) {
-            if (sub == 0) {
+            // (an atom of a half warp is taken again by the whole warp: spl_again)
+            if (LPA != 16 && sub == 0) {
                 set_status(d.status, ST_NB3_OVERFLOW);
                 atomicMax(d.status + SW_NB3MAX, n3);
             }
@@ -219,25 +245,12 @@ __device__ __forceinline__ int spline_atom(const Dev& d, const SplTab<T>& tab, i
         const int npair = n3 * (n3 - 1) / 2;
         for (int t = sub; t < npair; t += LPA) {
             const int q = tq[t], p = t - q * (q - 1) / 2;
-            const V vp = W.v[p], vq = W.v[q];
-            const T wx = vq.x - vp.x, wy = vq.y - vp.y, wz = vq.z - vp.z;
-            const T w2 = wx * wx + wy * wy + wz * wz;
-            const T ri3 = w2 > T(0) ? trsqrt(w2) : T(0);
-            const T r3 = w2 * ri3;
-            int qa, qb, qc;
-            T ba[4], dba[4], bb[4], dbb[4], bc[4], dbc[4];
-            bspline4<T>(vp.w * invh3, SPL_W3 - 1, qa, ba, dba);
-            bspline4<T>(vq.w * invh3, SPL_W3 - 1, qb, bb, dbb);
-            bspline4<T>(r3 * invhc, SPL_W3 - 1, qc, bc, dbc);
-            T val = T(0), d1 = T(0), d2 = T(0), d3 = T(0);
-            if (tab.na - qa <= 2 && tab.na - qb <= 2)
-                spl_contract<T, 2>(c3w + (qa * 8 + qb) * SPL_W3 + qc, ba, dba, bb, dbb, bc, dbc, val, d1, d2, d3);
-            else
-                spl_contract<T, 4>(c3w + (qa * 8 + qb) * SPL_W3 + qc, ba, dba, bb, dbb, bc, dbc, val, d1, d2, d3);
+            T val, d1, d2, d3;
+            spl_pair<T>(tab, W.v[p], W.v[q], c3w, val, d1, d2, d3);
             ep += val;
-            W.a1[t] = d1 * invh3;
-            W.a2[t] = d2 * invh3;
-            W.cc[t] = d3 * invhc * ri3;
+            W.a1[t] = d1;
+            W.a2[t] = d2;
+            W.cc[t] = d3;
         }
         __syncwarp(mask);
         // 3-body slots: 2-body part plus the sum over the other 3-body neighbours
@@ -288,6 +301,24 @@ __device__ __forceinline__ int spline_atom(const Dev& d, const SplTab<T>& tab, i
     return n3_all;
 }
 
+// The atoms of a warp's two half-warp groups whose 3-body neighbours did not fit
+// the group's table are evaluated again by the whole warp, which has the room of
+// both tables (and overwrites every row the half warp wrote): so half warps take
+// the same atoms as a warp would, up to NB3MAX neighbours.  n3: the group's count.
+template <typename T>
+__device__ __forceinline__ void spl_again(const Dev& d, const SplTab<T>& tab, int i, int n3,
+                                          const typename Vec4<T>::type* c2w, const typename Vec4<T>::type* c3w,
+                                          const unsigned char* tq, SplWarp<T, spl_nb<16>()>* w2) {
+    static_assert(2 * sizeof(SplWarp<T, spl_nb<16>()>) >= sizeof(SplWarp<T, NB3MAX>), "room for a warp's table");
+    const unsigned over = __ballot_sync(0xffffffffu, n3 > spl_nb<16>());
+    for (int g = 0; g < 2; ++g)
+        if (over >> (16 * g) & 0xffffu) {
+            __syncwarp();
+            spline_atom<T, 32>(d, tab, __shfl_sync(0xffffffffu, i, 16 * g), c2w, c3w, tq,
+                               *reinterpret_cast<SplWarp<T, NB3MAX>*>(w2));
+        }
+}
+
 // window counts of the two coefficient tables (4-vectors)
 constexpr int SPL_NW = 64 * SPL_W3 + SPL_W2;
 
@@ -300,7 +331,7 @@ __device__ __forceinline__ void spl_stage(typename Vec4<T>::type* dst, const T* 
 }
 
 template <typename T, int LPA>
-__global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 1) k_spline(Dev d, SplTab<T> tab) {
+__global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 3) k_spline(Dev d, SplTab<T> tab) {
     constexpr int G = 32 / LPA;   // atoms a warp works on at a time
     constexpr int NB = spl_nb<LPA>();
     using V = typename Vec4<T>::type;
@@ -312,7 +343,7 @@ __global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 1) k_spli
     unsigned char* tq = reinterpret_cast<unsigned char*>(ws + SPL_WARPS * G);
     const int warp = threadIdx.x >> 5, grp = (threadIdx.x & 31) / LPA;
     spl_stage<T>(c3s, tab.c3w, tab.c2w);
-    spl_fill_tq<NB>(tq);
+    spl_fill_tq<LPA == 16 ? NB3MAX : NB>(tq);
     __syncthreads();
     const int count = list_ok(d) ? d.status[SW_NCHEAP] : 0;
     const int stride = gridDim.x * SPL_WARPS * G;
@@ -335,12 +366,16 @@ __global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 1) k_spli
     if (a < count) hd = load_head(i);
     int in = a + stride < count ? d.act_c[a + stride] : 0;
     int nb3 = 0;   // the largest 3-body count this lane's group met
-    while (a < count) {
+    // (half warps: both groups of a warp stay for as long as one has an atom)
+    while (LPA == 16 ? __any_sync(0xffffffffu, a < count) : a < count) {
         const int an = a + stride;
         const int inn = an + stride < count ? d.act_c[an + stride] : 0;
         AtomHead hn{0, 0, 0};
         if (an < count) hn = load_head(in);
-        nb3 = max(nb3, spline_atom<T, LPA>(d, tab, i, c2s, c3s, tq, ws[warp * G + grp], &hd));
+        int n3 = 0;
+        if (LPA != 16 || a < count) n3 = spline_atom<T, LPA>(d, tab, i, c2s, c3s, tq, ws[warp * G + grp], &hd);
+        nb3 = max(nb3, n3);
+        if constexpr (LPA == 16) spl_again<T>(d, tab, i, n3, c2s, c3s, tq, ws + warp * G);
         a = an;
         i = in;
         in = inn;
@@ -357,7 +392,7 @@ __global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 1) k_spli
 // shared memory, as the single-system kernel does; otherwise they are read
 // through L1.
 template <typename T, int LPA>
-__global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 1) kb_spline(const Dev* __restrict__ devs,
+__global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 3) kb_spline(const Dev* __restrict__ devs,
                                                            const SplTab<T>* __restrict__ tabs,
                                                            const int2* __restrict__ list, const int* count_p,
                                                            const int* words, int uniform) {
@@ -372,18 +407,34 @@ __global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 1) kb_spl
     unsigned char* tq = reinterpret_cast<unsigned char*>(ws + SPL_WARPS * G);
     const int warp = threadIdx.x >> 5, grp = (threadIdx.x & 31) / LPA;
     if (uniform) spl_stage<T>(c3s, tabs[0].c3w, tabs[0].c2w);
-    spl_fill_tq<NB>(tq);
+    spl_fill_tq<LPA == 16 ? NB3MAX : NB>(tq);
     __syncthreads();
     const int count = list_ok(words) ? *count_p : 0;
     const int stride = gridDim.x * SPL_WARPS * G;
     int g = (blockIdx.x * SPL_WARPS + warp) * G + grp;
     int2 e = g < count ? list[g] : make_int2(0, 0);
-    while (g < count) {   // the next entry is loaded ahead
+    while (LPA == 16 ? __any_sync(0xffffffffu, g < count) : g < count) {   // the next entry is loaded ahead
         const int gn = g + stride;
         const int2 en = gn < count ? list[gn] : make_int2(0, 0);
         const SplTab<T>& tab = tabs[e.x];
-        spline_atom<T, LPA>(devs[e.x], tab, e.y, uniform ? c2s : reinterpret_cast<const V*>(tab.c2w),
-                            uniform ? c3s : reinterpret_cast<const V*>(tab.c3w), tq, ws[warp * G + grp]);
+        const V* c2 = uniform ? c2s : reinterpret_cast<const V*>(tab.c2w);
+        const V* c3 = uniform ? c3s : reinterpret_cast<const V*>(tab.c3w);
+        int n3 = 0;
+        if (LPA != 16 || g < count) n3 = spline_atom<T, LPA>(devs[e.x], tab, e.y, c2, c3, tq, ws[warp * G + grp]);
+        if constexpr (LPA == 16) {
+            // the two groups' atoms may be of two systems
+            for (int h = 0; h < 2; ++h) {
+                const int over = __shfl_sync(0xffffffffu, n3, 16 * h) > spl_nb<16>();
+                const int es = __shfl_sync(0xffffffffu, e.x, 16 * h), ea = __shfl_sync(0xffffffffu, e.y, 16 * h);
+                if (over) {
+                    const SplTab<T>& ta = tabs[es];
+                    __syncwarp();
+                    spline_atom<T, 32>(devs[es], ta, ea, uniform ? c2s : reinterpret_cast<const V*>(ta.c2w),
+                                       uniform ? c3s : reinterpret_cast<const V*>(ta.c3w), tq,
+                                       *reinterpret_cast<SplWarp<T, NB3MAX>*>(ws + warp * G));
+                }
+            }
+        }
         g = gn;
         e = en;
     }
@@ -393,7 +444,7 @@ template <typename T, int LPA>
 static size_t spl_bytes() {
     constexpr int NB = spl_nb<LPA>();
     return SPL_NW * sizeof(typename Vec4<T>::type) + SPL_WARPS * (32 / LPA) * sizeof(SplWarp<T, NB>) +
-           spl_tq_bytes<NB>();
+           spl_tq_bytes<LPA == 16 ? NB3MAX : NB>();
 }
 
 template <typename T, int LPA>

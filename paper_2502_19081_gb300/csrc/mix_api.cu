@@ -837,10 +837,11 @@ int evaluate(mix_ctx* c, int integrate, double dt) {
 }
 
 int read_status(mix_ctx* c) {
-    cudaError_t e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamSynchronize");
-    e = cudaMemcpy(c->pinned, c->dev.status, SW_COUNT * sizeof(int), cudaMemcpyDeviceToHost);
+    // the copy is queued behind the work it reports on: one wait for both
+    cudaError_t e = cudaMemcpyAsync(c->pinned, c->dev.status, SW_COUNT * sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "status read");
+    e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamSynchronize");
     const int st = c->pinned[SW_STATUS];
     if (st & ST_NBR_OVERFLOW)
         return fail(c, MIX_EOVERFLOW, "neighbour list overflow: %d neighbours, capacity %d", c->pinned[SW_MAXNB], c->cap);
@@ -1048,16 +1049,18 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
         delete c;
         return e == cudaErrorInvalidValue ? MIX_EINVAL : MIX_ECUDA;
     }
-    // Fewer lanes per cheap atom where atoms have few neighbours: in a periodic
-    // bulk whose mean count inside the 3-body cutoff is at most a third of what
-    // the group holds on chip, a quarter warp (16 slots) up to 5.3 or half a warp
-    // (24 slots) up to 8; a warp (32 slots) otherwise.  Si has about 5, bcc Fe 12.
+    // Fewer lanes per cheap atom where atoms have few neighbours.  In a periodic bulk
+    // whose mean count inside the 3-body cutoff is at most a third of what a quarter
+    // warp holds on chip (16 slots), a quarter warp: Si has about 5.  Up to a mean
+    // of two thirds of a half warp's pair table (24), half a warp (whose atoms with
+    // up to 32 neighbours are taken by the whole warp, spl_again): bcc Fe has 12 to
+    // 14 (198,128 atoms 360 -> 306 us).  A warp otherwise.
     {
         bool bulk = vol > 0;
         for (int k = 0; k < 3; ++k) bulk = bulk && sys->periodic[k];
         const double rho = vol > 0 ? (double)sys->n_atoms / vol : 0.0;
         const double n3 = rho * 4.0 / 3.0 * M_PI * sp->r_cut3 * sp->r_cut3 * sp->r_cut3;
-        c->spl_lpa = !bulk ? 32 : (n3 * 3.0 <= spline_nb3(8) ? 8 : (n3 * 3.0 <= spline_nb3(16) ? 16 : 32));
+        c->spl_lpa = !bulk ? 32 : (n3 * 3.0 <= spline_nb3(8) ? 8 : (n3 * 1.5 <= spline_nb3(16) ? 16 : 32));
         c->spl_bulk = bulk;
     }
     e = spline_configure(c->precision, c->spl_lpa, &c->spl_smem, &c->spl_grid);

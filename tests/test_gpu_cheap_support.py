@@ -30,3 +30,45 @@ def test_support_of_the_coefficients(orc, last):
         err = np.abs(f[:, :3] - ref[:, :3]).max()
         assert err < (tol if tol is not None else 1e-4 * np.abs(ref).max())
         ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("atoms", [25, 29, 33])
+def test_half_warps_with_more_neighbours_than_their_table(orc, atoms):
+    """A dense spot in a bcc bulk, whose cheap kernel runs half warps: 24 to 32
+    three-body neighbours do not fit a half warp's table and go to the whole warp (the
+    oracle's forces, float64, 1e-10 of the largest force of the spot), one more is an
+    overflow."""
+    from paper_2502_19081_gb300 import mix
+    wl = I.small_fe_box(5, nx=8, ny=8, nz=8, r_core=2.0, ramp=1.0, vacancy=False)
+    s = wl.system
+    ctx = mix.open_context(wl, precision=mix.MIX_FP64, nbr_cap=192, regions=[])
+    assert ctx.info()["cheap_lanes"] == 16
+    x, v, _, _ = ctx.get_state()
+    # atoms of the spot on a small sphere about its first: every one a neighbour of it
+    k = np.arange(1, atoms)
+    z = 1 - (2 * k - 1) / (atoms - 1)
+    ph = k * np.pi * (3 - 5 ** 0.5)
+    r = 1.5
+    pts = np.concatenate([[[0, 0, 0]], r * np.stack([np.sqrt(1 - z * z) * np.cos(ph), np.sqrt(1 - z * z) * np.sin(ph), z], 1)])
+    # the spot takes the place of the atoms inside it; those left over go with them
+    ctr = np.array([0.37, 0.41, 0.46]) * s.box_len
+    dist = np.sum((x[:, :3] - ctr) ** 2, axis=1)
+    x2 = x.copy()
+    x2[np.argsort(dist)[:atoms], :3] = ctr + pts
+    ctx.set_state(x2, v)
+    n3 = [int(((d2 := np.sum((x2[:, :3] - p) ** 2, axis=1)) < wl.spline.r_cut3 ** 2).sum()) - 1 for p in ctr + pts]
+    if max(n3) > 32:
+        with pytest.raises(mix.MixError) as e:
+            ctx.forces()
+            ctx.sync()
+        assert e.value.code == mix.MIX_EOVERFLOW
+    else:
+        assert max(n3) >= 24
+        ctx.forces()
+        x3, _, f, _ = ctx.get_state()
+        assert ctx.info()["cheap_lanes"] == 16
+        import dataclasses as dc
+        ref, _, _ = orc.Model(dc.replace(wl, regions=[])).forces(x3, orc.MODE_METHOD)
+        assert np.abs(f[:, :3] - ref[:, :3]).max() < 1e-10 * max(1.0, np.abs(ref).max())
+    ctx.close()
