@@ -567,6 +567,14 @@ __device__ __forceinline__ void ring_init(TileRing& ring, unsigned long long* ba
     __syncthreads();
 }
 
+// before the CTA returns: after a wait that ran out, once more (bounded) for the
+// copies that may still be in flight
+__device__ __forceinline__ void ring_drain(const TileRing& ring) {
+    if (!ring.abort) return;
+    mbar_wait(ring.full, ring.phase & 1u, TC_WAIT_POLLS);
+    mbar_wait(ring.full + 8, (ring.phase >> 1) & 1u, TC_WAIT_POLLS);
+}
+
 // rho = omega . R and sig = omega . R' of one row (q padded to NP with zeros):
 // float on packed pairs of even and odd q, float64 over the n real ones in two
 // chains each
@@ -1044,6 +1052,7 @@ __global__ void __launch_bounds__(ACE_MAX_WARPS * 32, ace_min_ctas_max<T>()) k_a
     const int ng = (count + WN - 1) / WN;
     for (int g = ace_next_group(d, &s_g); g < ng; g = ace_next_group(d, &s_g))
         ace_group<T, L, NP, QB>(d, tab, g * WN, count, smem_raw, nullptr, WN, &ring);
+    ring_drain(ring);
     ace_groups_done(d);
 }
 
@@ -1072,6 +1081,7 @@ __global__ void __launch_bounds__(ace_warps<T>() * 32, ace_min_ctas<T>()) kb_ace
         }
         ace_group<T, L, NP, QB>(s_dev, s_tab, e.y, s_dev.status[SW_NEXP], smem_raw, nullptr, ACE_GROUP, &ring);
     }
+    ring_drain(ring);
 }
 
 // launch shape: the shared memory of the layout, and as many resident CTAs as fit
