@@ -396,9 +396,9 @@ __device__ __forceinline__ bool front_batch_build(const BatchPlan& p, Grid& grid
     return grid.barrier();
 }
 
-__device__ __forceinline__ bool front_batch_body(const FrontBatch& f, Grid& grid, Dev& d, Regions& r, unsigned char* smem) {
+__device__ __forceinline__ void front_batch_disp(const FrontBatch& f, Dev& d, Regions& r) {
     const BatchPlan& p = f.p;
-    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x, lane = threadIdx.x & 31;
+    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x;
     for (int k = blockIdx.x; k < nent; k += gx) {
         const int4 e = front_entry(p, k, &d, &r);
         const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
@@ -412,10 +412,11 @@ __device__ __forceinline__ bool front_batch_body(const FrontBatch& f, Grid& grid
             lambda_atom(d, r, i);   // stands unless the lists are rebuilt
         }
     }
-    if (!grid.barrier()) return false;
-    const bool rebuild = ld_acquire(p.words + SW_ANY) != 0;
-    if (rebuild && !front_batch_build(p, grid, d, r, smem)) return false;
-    // buffers; a warp's 32 atoms are its own, so it counts them at once
+}
+
+// buffers; a warp's 32 atoms are its own, so it counts them at once
+__device__ __forceinline__ void front_batch_buffer(const BatchPlan& p, Dev& d) {
+    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x, lane = threadIdx.x & 31;
     for (int k = blockIdx.x; k < nent; k += gx) {
         const int4 e = front_entry(p, k, &d, nullptr);
         buffer_dispatch(d, e.y, e.z, 32);
@@ -446,7 +447,10 @@ __device__ __forceinline__ bool front_batch_body(const FrontBatch& f, Grid& grid
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) p.words[SW_ANY] = 0;   // every CTA has read it
-    if (!grid.barrier()) return false;
+}
+
+__device__ __forceinline__ void front_batch_lists(const BatchPlan& p, Dev& d) {
+    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x;
     const FlatArgs& fa = p.flat;
     for (int k = blockIdx.x; k < nent; k += gx) {
         const int4 e = front_entry(p, k, &d, nullptr);
@@ -490,6 +494,16 @@ __device__ __forceinline__ bool front_batch_body(const FrontBatch& f, Grid& grid
             }
         }
     }
+}
+
+__device__ __forceinline__ bool front_batch_body(const FrontBatch& f, Grid& grid, Dev& d, Regions& r, unsigned char* smem) {
+    front_batch_disp(f, d, r);
+    if (!grid.barrier()) return false;
+    const bool rebuild = ld_acquire(f.p.words + SW_ANY) != 0;
+    if (rebuild && !front_batch_build(f.p, grid, d, r, smem)) return false;
+    front_batch_buffer(f.p, d);
+    if (!grid.barrier()) return false;
+    front_batch_lists(f.p, d);
     return true;
 }
 
@@ -505,6 +519,68 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) kb_front(const __gr
         for (int s = threadIdx.x; s < f.p.flat.nsys; s += FRONT_THREADS)
             set_status(f.p.flat.devs[s].status, ST_GRID_TIMEOUT);
     }
+}
+
+// Large batches: the same phases as kernels of their own, each with its own block
+// size, registers and as many warps an SM as these allow, and the list rows in
+// blocks of 4 warps, so that a system that rebuilds is spread over many SMs.  One
+// kernel for all of them has 32 warps an SM and 64 registers: with 3,236 entries
+// (256 Si cells, 1.59 M atoms) it took 462 us a step without a rebuild, 380 so, and
+// 5.9 ms when every member rebuilt, 1.9 so.
+enum { FB_DISP, FB_BIN, FB_SCAN, FB_FILL, FB_ROWS, FB_REV, FB_BUFFER, FB_LISTS };
+
+__host__ __device__ constexpr int fb_threads(int ph) { return ph == FB_ROWS ? 128 : (ph == FB_REV ? 256 : FRONT_THREADS); }
+__host__ __device__ constexpr int fb_blocks(int ph) { return ph == FB_ROWS ? 16 : (ph == FB_REV ? 4 : 1); }   // blocks an entry
+
+template <int PH>
+__global__ void __launch_bounds__(fb_threads(PH), PH == FB_ROWS ? 8 : (PH == FB_REV ? 1 : 2))
+    kb_front_phase(const __grid_constant__ FrontBatch f) {
+    extern __shared__ __align__(16) unsigned char front_smem[];
+    __shared__ Dev d;
+    __shared__ Regions r;
+    const BatchPlan& p = f.p;
+    if (!list_ok(p.words)) return;
+    if constexpr (PH == FB_DISP) {
+        front_batch_disp(f, d, r);
+    } else if constexpr (PH == FB_BUFFER) {
+        front_batch_buffer(p, d);
+    } else if constexpr (PH == FB_LISTS) {
+        front_batch_lists(p, d);
+    } else {
+        if (!p.words[SW_ANY]) return;
+        // this block's share of the system, a block a system for the scan
+        constexpr int NB = fb_blocks(PH);
+        int4 e = make_int4(blockIdx.x, 0, 1, 0);
+        if constexpr (PH != FB_SCAN) e = p.ba[BT_FRONT].tab[blockIdx.x / NB];
+        if (!p.flat.devs[e.x].status[SW_REBUILD]) return;   // the whole block
+        load_dev(&d, p.flat.devs + e.x);
+        if constexpr (PH == FB_BIN) copy_shared(&r, p.regions + e.x);
+        __syncthreads();
+        const int bx = e.y * NB + (int)(blockIdx.x % NB), gx = e.z * NB;
+        if constexpr (PH == FB_BIN) {
+            const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
+            if (i < d.n) {
+                cell_bin_atom(d, i);
+                lambda_atom(d, r, i);   // of the folded position
+            }
+        } else if constexpr (PH == FB_SCAN) {
+            cell_scan_body(d);
+        } else if constexpr (PH == FB_FILL) {
+            cell_fill_body(d, bx, gx);
+        } else if constexpr (PH == FB_ROWS) {
+            neigh_build_body<fb_threads(FB_ROWS) / 32>(d, bx, gx, pow2_cap(d.cap), reinterpret_cast<int*>(front_smem));
+        } else {
+            neigh_rev_body(d, bx, gx);
+        }
+    }
+}
+
+template <int PH>
+cudaError_t launch_front_phase(const FrontBatch& f, int units, size_t smem, cudaStream_t s) {
+    const cudaError_t e = raise_smem_limit((const void*)kb_front_phase<PH>, smem);
+    if (e != cudaSuccess) return e;
+    kb_front_phase<PH><<<units * fb_blocks(PH), fb_threads(PH), smem, s>>>(f);
+    return cudaPeekAtLastError();
 }
 
 // CTAs that are resident together with `smem` bytes each (0 on an error)
@@ -572,12 +648,28 @@ cudaError_t launch_front(const Dev& d, const Regions& r, const SeedRule& sr, cud
     return cudaLaunchCooperativeKernel((const void*)k_front, dim3(grid), dim3(FRONT_THREADS), args, smem, s);
 }
 
+// kernels of a batch's front: one up to two entries a resident CTA
+int front_batch_kernels(const BatchPlan& p) { return p.nblk[BT_FRONT] > 2 * FRONT_CTAS * sm_count() ? 8 : 1; }
+
 cudaError_t launch_front_batch(const BatchPlan& p, cudaStream_t s, int integrate, double dt) {
     static_assert(FRONT_ATOMS == FRONT_THREADS, "an entry's atoms are a CTA's threads");
     FrontBatch f{p, integrate, dt};
     const size_t smem = (size_t)FRONT_WARPS * p.capp2 * sizeof(int);
     const int lim = front_resident((const void*)kb_front, smem);
     if (lim < 1) return cudaErrorInvalidConfiguration;
+    if (front_batch_kernels(p) > 1) {
+        const int nent = p.nblk[BT_FRONT];
+        const size_t rows = (size_t)(fb_threads(FB_ROWS) / 32) * p.capp2 * sizeof(int);
+        cudaError_t e = launch_front_phase<FB_DISP>(f, nent, 0, s);
+        if (e == cudaSuccess) e = launch_front_phase<FB_BIN>(f, nent, 0, s);
+        if (e == cudaSuccess) e = launch_front_phase<FB_SCAN>(f, p.flat.nsys, 0, s);
+        if (e == cudaSuccess) e = launch_front_phase<FB_FILL>(f, nent, 0, s);
+        if (e == cudaSuccess) e = launch_front_phase<FB_ROWS>(f, nent, rows, s);
+        if (e == cudaSuccess) e = launch_front_phase<FB_REV>(f, nent, 0, s);
+        if (e == cudaSuccess) e = launch_front_phase<FB_BUFFER>(f, nent, 0, s);
+        if (e == cudaSuccess) e = launch_front_phase<FB_LISTS>(f, nent, 0, s);
+        return e;
+    }
     const int grid = std::max(1, std::min(lim, std::max(p.nblk[BT_FRONT], p.flat.nsys)));
     void* args[] = {&f};
     return cudaLaunchCooperativeKernel((const void*)kb_front, dim3(grid), dim3(FRONT_THREADS), args, smem, s);

@@ -205,25 +205,32 @@ __global__ void __launch_bounds__(G_WARPS * 32, sizeof(T) == 4 ? 4 : 2) k_gather
 
 // Each block belongs to one system and gathers with that system's own lane
 // groups, so a system's forces are bit for bit those it gets alone.
-// GB_ATOMS atoms a warp: with 32, 24 silicon cells made 601 blocks for 456 resident
-// ones, 1.3 waves; their step 285 us with 32, 284 with 16, 281 with 8.
-template <typename T>
+// GA atoms a warp: with 32, 24 silicon cells made 601 blocks for 456 resident
+// ones, 1.3 waves; their step 285 us with 32, 284 with 16, 281 with 8.  With four
+// waves of blocks of 32 the last one no longer counts and fewer blocks load their
+// system: 256 cells 400 us with 8, 342 with 32.
+template <typename T, int GA>
 __global__ void __launch_bounds__(G_WARPS * 32, sizeof(T) == 4 ? 4 : 2) kb_gather(BatchArgs ba, const double* __restrict__ hk, int integrate) {
-    __shared__ GSum<T> park[G_WARPS * GB_ATOMS * 6];
+    __shared__ GSum<T> park[G_WARPS * GA * 6];
     MIX_BATCH_BLOCK(ba)
     if (!list_ok(s_dev)) return;
     const double h = hk[s_ent.x];
     const int lpa = gather_lpa(s_dev);
-    if (lpa == 8) gather_body<T, 8>(s_dev, s_ent.y, s_ent.z, integrate, h, GB_ATOMS, park);
-    else if (lpa == 16) gather_body<T, 16>(s_dev, s_ent.y, s_ent.z, integrate, h, GB_ATOMS, park);
-    else gather_body<T, 32>(s_dev, s_ent.y, s_ent.z, integrate, h, GB_ATOMS, park);
+    if (lpa == 8) gather_body<T, 8>(s_dev, s_ent.y, s_ent.z, integrate, h, GA, park);
+    else if (lpa == 16) gather_body<T, 16>(s_dev, s_ent.y, s_ent.z, integrate, h, GA, park);
+    else gather_body<T, 32>(s_dev, s_ent.y, s_ent.z, integrate, h, GA, park);
 }
 
 void launch_gather_batch(const BatchPlan& p, int precision, int integrate, cudaStream_t s) {
-    if (precision == MIX_FP64)
-        kb_gather<double><<<p.nblk[BT_GATHER], G_WARPS * 32, 0, s>>>(p.ba[BT_GATHER], p.hk, integrate);
-    else
-        kb_gather<float><<<p.nblk[BT_GATHER], G_WARPS * 32, 0, s>>>(p.ba[BT_GATHER], p.hk, integrate);
+    const int nb = p.nblk[BT_GATHER];
+    const BatchArgs& ba = p.ba[BT_GATHER];
+    if (p.gather_atoms == GB_ATOMS_BIG) {
+        if (precision == MIX_FP64) kb_gather<double, GB_ATOMS_BIG><<<nb, G_WARPS * 32, 0, s>>>(ba, p.hk, integrate);
+        else kb_gather<float, GB_ATOMS_BIG><<<nb, G_WARPS * 32, 0, s>>>(ba, p.hk, integrate);
+    } else {
+        if (precision == MIX_FP64) kb_gather<double, GB_ATOMS><<<nb, G_WARPS * 32, 0, s>>>(ba, p.hk, integrate);
+        else kb_gather<float, GB_ATOMS><<<nb, G_WARPS * 32, 0, s>>>(ba, p.hk, integrate);
+    }
 }
 
 void launch_gather(const Dev& d, int precision, int integrate, double h, cudaStream_t s) {

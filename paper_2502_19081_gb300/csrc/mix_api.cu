@@ -1821,11 +1821,14 @@ int fused_build(mix_batch* b, double dt) {
     // block tables
     std::vector<std::vector<int4>> tabs(BT_COUNT);
     int capp2 = 32;
+    auto blocks = [](int64_t units, int64_t per) { return (int)std::max<int64_t>(1, (units + per - 1) / per); };
+    int64_t big = 0;   // blocks of the gather with GB_ATOMS_BIG atoms a warp
+    for (const Dev& d : devs) big += blocks(d.n, 8 * GB_ATOMS_BIG);
+    const int ga = big >= (int64_t)4 * 4 * sm_count() ? GB_ATOMS_BIG : GB_ATOMS;
     for (int s = 0; s < ns; ++s) {
         const Dev& d = devs[s];
         const int64_t n = d.n;
-        auto blocks = [](int64_t units, int64_t per) { return (int)std::max<int64_t>(1, (units + per - 1) / per); };
-        const int gx[BT_COUNT] = {blocks(n, FRONT_ATOMS), blocks(n, 8 * GB_ATOMS)};
+        const int gx[BT_COUNT] = {blocks(n, FRONT_ATOMS), blocks(n, 8 * ga)};
         for (int k = 0; k < BT_COUNT; ++k)
             for (int bx = 0; bx < gx[k]; ++bx) tabs[k].push_back(make_int4(s, bx, gx[k], 0));
         while (capp2 < d.cap) capp2 <<= 1;
@@ -1887,6 +1890,7 @@ int fused_build(mix_batch* b, double dt) {
         P.nblk[k] = (int)tabs[k].size();
     }
     P.regions = reinterpret_cast<const Regions*>(base + o_regs);
+    P.gather_atoms = ga;
     P.capp2 = capp2;
     P.hk = reinterpret_cast<const double*>(base + o_hk);
     P.words = reinterpret_cast<int*>(base + o_words);   // zero, as the whole upload's gaps are
@@ -1927,7 +1931,9 @@ int fused_build(mix_batch* b, double dt) {
     return MIX_OK;
 }
 
-int fused_launches(const mix_batch* b) { return 3 + (int)b->groups.size(); }   // front, cheap, gather
+int fused_launches(const mix_batch* b) {   // front, cheap, gather
+    return 2 + front_batch_kernels(b->plan) + (int)b->groups.size();
+}
 
 // one fused step (or force evaluation) captured on the batch's private stream
 int fused_graph(mix_batch* b, int integrate, double dt, cudaGraph_t* graph, cudaGraphExec_t* exec) {

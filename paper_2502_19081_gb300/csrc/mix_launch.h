@@ -48,12 +48,12 @@ void launch_gather(const Dev& d, int precision, int integrate, double h, cudaStr
 // ---------------------------------------------------------------------------
 // multi-system step (batches of contexts sharing one stream)
 
-constexpr int GB_ATOMS = 8;   // atoms a warp of the batched gather
+constexpr int GB_ATOMS = 8, GB_ATOMS_BIG = 32;   // atoms a warp of the batched gather (BatchPlan::gather_atoms)
 
 // Block-table classes: every batched launch uses the table of its granularity.
 enum BatchTabClass : int {
     BT_FRONT = 0,  // FRONT_ATOMS atoms (front)
-    BT_GATHER,     // 8 warps of GB_ATOMS atoms each (gather)
+    BT_GATHER,     // 8 warps of gather_atoms atoms each (gather)
     BT_COUNT
 };
 
@@ -75,12 +75,14 @@ struct BatchPlan {
     const Regions* regions;   // [nsys]
     const double* hk;         // [nsys] half-kick factors of the plan's time step
     int* words;               // [SW_COUNT] status bits, grid barrier and rebuild flag of the front
+    int gather_atoms;         // GB_ATOMS or GB_ATOMS_BIG
     int capp2;                // largest power-of-two list capacity (build scratch)
     FlatArgs flat;
 };
 
 // displacement, lists, weights, sets and their flattened lists of every system in
-// one cooperative launch (k_front.cu)
+// one cooperative launch, or, in large batches, a kernel a phase (k_front.cu)
+int front_batch_kernels(const BatchPlan& p);
 cudaError_t launch_front_batch(const BatchPlan& p, cudaStream_t s, int integrate, double dt);
 cudaError_t ace_batch_configure(int precision, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid);
 void launch_ace_batch(int precision, const Dev* devs, const void* tabs, const int2* list, const int* count,
