@@ -301,18 +301,15 @@ def errors_against(ctx_F, ctx_E, F_ref, E_ref, flags):
 
 def phase_bytes(name: str, n: int, nst: dict, rebuild_frac: float) -> float:
     """Algorithmic DRAM bytes per step of a memory-bound phase (atom-major
-    float64 rows of 32 B, int32 lists): disp reads x, v, f and writes x, v;
-    lists (rebuild steps only) read x and write cell ids, nnb and the sorted
-    rows and reverse slots; sets read x and the list and write weights and
-    flags; gather reads both potentials' own and incoming slot rows (16 B a
-    slot in float) and writes f, v."""
+    float64 rows of 32 B, int32 lists): disp, the one kernel in front of the
+    potentials, reads x, v, f and writes x, v, reads x and the list for the
+    weights and sets and writes weights and flags, and on rebuild steps reads x
+    and writes cell ids, nnb and the sorted rows and reverse slots (lists and
+    sets are empty phases); gather reads both potentials' own and incoming slot
+    rows (16 B a slot in float) and writes f, v."""
     nb = nst["nnb_list"]
     if name == "disp":
-        return n * 96.0
-    if name == "lists":
-        return rebuild_frac * n * (32.0 + 4.0 + 4.0 + 8.0 * nb)
-    if name == "sets":
-        return n * (32.0 + 4.0 * nb + 9.0 + 4.0)
+        return n * (96.0 + 32.0 + 4.0 * nb + 9.0 + 4.0) + rebuild_frac * n * (32.0 + 4.0 + 4.0 + 8.0 * nb)
     if name == "gather":
         return nst["n_exp"] * 2 * 16.0 * nst["nnb_exp_rc"] + nst["n_cheap"] * 2 * 16.0 * nst["nnb_cheap_rc"] + n * 72.0
     return 0.0
@@ -631,8 +628,8 @@ def ours(args):
         roof = {"kernel": "k_ace" if names[dom] == "exp" else "k_spline", "bound": "alu",
                 "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s", "frac": ach / peak,
                 "traffic": (profiled_traffic(f"k_ace_{mix.PREC_NAMES[prec]}_{wl.name}.md",
-                                             ("k_ace.cuh", "k_ace_f32.cu") if prec == mix.MIX_FP32 else
-                                             ("k_ace.cuh", "k_ace_tc.cuh", "k_ace_tc1.cu", "tc.cuh"))
+                                             ("k_nu3.cuh", "k_ace.cuh") if prec == mix.MIX_FP32 else
+                                             ("k_nu3.cuh", "k_ace.cuh", "k_ace_tc.cuh", "tc.cuh"))
                             if names[dom] == "exp" and prec != mix.MIX_FP64 else None),
                 "algorithmic_flops_per_launch": fl,
                 "peak_source": "measured FMA microbenchmark "
