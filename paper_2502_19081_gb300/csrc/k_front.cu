@@ -648,8 +648,9 @@ cudaError_t launch_front(const Dev& d, const Regions& r, const SeedRule& sr, cud
     return cudaLaunchCooperativeKernel((const void*)k_front, dim3(grid), dim3(FRONT_THREADS), args, smem, s);
 }
 
-// kernels of a batch's front: one up to two entries a resident CTA
-int front_batch_kernels(const BatchPlan& p) { return p.nblk[BT_FRONT] > 2 * FRONT_CTAS * sm_count() ? 8 : 1; }
+// kernels of a batch's front: one up to an entry an SM, where launches count.  24
+// silicon cells (some 312 entries): three steps 832 us with one, 818 with eight.
+int front_batch_kernels(const BatchPlan& p) { return p.nblk[BT_FRONT] > sm_count() ? 8 : 1; }
 
 cudaError_t launch_front_batch(const BatchPlan& p, cudaStream_t s, int integrate, double dt) {
     static_assert(FRONT_ATOMS == FRONT_THREADS, "an entry's atoms are a CTA's threads");

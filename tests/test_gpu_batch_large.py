@@ -1,4 +1,4 @@
-"""Batches of more than two front entries (512 atoms) a resident CTA take the
+"""Batches of more than one front entry (512 atoms) an SM take the
 front's phases as kernels of their own; from four waves of blocks on, also wider
 gather chunks.  Each member's trajectory, through list rebuilds, is bit for bit
 the one it has alone."""
@@ -9,7 +9,7 @@ from paper_2502_19081_gb300 import inputs as I
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("members", [56, 104])   # 672 and 1,248 entries of 608; 1,344 and 2,496 blocks of 2,432
+@pytest.mark.parametrize("members", [12, 13, 104])   # 144, 156 and 1,248 entries of 152; 288, 312 and 2,496 blocks of 2,432
 def test_large_batch_equals_members_alone(members):
     from paper_2502_19081_gb300 import build, mix
     build.build()
