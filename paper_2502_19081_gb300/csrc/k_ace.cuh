@@ -520,10 +520,6 @@ __device__ __forceinline__ void nu2_float(const AceTab<float>& tab, const float*
     }
 }
 
-// polls of an mbarrier before a copy or a readout MMA is declared lost (status
-// bit ST_TC_TIMEOUT, reported as MIX_ETIMEOUT)
-constexpr int TC_WAIT_POLLS = 1 << 20;
-
 // The CUDA-core kernels' tile ring: two buffers filled by bulk copies (one thread
 // issues a whole tile) that complete on an mbarrier each; two tiles are on their
 // way before the atom's density is formed.  A warp counts itself done with a tile,
@@ -535,7 +531,7 @@ struct TileRing {
     uint32_t full;       // two mbarriers, 8 bytes apart (shared address)
     int* left;           // [2] warps still to finish the buffer's tile
     uint32_t phase;      // bit b: parity of buffer b's next completion
-    int abort;           // a wait ran out: no further waits
+    int abort;           // a wait ran out: no further waits (uniform over the warp)
 };
 
 __device__ __forceinline__ void bulk_fetch(void* dst, const void* src, int bytes, uint32_t bar) {
@@ -563,16 +559,17 @@ __device__ __forceinline__ void ring_init(TileRing& ring, unsigned long long* ba
     if (threadIdx.x == 0) {
         mbar_init(ring.full, 1u);
         mbar_init(ring.full + 8, 1u);
+        left[0] = left[1] = 0;
     }
     __syncthreads();
 }
 
 // before the CTA returns: after a wait that ran out, once more (bounded) for the
-// copies that may still be in flight
+// copies that may still be in flight (a tile was issued and not finished by every warp)
 __device__ __forceinline__ void ring_drain(const TileRing& ring) {
     if (!ring.abort) return;
-    mbar_wait(ring.full, ring.phase & 1u, TC_WAIT_POLLS);
-    mbar_wait(ring.full + 8, (ring.phase >> 1) & 1u, TC_WAIT_POLLS);
+    for (int b = 0; b < 2; ++b)
+        if (*(volatile int*)(ring.left + b) > 0) mbar_wait(ring.full + 8 * b, (ring.phase >> b) & 1u, TC_WAIT_POLLS);
 }
 
 // rho = omega . R and sig = omega . R' of one row (q padded to NP with zeros):
@@ -808,9 +805,10 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
             __syncthreads();
             const int bsel = t & 1;
             unsigned char* tile = smem + bsel * lay.tile;
-            if (!ring->abort && !mbar_wait(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, TC_WAIT_POLLS)) {
+            // (abort is the same for all lanes of a warp: see mbar_wait_warp)
+            if (!ring->abort && !mbar_wait_warp(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, d.tile_polls)) {
                 ring->abort = 1;
-                set_status(d.status, ST_TC_TIMEOUT);
+                if (lane == 0) set_status(d.status, ST_TC_TIMEOUT);
             }
             if (ring->abort) continue;   // no tile: the barrier above is all that is left to do
             ring->phase ^= 1u << bsel;

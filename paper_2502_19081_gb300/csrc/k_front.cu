@@ -37,9 +37,6 @@ constexpr int FRONT_REDUNDANT_CELLS = 8192;
 // 61 against 65 us, 200,000
 // atoms 442 against 480 us).
 constexpr int FRONT_TILED_CELLS = 1000;
-// polls of the grid barrier before a launch gives up (status ST_GRID_TIMEOUT)
-constexpr int GRID_POLLS = 1 << 22;
-
 struct FrontOpt {
     int integrate, force_rebuild;
     double dt, h;
@@ -60,8 +57,8 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 // status bit stays, and every later kernel of the context does nothing (list_ok).
 struct Grid {
     int* status;
-    int target;
-    __device__ __forceinline__ explicit Grid(int* s) : status(s), target(0) {}
+    int target, limit;   // limit: polls before a wait gives up
+    __device__ __forceinline__ Grid(int* s, int polls) : status(s), target(0), limit(polls) {}
     __device__ __forceinline__ bool barrier() {
         __shared__ int s_ok;
         target += (int)gridDim.x;
@@ -69,10 +66,10 @@ struct Grid {
         if (threadIdx.x == 0) {
             asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(status + SW_GRID_COUNT) : "memory");
             int polls = 0;
-            while (ld_acquire(status + SW_GRID_COUNT) < target && ++polls < GRID_POLLS) {
+            while (ld_acquire(status + SW_GRID_COUNT) < target && ++polls < limit) {
             }
-            if (polls >= GRID_POLLS) set_status(status, ST_GRID_TIMEOUT);
-            s_ok = polls < GRID_POLLS;
+            if (polls >= limit) set_status(status, ST_GRID_TIMEOUT);
+            s_ok = polls < limit;
         }
         __syncthreads();
         return s_ok != 0;
@@ -273,7 +270,7 @@ __device__ __forceinline__ void front_lambda(const Dev& d, const Regions& r) {
 __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front(Dev d, Regions r, SeedRule sr, FrontOpt o, int apw) {
     extern __shared__ __align__(16) unsigned char front_smem[];
     if (!list_ok(d)) return;
-    Grid grid(d.status);
+    Grid grid(d.status, d.grid_polls);
     const int bx = (int)blockIdx.x, gx = (int)gridDim.x;
     const bool g0 = bx == 0 && threadIdx.x == 0;
     if (g0) disp_reset(d, o.force_rebuild);
@@ -312,7 +309,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front(Dev d, Regi
 // lists alone: positions copied and checked, counts cleared, then the build
 __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front_lists(Dev d, FrontOpt o) {
     extern __shared__ __align__(16) unsigned char front_smem[];
-    Grid grid(d.status);
+    Grid grid(d.status, d.grid_polls);
     const int64_t g0 = (int64_t)blockIdx.x * FRONT_THREADS + threadIdx.x, gs = (int64_t)gridDim.x * FRONT_THREADS;
     for (int64_t k = g0; k < d.cells.ncell; k += gs) d.cell_count[k] = 0;
     for_atoms(d.n, [&](int64_t i) {
@@ -512,7 +509,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) kb_front(const __gr
     __shared__ Dev s_dev;
     __shared__ Regions s_reg;
     if (!list_ok(f.p.words)) return;
-    Grid grid(f.p.words);
+    Grid grid(f.p.words, f.p.grid_polls);
     if (front_batch_body(f, grid, s_dev, s_reg, front_smem)) {
         grid.done();
     } else {   // a barrier gave up: no kernel may walk the systems' lists

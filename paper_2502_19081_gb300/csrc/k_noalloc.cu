@@ -100,6 +100,7 @@ extern "C" int mix_neighbours_noalloc(int64_t n_atoms, const double* x_dev, cons
     d.cells.ncell = (int)ncell;
     d.rlist2 = r_list * r_list;
     d.nbs = nb_screen(d.rlist2, d.box);
+    d.grid_polls = GRID_POLLS;
     unsigned char* base = nullptr;
     int st = scratch_address(&base);
     if (st) return st;

@@ -1009,6 +1009,8 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
     d.cap = c->cap;
     d.rlist2 = c->rlist * c->rlist;
     d.nbs = nb_screen(d.rlist2, d.box);
+    d.tile_polls = TC_WAIT_POLLS;
+    d.grid_polls = GRID_POLLS;
     d.half_skin2 = 0.25 * opt->skin * opt->skin;
     d.rce = a->r_cut;
     d.rce2 = a->r_cut * a->r_cut;
@@ -1205,6 +1207,16 @@ int mix_set_regions(mix_ctx* c, const mix_region* r, int n) {
     c->seedrule.mode = 0;
     c->regions_version++;
     c->forces_valid = false;
+    return MIX_OK;
+}
+
+int mix_set_wait_limits(mix_ctx* c, int tile_polls, int grid_polls) {
+    if (!c) return MIX_EINVAL;
+    if (tile_polls > TC_WAIT_POLLS || grid_polls > GRID_POLLS) return fail(c, MIX_EINVAL, "wait limits");
+    c->dev.tile_polls = tile_polls < 0 ? TC_WAIT_POLLS : tile_polls;
+    c->dev.grid_polls = grid_polls < 0 ? GRID_POLLS : grid_polls;
+    drop_graph(c);
+    c->regions_version++;   // batches holding this context re-plan
     return MIX_OK;
 }
 
@@ -1891,6 +1903,8 @@ int fused_build(mix_batch* b, double dt) {
     }
     P.regions = reinterpret_cast<const Regions*>(base + o_regs);
     P.gather_atoms = ga;
+    P.grid_polls = devs[0].grid_polls;
+    for (const Dev& d : devs) P.grid_polls = std::min(P.grid_polls, d.grid_polls);
     P.capp2 = capp2;
     P.hk = reinterpret_cast<const double*>(base + o_hk);
     P.words = reinterpret_cast<int*>(base + o_words);   // zero, as the whole upload's gaps are

@@ -44,6 +44,13 @@ enum StatusWord : int {
     SW_COUNT = 64,
 };
 
+// polls of an mbarrier before a copy or a readout MMA is declared lost (status bit
+// ST_TC_TIMEOUT), and of the grid barrier before a front gives up
+// (ST_GRID_TIMEOUT); both are reported as MIX_ETIMEOUT.  A context's own limits
+// are Dev::tile_polls and Dev::grid_polls.
+constexpr int TC_WAIT_POLLS = 1 << 20;
+constexpr int GRID_POLLS = 1 << 22;
+
 constexpr int NB3MAX = 32;          // three-body neighbours per atom handled on chip
 constexpr int MAX_CAP = 256;        // neighbour slots per atom
 constexpr int FRONT_ATOMS = 512;       // atoms of a block-table entry of the batched front (a thread each)
@@ -195,6 +202,8 @@ struct Dev {
     int grid_front_max;  // CTAs of the front kernel that are resident together
     int grid_buffer;     // most CTAs of the front kernel (16 warps each)
     int grid_gather;     // CTAs of the gather (8 warps each)
+    int tile_polls;      // polls of a coefficient tile's copy before it is given up
+    int grid_polls;      // polls of a grid barrier before the front is given up
 };
 
 // ---------------------------------------------------------------------------

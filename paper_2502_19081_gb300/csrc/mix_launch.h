@@ -76,6 +76,7 @@ struct BatchPlan {
     const double* hk;         // [nsys] half-kick factors of the plan's time step
     int* words;               // [SW_COUNT] status bits, grid barrier and rebuild flag of the front
     int gather_atoms;         // GB_ATOMS or GB_ATOMS_BIG
+    int grid_polls;           // the smallest of the members' Dev::grid_polls
     int capp2;                // largest power-of-two list capacity (build scratch)
     FlatArgs flat;
 };

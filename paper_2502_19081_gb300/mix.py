@@ -51,7 +51,7 @@ EXPORTS = [
     "mix_batch_destroy", "mix_batch_last_error", "mix_set_seeds", "mix_set_seed_rule", "mix_get_seeds",
     "mix_server_create", "mix_server_submit", "mix_server_tick", "mix_server_request", "mix_server_fetch",
     "mix_server_destroy", "mix_server_last_error", "mix_admission_plan", "mix_batch_set_fused", "mix_batch_info",
-    "mix_tc_selftest",
+    "mix_tc_selftest", "mix_set_wait_limits",
 ]
 
 MIX_PHASES = 6
@@ -157,6 +157,7 @@ def lib():
             L.mix_set_seed_rule.argtypes = [P, ctypes.c_double, ctypes.c_double, ctypes.c_double, ctypes.c_int,
                                             ctypes.c_double, ctypes.c_double]
             L.mix_get_seeds.argtypes = [P, ctypes.POINTER(ctypes.c_uint8), i64p]
+            L.mix_set_wait_limits.argtypes = [P, ctypes.c_int, ctypes.c_int]
             L.mix_forces.argtypes = [P]
             L.mix_server_create.argtypes = [ctypes.POINTER(mix_server_options), P, ctypes.POINTER(P)]
             L.mix_server_submit.argtypes = [P, ctypes.POINTER(mix_system), ctypes.POINTER(mix_ace),
@@ -288,9 +289,7 @@ class Context:
                 self.x[:self.n].copy_(torch.from_numpy(_f64(s.x)))
                 self.v[:self.n].copy_(torch.from_numpy(_f64(s.v)))
             torch.cuda.synchronize(self.device)
-            self._check(self.L.mix_bind(self.h, ctypes.c_void_p(self.x.data_ptr()), ctypes.c_void_p(self.v.data_ptr()),
-                                        ctypes.c_void_p(self.f.data_ptr()), ctypes.c_void_p(self.ws.data_ptr())),
-                        "mix_bind")
+            self.bind()
             self.set_regions(workload.regions if regions is None else regions)
         cap = ctypes.c_int()
         self.L.mix_get_neighbours(self.h, ctypes.byref(cap), None, None, None)
@@ -314,7 +313,18 @@ class Context:
         except Exception:
             pass
 
+    def bind(self):
+        """Bind the context's buffers (again, after MIX_ETIMEOUT: clears the device status)."""
+        with self._torch.cuda.device(self.device):
+            self._check(self.L.mix_bind(self.h, ctypes.c_void_p(self.x.data_ptr()), ctypes.c_void_p(self.v.data_ptr()),
+                                        ctypes.c_void_p(self.f.data_ptr()), ctypes.c_void_p(self.ws.data_ptr())),
+                        "mix_bind")
+
     # -- calls --------------------------------------------------------------
+    def set_wait_limits(self, tile_polls: int = -1, grid_polls: int = -1):
+        """Polls before the context's bounded device waits give up (-1: default, 0: at once)."""
+        self._check(self.L.mix_set_wait_limits(self.h, int(tile_polls), int(grid_polls)), "mix_set_wait_limits")
+
     def set_regions(self, regions):
         arr = _regions_array(regions)
         self._check(self.L.mix_set_regions(self.h, arr, len(regions)), "mix_set_regions")

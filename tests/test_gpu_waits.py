@@ -1,0 +1,114 @@
+"""The bounded device waits: a wait that runs out (its limit set to no polls at all)
+gives MIX_ETIMEOUT at the next synchronising call, ends by itself, and leaves a
+context that works again after it is bound again.  Nothing here hangs or faults:
+every barrier and copy waited for does complete."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2502_19081_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def mx():
+    from paper_2502_19081_gb300 import build, mix
+    build.build()
+    return mix
+
+
+def _gives_up(mx, call):
+    with pytest.raises(mx.MixError) as e:
+        call()
+    assert e.value.code == mx.MIX_ETIMEOUT
+
+
+PROBE = """
+#include "tc.cuh"
+// lanes below 16 may poll, the others not at all: the wait's verdicts, one a lane
+__global__ void k_probe(int* out) {
+    __shared__ __align__(8) unsigned long long bar;
+    if (threadIdx.x == 0) {
+        mixd::mbar_init(mixd::smem_u32(&bar), 1u);
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mixd::smem_u32(&bar)) : "memory");
+    }
+    __syncthreads();
+    out[threadIdx.x] = mixd::mbar_wait_warp(mixd::smem_u32(&bar), 0u, threadIdx.x < 16 ? 1 << 10 : 0);
+    out[32 + threadIdx.x] = mixd::mbar_wait_warp(mixd::smem_u32(&bar), 0u, 1 << 10);
+}
+extern "C" int probe(int* out) {
+    k_probe<<<1, 32>>>(out);
+    return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+def test_a_warp_has_one_verdict(tmp_path):
+    import torch
+    from paper_2502_19081_gb300 import build
+    nvcc = build.nvcc()
+    if shutil.which(nvcc) is None:
+        pytest.skip("no nvcc")
+    src, so = tmp_path / "probe.cu", tmp_path / "libprobe.so"
+    src.write_text(PROBE)
+    subprocess.run([nvcc, *build.ARCH, "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", build.CSRC, "-I",
+                    build.INCLUDE, str(src), "-o", str(so)], check=True)
+    out = torch.full((64,), -1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    assert ctypes.CDLL(str(so)).probe(ctypes.c_void_p(out.data_ptr())) == 0
+    v = out.cpu().numpy()
+    assert (v[:32] == 0).all() and (v[32:] == 1).all()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("lmax", [0, 3])    # one l-triple (the second tile buffer stays empty), several
+def test_tile_wait_runs_out(mx, prec, lmax):
+    c = mx.open_context(I.small_fe_box(3, n_rad=5, l_max=lmax, r_core=4.0), precision=prec)
+    c.forces()
+    _, _, f0, _ = c.get_state()
+    c.set_wait_limits(tile_polls=0)
+    c.forces()
+    _gives_up(mx, c.sync)
+    c.set_wait_limits()
+    c.bind()
+    c.forces()
+    assert np.array_equal(c.get_state()[2], f0)
+    c.close()
+
+
+@pytest.mark.parametrize("n", [200, 9000])
+def test_grid_barrier_runs_out(mx, n):
+    import torch
+    wl = I.serve_request(4, "Si", n, 0.1, 300.0, I.serve_potentials())
+    c = mx.open_context(wl, precision=mx.MIX_FP32)
+    c.forces()
+    x0, v0, f0, _ = c.get_state()
+    c.set_wait_limits(grid_polls=0)
+    c.step(1.0, 1)
+    _gives_up(mx, c.sync)
+    torch.cuda.synchronize()
+    x1, v1 = c.x.clone(), c.v.clone()
+    c.set_wait_limits()
+    c.step(1.0, 3)               # the context's kernels do nothing any more
+    _gives_up(mx, c.sync)
+    torch.cuda.synchronize()
+    assert torch.equal(c.x, x1) and torch.equal(c.v, v1)
+    c.bind()
+    c.set_state(x0, v0)
+    c.forces()
+    assert np.array_equal(c.get_state()[2], f0)
+    c.close()
+
+
+def test_limits_are_checked(mx):
+    c = mx.open_context(I.small_fe_box(3), precision=mx.MIX_FP32)
+    with pytest.raises(mx.MixError) as e:
+        c.set_wait_limits(tile_polls=2 ** 31 - 1)
+    assert e.value.code == mx.MIX_EINVAL
+    c.close()
