@@ -806,11 +806,13 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
             const int bsel = t & 1;
             unsigned char* tile = smem + bsel * lay.tile;
             // (abort is the same for all lanes of a warp: see mbar_wait_warp)
-            if (!ring->abort && !mbar_wait_warp(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, d.tile_polls)) {
+            if (!ring->abort && !mbar_wait_warp(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, d.tile_polls))
                 ring->abort = 1;
+            if (ring->abort) {   // no tile: the barrier above is all that is left to do
+                // (said for every group that goes without: a batch's next one may be another system's)
                 if (lane == 0) set_status(d.status, ST_TC_TIMEOUT);
+                continue;
             }
-            if (ring->abort) continue;   // no tile: the barrier above is all that is left to do
             ring->phase ^= 1u << bsel;
             if constexpr (sizeof(T) == 8) {
                 if (has) nu3_tile<NP>(tile, tab, At, om, U1, P1, lane, ep);

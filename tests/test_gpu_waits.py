@@ -112,3 +112,27 @@ def test_limits_are_checked(mx):
         c.set_wait_limits(tile_polls=2 ** 31 - 1)
     assert e.value.code == mx.MIX_EINVAL
     c.close()
+
+
+def test_tile_wait_in_a_batch_is_said_for_every_member_it_cost(mx):
+    """A CTA that gave up goes on to other members' atoms without their tiles: each of
+    them must report it, and one that does not must have the forces it has alone."""
+    pots = I.serve_potentials()
+    wls = [I.serve_request(50 + k, "Fe", 4000, 0.6, 300.0, pots) for k in range(3)]
+    members = [mx.open_context(wl, precision=mx.MIX_FP32) for wl in wls]
+    alone = [mx.open_context(wl, precision=mx.MIX_FP32) for wl in wls]
+    for c in members:
+        c.forces()
+        c.sync()
+    members[0].set_wait_limits(tile_polls=0)
+    b = mx.Batch(members)
+    b.set_fused(True)
+    b.step(1.0, 1)
+    _gives_up(mx, b.sync)
+    assert b.info()["fused"]
+    for k, (c, a) in enumerate(zip(members, alone)):
+        a.step(1.0, 1)
+        if c.stats(check=False)["status_bits"] & 32:
+            continue
+        assert k > 0 and np.array_equal(c.get_state()[2], a.get_state()[2])
+    b.close()
