@@ -214,11 +214,10 @@ int mix_bind(mix_ctx* ctx, double* x_dev, double* v_dev, double* f_dev, void* wo
 
 /* Limits of the context's bounded device waits, in polls: of the copy of a
  * coefficient tile (float and float64 expensive kernels) and of a grid barrier
- * of the kernel that opens an evaluation (a batch takes the smallest of its
- * members').  Negative: the default, which is also the largest accepted; 0: every
- * such wait gives up at once, so that a caller's handling of MIX_ETIMEOUT can
- * be exercised.  After MIX_ETIMEOUT the context is of use again from the next
- * mix_bind.  Takes effect at the next evaluation. */
+ * of the kernel that opens an evaluation.  Negative: the default, which is also
+ * the largest accepted; 0: every such wait gives up at once, so that a caller's
+ * handling of MIX_ETIMEOUT can be exercised.  After MIX_ETIMEOUT the context is
+ * of use again from the next mix_bind.  Takes effect at the next evaluation. */
 int mix_set_wait_limits(mix_ctx* ctx, int tile_polls, int grid_polls);
 
 /* Set the core regions (at most MIX_MAX_REGIONS; n = 0 gives lambda = 0

@@ -1068,7 +1068,7 @@ __global__ void __launch_bounds__(ace_warps<T>() * 32, ace_min_ctas<T>()) kb_ace
     __shared__ __align__(8) unsigned long long s_bar[2];
     TileRing ring;
     ring_init(ring, s_bar, s_left);
-    const int count = list_ok(b.words) ? *b.count : 0;
+    const int count = *b.count;
     int cur = -1;
     for (int g = blockIdx.x; g < count; g += gridDim.x) {
         const int2 e = b.list[g];

@@ -48,13 +48,13 @@ cudaError_t ace_batch_configure(int precision, int L, int n, int cap, int tile_m
 }
 
 void launch_ace_batch(int precision, const Dev* devs, const void* tabs, const int2* list, const int* count,
-                      const int* words, int n, int L, size_t smem, int grid, cudaStream_t s) {
+                      int n, int L, size_t smem, int grid, cudaStream_t s) {
     if (precision == MIX_FP64)
         OPS_F64[ace_class(n)].launch_batch(
-            AceBatch<double>{devs, static_cast<const AceTab<double>*>(tabs), list, count, words}, L, smem, grid, s);
+            AceBatch<double>{devs, static_cast<const AceTab<double>*>(tabs), list, count}, L, smem, grid, s);
     else
         OPS_F32[ace_class(n)]->launch_batch(
-            AceBatch<float>{devs, static_cast<const AceTab<float>*>(tabs), list, count, words}, L, smem, grid, s);
+            AceBatch<float>{devs, static_cast<const AceTab<float>*>(tabs), list, count}, L, smem, grid, s);
 }
 
 cudaError_t ace_tc_configure(int tcm, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid,

@@ -17,7 +17,6 @@ struct AceBatch {
     const AceTab<T>* tabs;
     const int2* list;
     const int* count;
-    const int* words;   // the plan's status words (list_ok)
 };
 
 template <typename T>

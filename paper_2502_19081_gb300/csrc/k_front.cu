@@ -328,206 +328,119 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front_lists(Dev d
     if (front_build(d, grid, o.capp2, o.tiled, front_smem)) grid.done();
 }
 
-// The front of every system of a batch.  The work comes in table entries of
-// FRONT_ATOMS consecutive atoms of one system (a thread each); a CTA walks its
-// entries in every phase, with the entry's system in shared memory.  The phases and
-// bodies are those of k_front, so a system's lists and sets are the ones it gets
-// alone; the list phases run when some system needs them and skip the others; the
-// compaction also writes the flattened lists the batched potentials walk.  As
-// twelve kernels this took 150 us of a step of 24 silicon cells (151,200 atoms),
-// 77 as one.
+// The front of every system of a batch: the phases of k_front as kernels of their
+// own.  The work comes in table entries of FRONT_ATOMS consecutive atoms of one
+// system (a thread each), a block an entry with the entry's system in shared
+// memory.  The bodies are those of k_front, so a system's lists and sets are the
+// ones it gets alone; the list phases return at once when no system needs them and
+// for the systems that do not; the compaction also writes the flattened lists the
+// batched potentials walk.
+// One cooperative launch for all phases, as for a single system, loses here: its 64
+// registers and 32 warps an SM hold in every phase, and in a batch some member
+// rebuilds in most steps, with its few entries on as many blocks.  Steps at 50 K,
+// 20 at a time, one kernel / eight, us: 2 systems of 1,000 silicon atoms 112 / 90, 8
+// of them 187 / 124, 24 of them 305 / 186, 11 of 5,831 atoms 294 / 219, 8 iron
+// systems of 1,023 atoms 424 / 322, 8 of 8,191 atoms 1,034 / 958; 256 of 5,831 silicon
+// atoms with every member rebuilding 5.9 / 1.9 ms for the front alone.
 struct FrontBatch {
     BatchPlan p;
     int integrate;
     double dt;
 };
 
-// opens an entry: its system in d (and regions in r), the entry in e
-__device__ __forceinline__ int4 front_entry(const BatchPlan& p, int k, Dev* d, Regions* r) {
-    __shared__ int4 s_ent;
-    __syncthreads();   // the previous entry is done with
-    if (threadIdx.x == 0) s_ent = p.ba[BT_FRONT].tab[k];
-    __syncthreads();
-    const int4 e = s_ent;
-    load_dev(d, p.flat.devs + e.x);
-    if (r) copy_shared(r, p.regions + e.x);
-    __syncthreads();
-    return e;
-}
+enum { FB_DISP, FB_BIN, FB_SCAN, FB_FILL, FB_ROWS, FB_REV, FB_BUFFER, FB_LISTS, FB_COUNT };
 
-__device__ __forceinline__ bool front_batch_build(const BatchPlan& p, Grid& grid, Dev& d, Regions& r,
-                                                  unsigned char* smem) {
-    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x;
-    for (int k = blockIdx.x; k < nent; k += gx) {
-        const int4 e = front_entry(p, k, &d, nullptr);
-        const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-        if (d.status[SW_REBUILD] && i < d.n) cell_bin_atom(d, i);
-    }
-    if (!grid.barrier()) return false;
-    for (int s = blockIdx.x; s < p.flat.nsys; s += gx) {
-        __syncthreads();
-        load_dev(&d, p.flat.devs + s);
-        __syncthreads();
-        if (d.status[SW_REBUILD]) cell_scan_body(d);
-    }
-    if (!grid.barrier()) return false;
-    for (int k = blockIdx.x; k < nent; k += gx) {
-        const int4 e = front_entry(p, k, &d, nullptr);
-        if (d.status[SW_REBUILD]) cell_fill_body(d, e.y, e.z);
-    }
-    if (!grid.barrier()) return false;
-    for (int k = blockIdx.x; k < nent; k += gx) {
-        const int4 e = front_entry(p, k, &d, nullptr);
-        if (d.status[SW_REBUILD])
-            neigh_build_body<FRONT_WARPS>(d, e.y, e.z, pow2_cap(d.cap), reinterpret_cast<int*>(smem));
-    }
-    if (!grid.barrier()) return false;
-    for (int k = blockIdx.x; k < nent; k += gx) {
-        const int4 e = front_entry(p, k, &d, &r);
-        const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-        if (d.status[SW_REBUILD]) {
-            neigh_rev_body(d, e.y, e.z);
-            if (i < d.n) lambda_atom(d, r, i);
-        }
-    }
-    return grid.barrier();
-}
+// list rows in blocks of 4 warps, so that a system that rebuilds is spread over many SMs
+__host__ __device__ constexpr int fb_threads(int ph) { return ph == FB_ROWS ? 128 : (ph == FB_REV ? 256 : FRONT_THREADS); }
+__host__ __device__ constexpr int fb_blocks(int ph) { return ph == FB_ROWS ? 16 : (ph == FB_REV ? 4 : 1); }   // blocks an entry
 
-__device__ __forceinline__ void front_batch_disp(const FrontBatch& f, Dev& d, Regions& r) {
-    const BatchPlan& p = f.p;
-    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x;
-    for (int k = blockIdx.x; k < nent; k += gx) {
-        const int4 e = front_entry(p, k, &d, &r);
-        const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-        if (e.y == 0 && threadIdx.x == 0) {
-            disp_reset(d, 0);
-            d.status[SW_NEXP] = 0;
-            d.status[SW_NCHEAP] = 0;
-        }
-        if (i < d.n) {
-            if (disp_atom(d, i, f.integrate, f.dt, p.hk[e.x], 0)) p.words[SW_ANY] = 1;
-            lambda_atom(d, r, i);   // stands unless the lists are rebuilt
-        }
+__device__ __forceinline__ void front_batch_disp(const FrontBatch& f, const int4& e, const Dev& d, const Regions& r) {
+    const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
+    if (e.y == 0 && threadIdx.x == 0) {
+        disp_reset(d, 0);
+        d.status[SW_NEXP] = 0;
+        d.status[SW_NCHEAP] = 0;
+    }
+    if (i < d.n) {
+        if (disp_atom(d, i, f.integrate, f.dt, f.p.hk[e.x], 0)) *f.p.any = 1;
+        lambda_atom(d, r, i);   // stands unless the lists are rebuilt
     }
 }
 
 // buffers; a warp's 32 atoms are its own, so it counts them at once
-__device__ __forceinline__ void front_batch_buffer(const BatchPlan& p, Dev& d) {
-    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x, lane = threadIdx.x & 31;
-    for (int k = blockIdx.x; k < nent; k += gx) {
-        const int4 e = front_entry(p, k, &d, nullptr);
-        buffer_dispatch(d, e.y, e.z, 32);
-        const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-        const bool in = i < d.n;
-        const int fl = in ? d.flags[i] : 0;
-        const double lam = in ? d.lam[i] : 0.0;
-        const int2 own = block_sum2((fl >> 2) & 1, (fl >> 3) & 1);
-        if (threadIdx.x == 0) {
-            d.blk_e[e.y] = own.x;
-            d.blk_c[e.y] = own.y;
-            if (own.x) atomicAdd(d.status + SW_NEXP, own.x);
-            if (own.y) atomicAdd(d.status + SW_NCHEAP, own.y);
-            if (e.y == 0 && d.status[SW_REBUILD]) {
-                d.status[SW_REBUILDS] += 1;
-                d.status[SW_REBUILD] = 0;
-            }
+__device__ __forceinline__ void front_batch_buffer(const BatchPlan& p, const int4& e, const Dev& d) {
+    const int lane = threadIdx.x & 31;
+    buffer_dispatch(d, e.y, e.z, 32);
+    const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
+    const bool in = i < d.n;
+    const int fl = in ? d.flags[i] : 0;
+    const double lam = in ? d.lam[i] : 0.0;
+    const int2 own = block_sum2((fl >> 2) & 1, (fl >> 3) & 1);
+    if (threadIdx.x == 0) {
+        d.blk_e[e.y] = own.x;
+        d.blk_c[e.y] = own.y;
+        if (own.x) atomicAdd(d.status + SW_NEXP, own.x);
+        if (own.y) atomicAdd(d.status + SW_NCHEAP, own.y);
+        if (e.y == 0 && d.status[SW_REBUILD]) {
+            d.status[SW_REBUILDS] += 1;
+            d.status[SW_REBUILD] = 0;
         }
-        const int ncore = __popc(__ballot_sync(0xffffffffu, in && lam == 1.0));
-        const int nramp = __popc(__ballot_sync(0xffffffffu, in && lam > 0.0 && lam < 1.0));
-        const int nle = __popc(__ballot_sync(0xffffffffu, (fl & 1) != 0));
-        const int nlc = __popc(__ballot_sync(0xffffffffu, (fl & 2) != 0));
-        if (lane == 0) {
-            if (ncore) atomicAdd(d.status + SW_NCORE, ncore);
-            if (nramp) atomicAdd(d.status + SW_NRAMP, nramp);
-            if (nle) atomicAdd(d.status + SW_NLE, nle);
-            if (nlc) atomicAdd(d.status + SW_NLC, nlc);
-        }
+        if (blockIdx.x == 0) *p.any = 0;   // the list phases are over
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) p.words[SW_ANY] = 0;   // every CTA has read it
+    const int ncore = __popc(__ballot_sync(0xffffffffu, in && lam == 1.0));
+    const int nramp = __popc(__ballot_sync(0xffffffffu, in && lam > 0.0 && lam < 1.0));
+    const int nle = __popc(__ballot_sync(0xffffffffu, (fl & 1) != 0));
+    const int nlc = __popc(__ballot_sync(0xffffffffu, (fl & 2) != 0));
+    if (lane == 0) {
+        if (ncore) atomicAdd(d.status + SW_NCORE, ncore);
+        if (nramp) atomicAdd(d.status + SW_NRAMP, nramp);
+        if (nle) atomicAdd(d.status + SW_NLE, nle);
+        if (nlc) atomicAdd(d.status + SW_NLC, nlc);
+    }
 }
 
-__device__ __forceinline__ void front_batch_lists(const BatchPlan& p, Dev& d) {
-    const int nent = p.nblk[BT_FRONT], gx = (int)gridDim.x;
+__device__ __forceinline__ void front_batch_lists(const BatchPlan& p, const int4& e, const Dev& d) {
     const FlatArgs& fa = p.flat;
-    for (int k = blockIdx.x; k < nent; k += gx) {
-        const int4 e = front_entry(p, k, &d, nullptr);
-        const int s = e.x;
-        // this entry's place in its system's lists, and the system's in the flattened ones
-        int se = 0, sc = 0, oe = 0, oc = 0;
-        for (int t = threadIdx.x; t < e.y; t += FRONT_THREADS) {
-            se += d.blk_e[t];
-            sc += d.blk_c[t];
+    const int s = e.x;
+    // this entry's place in its system's lists, and the system's in the flattened ones
+    int se = 0, sc = 0, oe = 0, oc = 0;
+    for (int t = threadIdx.x; t < e.y; t += FRONT_THREADS) {
+        se += d.blk_e[t];
+        sc += d.blk_c[t];
+    }
+    const int g = fa.egroup[s];
+    for (int t = threadIdx.x; t < s; t += FRONT_THREADS) {
+        const int* st = fa.devs[t].status;
+        if (fa.egroup[t] == g) oe += (st[SW_NEXP] + ACE_GROUP - 1) / ACE_GROUP;
+        oc += st[SW_NCHEAP];
+    }
+    const int2 before = block_sum2(se, sc), flat = block_sum2(oe, oc);
+    const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
+    const bool in = i < d.n;
+    const int fl = in ? d.flags[i] : 0;
+    const int ie = (fl >> 2) & 1, ic = (fl >> 3) & 1;
+    int2 tot;
+    const int2 ex = block_scan2(ie, ic, &tot);
+    if (in) {
+        const int pe = before.x + ex.x, pc = before.y + ex.y;
+        if (ie) d.act_e[pe] = (int)i;
+        if (ic) {
+            d.act_c[pc] = (int)i;
+            fa.list_c[flat.y + pc] = make_int2(s, (int)i);
         }
-        const int g = fa.egroup[s];
-        for (int t = threadIdx.x; t < s; t += FRONT_THREADS) {
-            const int* st = fa.devs[t].status;
-            if (fa.egroup[t] == g) oe += (st[SW_NEXP] + ACE_GROUP - 1) / ACE_GROUP;
-            oc += st[SW_NCHEAP];
-        }
-        const int2 before = block_sum2(se, sc), flat = block_sum2(oe, oc);
-        const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-        const bool in = i < d.n;
-        const int fl = in ? d.flags[i] : 0;
-        const int ie = (fl >> 2) & 1, ic = (fl >> 3) & 1;
-        int2 tot;
-        const int2 ex = block_scan2(ie, ic, &tot);
-        if (in) {
-            const int pe = before.x + ex.x, pc = before.y + ex.y;
-            if (ie) d.act_e[pe] = (int)i;
-            if (ic) {
-                d.act_c[pc] = (int)i;
-                fa.list_c[flat.y + pc] = make_int2(s, (int)i);
-            }
-            d.pos_e[i] = ie ? pe : -1;
-            d.pos_c[i] = ic ? pc : -1;
-        }
-        if (e.y == 0) {
-            const int ne = (d.status[SW_NEXP] + ACE_GROUP - 1) / ACE_GROUP, nc = d.status[SW_NCHEAP];
-            int2* le = fa.list_e + fa.ebase[g] + flat.x;
-            for (int t = threadIdx.x; t < ne; t += FRONT_THREADS) le[t] = make_int2(s, t * ACE_GROUP);
-            if (threadIdx.x == 0) {
-                if (fa.elast[s]) fa.counts[g] = flat.x + ne;
-                if (s == fa.nsys - 1) fa.counts[fa.ngrp] = flat.y + nc;
-            }
+        d.pos_e[i] = ie ? pe : -1;
+        d.pos_c[i] = ic ? pc : -1;
+    }
+    if (e.y == 0) {
+        const int ne = (d.status[SW_NEXP] + ACE_GROUP - 1) / ACE_GROUP, nc = d.status[SW_NCHEAP];
+        int2* le = fa.list_e + fa.ebase[g] + flat.x;
+        for (int t = threadIdx.x; t < ne; t += FRONT_THREADS) le[t] = make_int2(s, t * ACE_GROUP);
+        if (threadIdx.x == 0) {
+            if (fa.elast[s]) fa.counts[g] = flat.x + ne;
+            if (s == fa.nsys - 1) fa.counts[fa.ngrp] = flat.y + nc;
         }
     }
 }
-
-__device__ __forceinline__ bool front_batch_body(const FrontBatch& f, Grid& grid, Dev& d, Regions& r, unsigned char* smem) {
-    front_batch_disp(f, d, r);
-    if (!grid.barrier()) return false;
-    const bool rebuild = ld_acquire(f.p.words + SW_ANY) != 0;
-    if (rebuild && !front_batch_build(f.p, grid, d, r, smem)) return false;
-    front_batch_buffer(f.p, d);
-    if (!grid.barrier()) return false;
-    front_batch_lists(f.p, d);
-    return true;
-}
-
-__global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) kb_front(const __grid_constant__ FrontBatch f) {
-    extern __shared__ __align__(16) unsigned char front_smem[];
-    __shared__ Dev s_dev;
-    __shared__ Regions s_reg;
-    if (!list_ok(f.p.words)) return;
-    Grid grid(f.p.words, f.p.grid_polls);
-    if (front_batch_body(f, grid, s_dev, s_reg, front_smem)) {
-        grid.done();
-    } else {   // a barrier gave up: no kernel may walk the systems' lists
-        for (int s = threadIdx.x; s < f.p.flat.nsys; s += FRONT_THREADS)
-            set_status(f.p.flat.devs[s].status, ST_GRID_TIMEOUT);
-    }
-}
-
-// Large batches: the same phases as kernels of their own, each with its own block
-// size, registers and as many warps an SM as these allow, and the list rows in
-// blocks of 4 warps, so that a system that rebuilds is spread over many SMs.  One
-// kernel for all of them has 32 warps an SM and 64 registers: with 3,236 entries
-// (256 Si cells, 1.59 M atoms) it took 462 us a step without a rebuild, 380 so, and
-// 5.9 ms when every member rebuilt, 1.9 so.
-enum { FB_DISP, FB_BIN, FB_SCAN, FB_FILL, FB_ROWS, FB_REV, FB_BUFFER, FB_LISTS };
-
-__host__ __device__ constexpr int fb_threads(int ph) { return ph == FB_ROWS ? 128 : (ph == FB_REV ? 256 : FRONT_THREADS); }
-__host__ __device__ constexpr int fb_blocks(int ph) { return ph == FB_ROWS ? 16 : (ph == FB_REV ? 4 : 1); }   // blocks an entry
 
 template <int PH>
 __global__ void __launch_bounds__(fb_threads(PH), PH == FB_ROWS ? 8 : (PH == FB_REV ? 1 : 2))
@@ -536,39 +449,37 @@ __global__ void __launch_bounds__(fb_threads(PH), PH == FB_ROWS ? 8 : (PH == FB_
     __shared__ Dev d;
     __shared__ Regions r;
     const BatchPlan& p = f.p;
-    if (!list_ok(p.words)) return;
+    constexpr bool LISTS = PH != FB_DISP && PH != FB_BUFFER && PH != FB_LISTS;   // a phase of the rebuild
+    if (LISTS && !*p.any) return;
+    // this block's share of the system, a block a system for the scan
+    constexpr int NB = fb_blocks(PH);
+    int4 e = make_int4(blockIdx.x, 0, 1, 0);
+    if constexpr (PH != FB_SCAN) e = p.ba[BT_FRONT].tab[blockIdx.x / NB];
+    if (LISTS && !p.flat.devs[e.x].status[SW_REBUILD]) return;   // the whole block
+    load_dev(&d, p.flat.devs + e.x);
+    if constexpr (PH == FB_DISP || PH == FB_BIN) copy_shared(&r, p.regions + e.x);
+    __syncthreads();
+    const int bx = e.y * NB + (int)(blockIdx.x % NB), gx = e.z * NB;
     if constexpr (PH == FB_DISP) {
-        front_batch_disp(f, d, r);
+        front_batch_disp(f, e, d, r);
     } else if constexpr (PH == FB_BUFFER) {
-        front_batch_buffer(p, d);
+        front_batch_buffer(p, e, d);
     } else if constexpr (PH == FB_LISTS) {
-        front_batch_lists(p, d);
-    } else {
-        if (!p.words[SW_ANY]) return;
-        // this block's share of the system, a block a system for the scan
-        constexpr int NB = fb_blocks(PH);
-        int4 e = make_int4(blockIdx.x, 0, 1, 0);
-        if constexpr (PH != FB_SCAN) e = p.ba[BT_FRONT].tab[blockIdx.x / NB];
-        if (!p.flat.devs[e.x].status[SW_REBUILD]) return;   // the whole block
-        load_dev(&d, p.flat.devs + e.x);
-        if constexpr (PH == FB_BIN) copy_shared(&r, p.regions + e.x);
-        __syncthreads();
-        const int bx = e.y * NB + (int)(blockIdx.x % NB), gx = e.z * NB;
-        if constexpr (PH == FB_BIN) {
-            const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-            if (i < d.n) {
-                cell_bin_atom(d, i);
-                lambda_atom(d, r, i);   // of the folded position
-            }
-        } else if constexpr (PH == FB_SCAN) {
-            cell_scan_body(d);
-        } else if constexpr (PH == FB_FILL) {
-            cell_fill_body(d, bx, gx);
-        } else if constexpr (PH == FB_ROWS) {
-            neigh_build_body<fb_threads(FB_ROWS) / 32>(d, bx, gx, pow2_cap(d.cap), reinterpret_cast<int*>(front_smem));
-        } else {
-            neigh_rev_body(d, bx, gx);
+        front_batch_lists(p, e, d);
+    } else if constexpr (PH == FB_BIN) {
+        const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
+        if (i < d.n) {
+            cell_bin_atom(d, i);
+            lambda_atom(d, r, i);   // of the folded position
         }
+    } else if constexpr (PH == FB_SCAN) {
+        cell_scan_body(d);
+    } else if constexpr (PH == FB_FILL) {
+        cell_fill_body(d, bx, gx);
+    } else if constexpr (PH == FB_ROWS) {
+        neigh_build_body<fb_threads(FB_ROWS) / 32>(d, bx, gx, pow2_cap(d.cap), reinterpret_cast<int*>(front_smem));
+    } else {
+        neigh_rev_body(d, bx, gx);
     }
 }
 
@@ -645,32 +556,22 @@ cudaError_t launch_front(const Dev& d, const Regions& r, const SeedRule& sr, cud
     return cudaLaunchCooperativeKernel((const void*)k_front, dim3(grid), dim3(FRONT_THREADS), args, smem, s);
 }
 
-// kernels of a batch's front: one up to an entry an SM, where launches count.  24
-// silicon cells (some 312 entries): three steps 832 us with one, 818 with eight.
-int front_batch_kernels(const BatchPlan& p) { return p.nblk[BT_FRONT] > sm_count() ? 8 : 1; }
+int front_batch_kernels() { return FB_COUNT; }
 
 cudaError_t launch_front_batch(const BatchPlan& p, cudaStream_t s, int integrate, double dt) {
-    static_assert(FRONT_ATOMS == FRONT_THREADS, "an entry's atoms are a CTA's threads");
-    FrontBatch f{p, integrate, dt};
-    const size_t smem = (size_t)FRONT_WARPS * p.capp2 * sizeof(int);
-    const int lim = front_resident((const void*)kb_front, smem);
-    if (lim < 1) return cudaErrorInvalidConfiguration;
-    if (front_batch_kernels(p) > 1) {
-        const int nent = p.nblk[BT_FRONT];
-        const size_t rows = (size_t)(fb_threads(FB_ROWS) / 32) * p.capp2 * sizeof(int);
-        cudaError_t e = launch_front_phase<FB_DISP>(f, nent, 0, s);
-        if (e == cudaSuccess) e = launch_front_phase<FB_BIN>(f, nent, 0, s);
-        if (e == cudaSuccess) e = launch_front_phase<FB_SCAN>(f, p.flat.nsys, 0, s);
-        if (e == cudaSuccess) e = launch_front_phase<FB_FILL>(f, nent, 0, s);
-        if (e == cudaSuccess) e = launch_front_phase<FB_ROWS>(f, nent, rows, s);
-        if (e == cudaSuccess) e = launch_front_phase<FB_REV>(f, nent, 0, s);
-        if (e == cudaSuccess) e = launch_front_phase<FB_BUFFER>(f, nent, 0, s);
-        if (e == cudaSuccess) e = launch_front_phase<FB_LISTS>(f, nent, 0, s);
-        return e;
-    }
-    const int grid = std::max(1, std::min(lim, std::max(p.nblk[BT_FRONT], p.flat.nsys)));
-    void* args[] = {&f};
-    return cudaLaunchCooperativeKernel((const void*)kb_front, dim3(grid), dim3(FRONT_THREADS), args, smem, s);
+    static_assert(FRONT_ATOMS == FRONT_THREADS, "an entry's atoms are a block's threads");
+    const FrontBatch f{p, integrate, dt};
+    const int nent = p.nblk[BT_FRONT];
+    const size_t rows = (size_t)(fb_threads(FB_ROWS) / 32) * p.capp2 * sizeof(int);
+    cudaError_t e = launch_front_phase<FB_DISP>(f, nent, 0, s);
+    if (e == cudaSuccess) e = launch_front_phase<FB_BIN>(f, nent, 0, s);
+    if (e == cudaSuccess) e = launch_front_phase<FB_SCAN>(f, p.flat.nsys, 0, s);
+    if (e == cudaSuccess) e = launch_front_phase<FB_FILL>(f, nent, 0, s);
+    if (e == cudaSuccess) e = launch_front_phase<FB_ROWS>(f, nent, rows, s);
+    if (e == cudaSuccess) e = launch_front_phase<FB_REV>(f, nent, 0, s);
+    if (e == cudaSuccess) e = launch_front_phase<FB_BUFFER>(f, nent, 0, s);
+    if (e == cudaSuccess) e = launch_front_phase<FB_LISTS>(f, nent, 0, s);
+    return e;
 }
 
 cudaError_t launch_front_lists(const Dev& d, const double4* x_in, cudaStream_t s) {

@@ -395,7 +395,7 @@ template <typename T, int LPA>
 __global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 3) kb_spline(const Dev* __restrict__ devs,
                                                            const SplTab<T>* __restrict__ tabs,
                                                            const int2* __restrict__ list, const int* count_p,
-                                                           const int* words, int uniform) {
+                                                           int uniform) {
     constexpr int G = 32 / LPA;
     constexpr int NB = spl_nb<LPA>();
     using V = typename Vec4<T>::type;
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(SPL_WARPS * 32, sizeof(T) == 4 ? 6 : 3) kb_spl
     if (uniform) spl_stage<T>(c3s, tabs[0].c3w, tabs[0].c2w);
     spl_fill_tq<LPA == 16 ? NB3MAX : NB>(tq);
     __syncthreads();
-    const int count = list_ok(words) ? *count_p : 0;
+    const int count = *count_p;
     const int stride = gridDim.x * SPL_WARPS * G;
     int g = (blockIdx.x * SPL_WARPS + warp) * G + grp;
     int2 e = g < count ? list[g] : make_int2(0, 0);
@@ -476,19 +476,19 @@ cudaError_t spline_batch_configure(int precision, int lpa, size_t* smem, int* gr
 
 template <typename T>
 static void spl_batch_launch(int lpa, const Dev* devs, const SplTab<T>* t, const int2* list, const int* count,
-                             const int* words, int uniform, size_t smem, int grid, cudaStream_t s) {
-    if (lpa == 8) kb_spline<T, 8><<<grid, SPL_WARPS * 32, smem, s>>>(devs, t, list, count, words, uniform);
-    else if (lpa == 16) kb_spline<T, 16><<<grid, SPL_WARPS * 32, smem, s>>>(devs, t, list, count, words, uniform);
-    else kb_spline<T, 32><<<grid, SPL_WARPS * 32, smem, s>>>(devs, t, list, count, words, uniform);
+                             int uniform, size_t smem, int grid, cudaStream_t s) {
+    if (lpa == 8) kb_spline<T, 8><<<grid, SPL_WARPS * 32, smem, s>>>(devs, t, list, count, uniform);
+    else if (lpa == 16) kb_spline<T, 16><<<grid, SPL_WARPS * 32, smem, s>>>(devs, t, list, count, uniform);
+    else kb_spline<T, 32><<<grid, SPL_WARPS * 32, smem, s>>>(devs, t, list, count, uniform);
 }
 
 void launch_spline_batch(int precision, int lpa, const Dev* devs, const void* tabs, const int2* list,
-                         const int* count, const int* words, int uniform, size_t smem, int grid, cudaStream_t s) {
+                         const int* count, int uniform, size_t smem, int grid, cudaStream_t s) {
     if (precision == MIX_FP64)
-        spl_batch_launch<double>(lpa, devs, static_cast<const SplTab<double>*>(tabs), list, count, words, uniform, smem,
+        spl_batch_launch<double>(lpa, devs, static_cast<const SplTab<double>*>(tabs), list, count, uniform, smem,
                                  grid, s);
     else
-        spl_batch_launch<float>(lpa, devs, static_cast<const SplTab<float>*>(tabs), list, count, words, uniform, smem,
+        spl_batch_launch<float>(lpa, devs, static_cast<const SplTab<float>*>(tabs), list, count, uniform, smem,
                                 grid, s);
 }
 

@@ -1856,7 +1856,7 @@ int fused_build(mix_batch* b, double dt) {
     };
     const size_t o_devs = take(ns * sizeof(Dev)), o_regs = take(ns * sizeof(Regions)), o_ace = take(ns * tsz),
                  o_spl = take(ns * ssz), o_eg = take(ns * 4), o_el = take(ns * 4), o_eb = take(ng * 4),
-                 o_cnt = take((ng + 1) * 4), o_hk = take(ns * sizeof(double)), o_words = take(SW_COUNT * 4),
+                 o_cnt = take((ng + 1) * 4), o_hk = take(ns * sizeof(double)), o_any = take(4),
                  o_le = take(tot * sizeof(int2)), o_lc = take(tot * sizeof(int2));
     size_t o_tab[BT_COUNT];
     for (int k = 0; k < BT_COUNT; ++k) o_tab[k] = take(tabs[k].size() * sizeof(int4));
@@ -1903,11 +1903,9 @@ int fused_build(mix_batch* b, double dt) {
     }
     P.regions = reinterpret_cast<const Regions*>(base + o_regs);
     P.gather_atoms = ga;
-    P.grid_polls = devs[0].grid_polls;
-    for (const Dev& d : devs) P.grid_polls = std::min(P.grid_polls, d.grid_polls);
     P.capp2 = capp2;
     P.hk = reinterpret_cast<const double*>(base + o_hk);
-    P.words = reinterpret_cast<int*>(base + o_words);   // zero, as the whole upload's gaps are
+    P.any = reinterpret_cast<int*>(base + o_any);   // zero, as the whole upload's gaps are
     FlatArgs& F = P.flat;
     F.devs = b->ddevs;
     F.nsys = ns;
@@ -1946,7 +1944,7 @@ int fused_build(mix_batch* b, double dt) {
 }
 
 int fused_launches(const mix_batch* b) {   // front, cheap, gather
-    return 2 + front_batch_kernels(b->plan) + (int)b->groups.size();
+    return 2 + front_batch_kernels() + (int)b->groups.size();
 }
 
 // one fused step (or force evaluation) captured on the batch's private stream
@@ -1970,11 +1968,11 @@ int fused_graph(mix_batch* b, int integrate, double dt, cudaGraph_t* graph, cuda
     cudaEventRecord(b->ev_fork, s);
     cudaStreamWaitEvent(b->aux, b->ev_fork, 0);
     launch_spline_batch(b->precision, b->spl_lpa, b->ddevs, b->dspl, P.flat.list_c, P.flat.counts + b->groups.size(),
-                        P.words, b->spl_uniform, b->spl_smem, b->spl_grid, b->aux);
+                        b->spl_uniform, b->spl_smem, b->spl_grid, b->aux);
     cudaEventRecord(b->ev_join, b->aux);
     for (size_t g = 0; g < b->groups.size(); ++g) {
         const mix_batch::Group& G = b->groups[g];
-        launch_ace_batch(b->precision, b->ddevs, b->dace, P.flat.list_e + G.base, P.flat.counts + g, P.words, G.n, G.L, G.smem,
+        launch_ace_batch(b->precision, b->ddevs, b->dace, P.flat.list_e + G.base, P.flat.counts + g, G.n, G.L, G.smem,
                          G.grid, s);
     }
     cudaStreamWaitEvent(s, b->ev_join, 0);

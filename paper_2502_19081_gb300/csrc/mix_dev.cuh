@@ -40,7 +40,6 @@ enum StatusWord : int {
     SW_GRID_COUNT = 32, // arrivals at the grid barriers of the running front kernel (0 between launches;
                         // a 128-byte line of its own)
     SW_GRID_DONE = 16,  // CTAs of the front kernel that have left (0 between launches)
-    SW_ANY = 1,         // batch plan words: some system rebuilds its lists in this step (word 0: status bits)
     SW_COUNT = 64,
 };
 

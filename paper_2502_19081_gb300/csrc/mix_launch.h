@@ -74,23 +74,22 @@ struct BatchPlan {
     int nblk[BT_COUNT];
     const Regions* regions;   // [nsys]
     const double* hk;         // [nsys] half-kick factors of the plan's time step
-    int* words;               // [SW_COUNT] status bits, grid barrier and rebuild flag of the front
+    int* any;                 // set while some system rebuilds its lists in this step
     int gather_atoms;         // GB_ATOMS or GB_ATOMS_BIG
-    int grid_polls;           // the smallest of the members' Dev::grid_polls
     int capp2;                // largest power-of-two list capacity (build scratch)
     FlatArgs flat;
 };
 
-// displacement, lists, weights, sets and their flattened lists of every system in
-// one cooperative launch, or, in large batches, a kernel a phase (k_front.cu)
-int front_batch_kernels(const BatchPlan& p);
+// displacement, lists, weights, sets and their flattened lists of every system, a
+// kernel a phase (k_front.cu)
+int front_batch_kernels();
 cudaError_t launch_front_batch(const BatchPlan& p, cudaStream_t s, int integrate, double dt);
 cudaError_t ace_batch_configure(int precision, int L, int n, int cap, int tile_max, int qb, size_t* smem, int* grid);
 void launch_ace_batch(int precision, const Dev* devs, const void* tabs, const int2* list, const int* count,
-                      const int* words, int n, int L, size_t smem, int grid, cudaStream_t s);
+                      int n, int L, size_t smem, int grid, cudaStream_t s);
 cudaError_t spline_batch_configure(int precision, int lpa, size_t* smem, int* grid);
 void launch_spline_batch(int precision, int lpa, const Dev* devs, const void* tabs, const int2* list,
-                         const int* count, const int* words, int uniform, size_t smem, int grid, cudaStream_t s);
+                         const int* count, int uniform, size_t smem, int grid, cudaStream_t s);
 void launch_gather_batch(const BatchPlan& p, int precision, int integrate, cudaStream_t s);
 
 int sm_count();
