@@ -361,7 +361,7 @@ __device__ __forceinline__ void front_batch_disp(const FrontBatch& f, const int4
         d.status[SW_NEXP] = 0;
         d.status[SW_NCHEAP] = 0;
     }
-    if (i < d.n) {
+    if (list_ok(d) && i < d.n) {
         if (disp_atom(d, i, f.integrate, f.dt, f.p.hk[e.x], 0)) *f.p.any = 1;
         lambda_atom(d, r, i);   // stands unless the lists are rebuilt
     }
@@ -370,9 +370,10 @@ __device__ __forceinline__ void front_batch_disp(const FrontBatch& f, const int4
 // buffers; a warp's 32 atoms are its own, so it counts them at once
 __device__ __forceinline__ void front_batch_buffer(const BatchPlan& p, const int4& e, const Dev& d) {
     const int lane = threadIdx.x & 31;
-    buffer_dispatch(d, e.y, e.z, 32);
+    const bool ok = list_ok(d);
+    if (ok) buffer_dispatch(d, e.y, e.z, 32);
     const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-    const bool in = i < d.n;
+    const bool in = ok && i < d.n;
     const int fl = in ? d.flags[i] : 0;
     const double lam = in ? d.lam[i] : 0.0;
     const int2 own = block_sum2((fl >> 2) & 1, (fl >> 3) & 1);
@@ -381,7 +382,7 @@ __device__ __forceinline__ void front_batch_buffer(const BatchPlan& p, const int
         d.blk_c[e.y] = own.y;
         if (own.x) atomicAdd(d.status + SW_NEXP, own.x);
         if (own.y) atomicAdd(d.status + SW_NCHEAP, own.y);
-        if (e.y == 0 && d.status[SW_REBUILD]) {
+        if (ok && e.y == 0 && d.status[SW_REBUILD]) {
             d.status[SW_REBUILDS] += 1;
             d.status[SW_REBUILD] = 0;
         }
@@ -416,7 +417,7 @@ __device__ __forceinline__ void front_batch_lists(const BatchPlan& p, const int4
     }
     const int2 before = block_sum2(se, sc), flat = block_sum2(oe, oc);
     const int64_t i = (int64_t)e.y * FRONT_ATOMS + threadIdx.x;
-    const bool in = i < d.n;
+    const bool in = list_ok(d) && i < d.n;
     const int fl = in ? d.flags[i] : 0;
     const int ie = (fl >> 2) & 1, ic = (fl >> 3) & 1;
     int2 tot;
@@ -442,6 +443,9 @@ __device__ __forceinline__ void front_batch_lists(const BatchPlan& p, const int4
     }
 }
 
+// A member whose own front gave up at a barrier before it was stepped with the batch
+// (list_ok) may have half-written lists: it takes no part, with empty sets, until it
+// is bound again.  No kernel of a batch sets that bit, so a block reads one value.
 template <int PH>
 __global__ void __launch_bounds__(fb_threads(PH), PH == FB_ROWS ? 8 : (PH == FB_REV ? 1 : 2))
     kb_front_phase(const __grid_constant__ FrontBatch f) {
@@ -456,6 +460,7 @@ __global__ void __launch_bounds__(fb_threads(PH), PH == FB_ROWS ? 8 : (PH == FB_
     int4 e = make_int4(blockIdx.x, 0, 1, 0);
     if constexpr (PH != FB_SCAN) e = p.ba[BT_FRONT].tab[blockIdx.x / NB];
     if (LISTS && !p.flat.devs[e.x].status[SW_REBUILD]) return;   // the whole block
+    if (LISTS && !list_ok(p.flat.devs[e.x].status)) return;
     load_dev(&d, p.flat.devs + e.x);
     if constexpr (PH == FB_DISP || PH == FB_BIN) copy_shared(&r, p.regions + e.x);
     __syncthreads();

@@ -136,3 +136,41 @@ def test_tile_wait_in_a_batch_is_said_for_every_member_it_cost(mx):
             continue
         assert k > 0 and np.array_equal(c.get_state()[2], a.get_state()[2])
     b.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_member_whose_front_gave_up_takes_no_part_in_a_batch(mx, prec):
+    """One member gives up alone, unnoticed, and is then stepped with the others: it
+    does not move and is reported; the others go as they go alone."""
+    import torch
+    pots = I.serve_potentials()
+    wls = [I.serve_request(60 + k, "Si", 900 + 700 * k, 0.2, 1200.0, pots) for k in range(3)]
+    members = [mx.open_context(wl, precision=prec) for wl in wls]
+    state = [c.get_state() for c in members]
+    b = mx.Batch(members)
+    b.set_fused(True)
+    members[1].set_wait_limits(grid_polls=0)
+    members[1].set_state(*state[1][:2])
+    members[1].step(1.0, 1)                 # a first list build that is given up
+    members[1].set_wait_limits()
+    torch.cuda.synchronize()
+    x1 = members[1].x.clone()
+    b.step(1.0, 25)
+    _gives_up(mx, b.sync)
+    assert b.info()["fused"] and torch.equal(members[1].x, x1)
+    for k in (0, 2):
+        a = mx.open_context(wls[k], precision=prec)
+        a.step(1.0, 25)
+        assert a.stats()["rebuilds"] > 1
+        for u, w in zip(members[k].get_state()[:3], a.get_state()[:3]):
+            assert np.array_equal(u, w)
+    # bound again, it is a member like the others
+    for c, s in zip(members, state):
+        c.bind()
+        c.set_state(*s[:2])
+    b.step(1.0, 5)
+    b.sync()
+    a = mx.open_context(wls[1], precision=prec)
+    a.step(1.0, 5)
+    assert np.array_equal(members[1].get_state()[2], a.get_state()[2])
+    b.close()
