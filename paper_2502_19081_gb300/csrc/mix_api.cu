@@ -728,13 +728,18 @@ int evals_launches(const mix_ctx*) { return LAUNCHES_PER_EVAL; }
 
 // the kernels of one evaluation, in order, on stream s (events between the
 // phases when profiling)
-// (captured = true: the events become record nodes of the graph being captured)
-void enqueue_evaluation(mix_ctx* c, cudaStream_t s, int integrate, double dt, int force_rebuild, bool prof,
+// (captured = true: the events become record nodes of the graph being captured).
+// Returns the front's launch error; nothing is enqueued behind a front that was not launched.
+cudaError_t enqueue_evaluation(mix_ctx* c, cudaStream_t s, int integrate, double dt, int force_rebuild, bool prof,
                         bool captured = false) {
     const double h = half_kick(dt, c->sys.mass);
     const unsigned ef = captured ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (prof) cudaEventRecordWithFlags(c->ev[0], s, ef);
-    launch_front(c->dev, c->regions, c->seedrule, s, integrate, dt, h, force_rebuild);
+    const cudaError_t ef_front = launch_front(c->dev, c->regions, c->seedrule, s, integrate, dt, h, force_rebuild);
+    if (ef_front != cudaSuccess) {
+        cudaGetLastError();   // the caller reports it
+        return ef_front;
+    }
     // one kernel: its time is the first phase's, the list and set phases are empty
     if (prof) cudaEventRecordWithFlags(c->ev[1], s, ef);
     if (prof) cudaEventRecordWithFlags(c->ev[2], s, ef);
@@ -769,6 +774,23 @@ void enqueue_evaluation(mix_ctx* c, cudaStream_t s, int integrate, double dt, in
     }
     launch_gather(c->dev, c->precision, integrate, h, s);
     if (prof) cudaEventRecordWithFlags(c->ev[6], s, ef);
+    return cudaSuccess;
+}
+
+// enqueue_evaluation captured on the context's private stream into *g; on an error
+// there is no graph
+cudaError_t capture_evaluation(mix_ctx* c, int integrate, double dt, bool prof, cudaGraph_t* g) {
+    *g = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!c->cap_stream) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    const cudaError_t ef = enqueue_evaluation(c, c->cap_stream, integrate, dt, 0, prof, true);
+    e = cudaStreamEndCapture(c->cap_stream, g);
+    if (ef == cudaSuccess) return e;
+    if (e == cudaSuccess) cudaGraphDestroy(*g);
+    *g = nullptr;
+    return ef;
 }
 
 void drop_graph(mix_ctx* c) {
@@ -783,16 +805,9 @@ void drop_graph(mix_ctx* c) {
 // cudaGraphLaunch on the context stream.
 int capture_step(mix_ctx* c, double dt) {
     drop_graph(c);
-    if (!c->cap_stream) {
-        cudaError_t e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return cuda_fail(c, e, "capture stream");
-    }
-    cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamBeginCapture");
-    enqueue_evaluation(c, c->cap_stream, 1, dt, 0, c->profiling, true);
     cudaGraph_t g = nullptr;
-    e = cudaStreamEndCapture(c->cap_stream, &g);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamEndCapture");
+    cudaError_t e = capture_evaluation(c, 1, dt, c->profiling, &g);
+    if (e != cudaSuccess) return cuda_fail(c, e, "step capture");
     c->graph = g;
     e = cudaGraphInstantiate(&c->gexec, g, 0);
     if (e != cudaSuccess) {
@@ -818,7 +833,8 @@ int evaluate(mix_ctx* c, int integrate, double dt) {
         cudaError_t e = cudaGraphLaunch(c->gexec, s);
         if (e != cudaSuccess) return cuda_fail(c, e, "cudaGraphLaunch");
     } else {
-        enqueue_evaluation(c, s, integrate, dt, c->need_build ? 1 : 0, prof);
+        cudaError_t e = enqueue_evaluation(c, s, integrate, dt, c->need_build ? 1 : 0, prof);
+        if (e != cudaSuccess) return cuda_fail(c, e, "front launch");
     }
     c->need_build = false;
     c->launches += evals_launches(c);
@@ -1494,16 +1510,9 @@ namespace {
 // graph replays and launches on streams).
 int capture_eval(mix_ctx* c, cudaGraphExec_t* out) {
     *out = nullptr;
-    if (!c->cap_stream) {
-        cudaError_t e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return cuda_fail(c, e, "capture stream");
-    }
-    cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamBeginCapture");
-    enqueue_evaluation(c, c->cap_stream, 0, 0.0, 0, false, true);
     cudaGraph_t g = nullptr;
-    e = cudaStreamEndCapture(c->cap_stream, &g);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamEndCapture");
+    cudaError_t e = capture_evaluation(c, 0, 0.0, false, &g);
+    if (e != cudaSuccess) return cuda_fail(c, e, "evaluation capture");
     e = cudaGraphInstantiate(out, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
@@ -1538,10 +1547,10 @@ int time_force_evals(mix_ctx* c, int reps, float* ms) {
     std::vector<float> v;
     for (int r = 0; r < reps; ++r) {
         cudaEventRecord(e0, c->stream);
-        if (gx) cudaGraphLaunch(gx, c->stream);
-        else enqueue_evaluation(c, c->stream, 0, 0.0, 0, false);
+        cudaError_t e = gx ? cudaGraphLaunch(gx, c->stream) : enqueue_evaluation(c, c->stream, 0, 0.0, 0, false);
         cudaEventRecord(e1, c->stream);
-        cudaError_t e = cudaEventSynchronize(e1);
+        const cudaError_t es = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = es;
         if (e != cudaSuccess) {
             cudaEventDestroy(e0);
             cudaEventDestroy(e1);
@@ -1672,16 +1681,8 @@ int seed_restore(mix_ctx* c, const SeedSave& s) {
 
 // one member evaluation captured into a (not instantiated) graph
 int member_graph(mix_ctx* c, int integrate, double dt, cudaGraph_t* g) {
-    if (!c->cap_stream) {
-        cudaError_t e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return cuda_fail(c, e, "capture stream");
-    }
-    cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamBeginCapture");
-    enqueue_evaluation(c, c->cap_stream, integrate, dt, 0, false, true);
-    e = cudaStreamEndCapture(c->cap_stream, g);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamEndCapture");
-    return MIX_OK;
+    const cudaError_t e = capture_evaluation(c, integrate, dt, false, g);
+    return e == cudaSuccess ? MIX_OK : cuda_fail(c, e, "evaluation capture");
 }
 
 }  // namespace
