@@ -31,12 +31,6 @@ constexpr int FRONT_CTAS = 2;   // resident CTAs an SM the kernel is compiled fo
 // and crossing the grid once more.
 constexpr int FRONT_REDUNDANT = 32768;
 constexpr int FRONT_REDUNDANT_CELLS = 8192;
-// Cells from which a CTA builds the lists a cell at a time (candidates staged in
-// shared memory) rather than a warp an atom: with few cells the CTAs run out of
-// them (bcc iron, build and its barrier: 729 cells 45 against 41 us, 1,000 cells
-// 61 against 65 us, 200,000
-// atoms 442 against 480 us).
-constexpr int FRONT_TILED_CELLS = 1000;
 struct FrontOpt {
     int integrate, force_rebuild;
     double dt, h;
@@ -519,10 +513,25 @@ int lists_resident(size_t smem) {
     return n;
 }
 
+// Lists a cell at a time (candidates staged in shared memory, a team of warps a
+// cell) or an atom at a time: the first where the cells fill the resident teams,
+// the waves of cells at least three quarters full on the whole or more than four.  Some
+// cells more than a wave leave most teams idle for its length.  Front of an
+// evaluation that rebuilds, us, a cell / an atom at a time, 1,216 teams: iron, 343
+// cells 111 / 80, 729 121 / 116, 1,000 122 / 129, 1,331 151 / 130, 1,584 166 / 165, 2,744
+// 223 / 230; silicon,
+// 512 cells 51 / 47, 1,000 55 / 56, 1,728 69 / 67, 2,548 82 / 82, 4,096 98 / 102.
+bool front_tiled(const Dev& d) {
+    if (!nb_tiled_ok(d)) return false;
+    const int64_t teams = (int64_t)sm_count() * FRONT_CTAS * (FRONT_WARPS / NB_TEAM);
+    const int64_t waves = (d.cells.ncell + teams - 1) / teams;
+    return waves > 4 || 4 * (int64_t)d.cells.ncell >= 3 * waves * teams;
+}
+
 size_t front_shape(const Dev& d, FrontOpt& o) {
     o.capp2 = 32;
     while (o.capp2 < d.cap) o.capp2 <<= 1;
-    o.tiled = d.cells.ncell >= FRONT_TILED_CELLS && nb_tiled_ok(d) ? 1 : 0;
+    o.tiled = front_tiled(d) ? 1 : 0;
     return o.tiled ? nb_tiled_smem(o.capp2, FRONT_WARPS) : (size_t)FRONT_WARPS * o.capp2 * sizeof(int);
 }
 

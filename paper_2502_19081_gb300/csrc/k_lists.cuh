@@ -310,11 +310,16 @@ __device__ __forceinline__ void neigh_build_body(const Dev& d, int bx, int gx, i
 }
 
 // The list build of a single context with neighbour-cell tiles staged in shared
-// memory: a CTA takes a cell at a time, copies the candidates of its 27-cell
-// stencil (atom index and float position, in run order) into shared memory
+// memory: a team of NB_TEAM warps takes a cell at a time, copies the candidates of its
+// 27-cell stencil (float position and atom index, in run order) into shared memory
 // once, and its warps take the cell's atoms, a warp per atom, testing 32
 // staged candidates at a time; the candidates cross L2 once per cell instead
-// of once per atom.  The staged positions are taken relative to the cell's centre,
+// of once per atom.  A CTA of 16 warps is four teams that do not wait for each
+// other: a cell holds some 8 atoms in silicon and 17 in iron, so 16 warps on one cell
+// left half of them idle (evaluations that rebuild, front, us, 16 warps a cell / 8 / 4 /
+// 2: 20,383 silicon atoms 92 / 82 / 81 / 95, 499,199 of them 1247 / 899 / 802 / 1090, 50,459
+// iron atoms 234 / 214 / 223 / 294, 198,903 of them 691 / 628 / 613 / 840, 998,559 of them
+// 3606 / 3046 / 2935 / 4087).  The staged positions are taken relative to the cell's centre,
 // each as the periodic image next to it, so that the test of a pair is a
 // difference and three products (a periodic dimension has at least four cells
 // here, nb_tiled_ok, each at least as wide as the list radius: the stencil lies
@@ -325,6 +330,7 @@ __device__ __forceinline__ void neigh_build_body(const Dev& d, int bx, int gx, i
 // the warp-per-atom build (neigh_build_body).  A stencil with more than NB_TILE
 // candidates (a dense spot) is tested from global memory instead.
 constexpr int NB_TILE = 1024;
+constexpr int NB_TEAM = 4;
 
 inline bool nb_tiled_ok(const Dev& d) {
     for (int k = 0; k < 3; ++k)
@@ -333,26 +339,32 @@ inline bool nb_tiled_ok(const Dev& d) {
 }
 
 inline size_t nb_tiled_smem(int capp2, int warps) {
-    return (size_t)NB_TILE * (sizeof(float4) + sizeof(int)) + (size_t)warps * capp2 * sizeof(int);
+    return (size_t)NB_TILE * (warps / NB_TEAM) * sizeof(float4) + (size_t)warps * capp2 * sizeof(int);
+}
+
+// barrier of one team (the CTA's barrier is number 0)
+__device__ __forceinline__ void nb_team_sync(int team) {
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(NB_TEAM * 32) : "memory");
 }
 
 template <int NBW>
 __device__ __forceinline__ void neigh_build_tiled_body(const Dev& d, int bx, int gx, int capp2, unsigned char* nb_smem) {
-    float4* tpos = reinterpret_cast<float4*>(nb_smem);
-    int* tidx = reinterpret_cast<int*>(tpos + NB_TILE);
-    int* sbuf = tidx + NB_TILE;
-    __shared__ int s_runx[NB_RUNS], s_runi[NB_RUNS];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int* buf = sbuf + warp * capp2;
+    constexpr int NT = NBW / NB_TEAM;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, team = warp / NB_TEAM, tw = warp % NB_TEAM;
+    float4* tile = reinterpret_cast<float4*>(nb_smem) + team * NB_TILE;   // position, atom index in w
+    int* buf = reinterpret_cast<int*>(reinterpret_cast<float4*>(nb_smem) + NT * NB_TILE) + warp * capp2;
+    __shared__ int s_runx[NT][NB_RUNS], s_runi[NT][NB_RUNS];
+    int* runx = s_runx[team];
+    int* runi = s_runi[team];
     const unsigned lt = (1u << lane) - 1u;
     const int ncx = d.cells.nc[0], ncy = d.cells.nc[1];
     const int ncell = d.cells.ncell;
     int most = 0;
-    for (int c = bx; c < ncell; c += gx) {
+    for (int c = bx * NT + team; c < ncell; c += gx * NT) {
         const int a0 = d.cell_start[c], a1 = d.cell_start[c + 1];
-        if (a0 == a1) continue;   // the same for the whole CTA
+        if (a0 == a1) continue;   // the same for the whole team
         const int cx = c % ncx, cy = (c / ncx) % ncy, cz = c / (ncx * ncy);
-        if (warp == 0) {
+        if (tw == 0) {
             int t0, len;
             nb_run(d, cx, cy, cz, lane, t0, len);
             int inc = len;
@@ -362,8 +374,8 @@ __device__ __forceinline__ void neigh_build_tiled_body(const Dev& d, int bx, int
                 if (lane >= o) inc += v;
             }
             if (lane < NB_RUNS) {
-                s_runi[lane] = inc;
-                s_runx[lane] = t0 - (inc - len);
+                runi[lane] = inc;
+                runx[lane] = t0 - (inc - len);
             }
         }
         // the cell's centre, and a position as its periodic image next to it
@@ -376,20 +388,21 @@ __device__ __forceinline__ void neigh_build_tiled_body(const Dev& d, int bx, int
                 if (d.box.per[k]) v[k] -= d.nbs.L[k] * rintf(v[k] * d.nbs.iL[k]);
             return make_float4(v[0], v[1], v[2], 0.f);
         };
-        __syncthreads();
-        const int total = s_runi[NB_RUNS - 1];
+        nb_team_sync(team);
+        const int total = runi[NB_RUNS - 1];
         const bool staged = total <= NB_TILE;
         if (staged) {
-            for (int t = threadIdx.x; t < total; t += blockDim.x) {
-                int r = 0;
-                while (t >= s_runi[r]) ++r;
-                const int j = d.cell_atoms[s_runx[r] + t];
-                tidx[t] = j;
-                tpos[t] = relative(d.xf[j]);
+            int r = 0;
+            for (int t = tw * 32 + lane; t < total; t += NB_TEAM * 32) {
+                while (t >= runi[r]) ++r;
+                const int j = d.cell_atoms[runx[r] + t];
+                float4 v = relative(d.xf[j]);
+                v.w = __int_as_float(j);
+                tile[t] = v;
             }
         }
-        __syncthreads();
-        for (int a = a0 + warp; a < a1; a += NBW) {
+        nb_team_sync(team);
+        for (int a = a0 + tw; a < a1; a += NB_TEAM) {
             const int i = d.cell_atoms[a];
             const double4 xi = d.x[i];
             const float4 xif = d.xf[i];
@@ -401,8 +414,8 @@ __device__ __forceinline__ void neigh_build_tiled_body(const Dev& d, int bx, int
                 int j = -1;
                 if (u < total) {
                     if (staged) {
-                        j = tidx[u];
-                        const float4 rj = tpos[u];
+                        const float4 rj = tile[u];
+                        j = __float_as_int(rj.w);
                         const float dx = rj.x - ri.x, dy = rj.y - ri.y, dz = rj.z - ri.z;
                         const float r2f = dx * dx + dy * dy + dz * dz;
                         ok = r2f < d.nbs.lo2;
@@ -413,8 +426,8 @@ __device__ __forceinline__ void neigh_build_tiled_body(const Dev& d, int bx, int
                         }
                         ok = ok && j != i;
                     } else {
-                        while (u >= s_runi[r]) ++r;
-                        j = d.cell_atoms[s_runx[r] + u];
+                        while (u >= runi[r]) ++r;
+                        j = d.cell_atoms[runx[r] + u];
                         if (j != i) ok = nb_accept(d, xi, xif, d.xf[j], j);
                     }
                 }
@@ -428,7 +441,7 @@ __device__ __forceinline__ void neigh_build_tiled_body(const Dev& d, int bx, int
             nb_write_row(d, i, xi, cnt, buf, lane);
             most = max(most, cnt);
         }
-        __syncthreads();   // the tile and the runs are rewritten for the next cell
+        nb_team_sync(team);   // the tile and the runs are rewritten for the next cell
     }
     nb_report_max(d, most, lane);
 }
