@@ -301,15 +301,18 @@ def errors_against(ctx_F, ctx_E, F_ref, E_ref, flags):
 
 def phase_bytes(name: str, n: int, nst: dict, rebuild_frac: float) -> float:
     """Algorithmic DRAM bytes per step of a memory-bound phase (atom-major
-    float64 rows of 32 B, int32 lists): disp, the one kernel in front of the
-    potentials, reads x, v, f and writes x, v, reads x and the list for the
-    weights and sets and writes weights and flags, and on rebuild steps reads x
-    and writes cell ids, nnb and the sorted rows and reverse slots (lists and
-    sets are empty phases); gather reads both potentials' own and incoming slot
-    rows (16 B a slot in float) and writes f, v."""
+    float64 rows of 32 B, int32 lists): disp reads x, v, f and writes x, v;
+    lists (rebuild steps only) read x and write cell ids, nnb and the sorted
+    rows and reverse slots; sets read x and the list and write weights and
+    flags; gather reads both potentials' own and incoming slot rows (16 B a
+    slot in float) and writes f, v."""
     nb = nst["nnb_list"]
     if name == "disp":
-        return n * (96.0 + 32.0 + 4.0 * nb + 9.0 + 4.0) + rebuild_frac * n * (32.0 + 4.0 + 4.0 + 8.0 * nb)
+        return n * 96.0
+    if name == "lists":
+        return rebuild_frac * n * (32.0 + 4.0 + 4.0 + 8.0 * nb)
+    if name == "sets":
+        return n * (32.0 + 4.0 * nb + 9.0 + 4.0)
     if name == "gather":
         return nst["n_exp"] * 2 * 16.0 * nst["nnb_exp_rc"] + nst["n_cheap"] * 2 * 16.0 * nst["nnb_cheap_rc"] + n * 72.0
     return 0.0

@@ -302,11 +302,12 @@ const char* mix_last_error(const mix_ctx* ctx);
 /* Measurement helpers.  The paper has no counterpart: they exist to time the  */
 /* kernels and to state roofline fractions.                                   */
 
-/* Kernel groups of one force evaluation, in launch order. */
-#define MIX_PHASE_DISP 0     /* first half-kick, drift, skin test; the lists when they are
-                                rebuilt; weights, buffers, compaction (one kernel) */
-#define MIX_PHASE_LISTS 1    /* empty: part of the kernel above */
-#define MIX_PHASE_SETS 2     /* empty: part of the kernel above */
+/* Parts of one force evaluation, in order.  The first three are one kernel, whose
+ * time is shared out by the clock of one of its blocks. */
+#define MIX_PHASE_DISP 0     /* first half-kick, drift, skin test (and the weights of the
+                                drifted positions) */
+#define MIX_PHASE_LISTS 1    /* cell list and neighbour list (0 unless rebuilding) */
+#define MIX_PHASE_SETS 2     /* buffers, compaction; seed-atom weights */
 #define MIX_PHASE_EXP 3      /* expensive potential (one kernel) */
 #define MIX_PHASE_CHEAP 4    /* cheap potential (one kernel) */
 #define MIX_PHASE_GATHER 5   /* gather, blend, second half-kick (one kernel) */

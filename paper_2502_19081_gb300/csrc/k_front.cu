@@ -35,6 +35,7 @@ struct FrontOpt {
     int integrate, force_rebuild;
     double dt, h;
     int capp2, tiled;
+    int prof;              // write SW_CLOCK
     const double4* x_in;   // lists alone (mix_neighbours_noalloc): positions to copy; else null
 };
 
@@ -267,6 +268,11 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front(Dev d, Regi
     Grid grid(d.status, d.grid_polls);
     const int bx = (int)blockIdx.x, gx = (int)gridDim.x;
     const bool g0 = bx == 0 && threadIdx.x == 0;
+    // a phase ends (k = 1: displacement, 2: lists, 3: sets) as this CTA sees it
+    auto stamp = [&](int k) {
+        if (o.prof && g0) reinterpret_cast<long long*>(d.status + SW_CLOCK)[k] = clock64();
+    };
+    stamp(0);
     if (g0) disp_reset(d, o.force_rebuild);
     // displacement, and the weights of the drifted positions at once: they stand
     // unless the lists are rebuilt (which folds the positions)
@@ -275,6 +281,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front(Dev d, Regi
         if (sr.mode == 0 && !o.force_rebuild) lambda_atom(d, r, i);
     });
     if (!grid.barrier()) return;
+    stamp(1);
     const bool rebuild = o.force_rebuild || ld_acquire(d.status + SW_REBUILD) != 0;
     if (rebuild) {
         if (!front_build(d, grid, o.capp2, o.tiled, front_smem)) return;
@@ -284,6 +291,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front(Dev d, Regi
             d.status[SW_REBUILDS] += 1;
             d.status[SW_REBUILD] = 0;
         }
+        stamp(2);
     }
     if (sr.mode != 0) {
         if (sr.mode == 2) {
@@ -297,7 +305,14 @@ __global__ void __launch_bounds__(FRONT_THREADS, FRONT_CTAS) k_front(Dev d, Regi
     }
     buffer_dispatch(d, bx, gx, apw);
     if (!grid.barrier()) return;
-    if (front_compact(d, grid)) grid.done();
+    if (front_compact(d, grid)) {
+        if (!rebuild && o.prof && g0) {   // no lists
+            const volatile long long* t = reinterpret_cast<const long long*>(d.status + SW_CLOCK);
+            reinterpret_cast<long long*>(d.status + SW_CLOCK)[2] = t[1];
+        }
+        stamp(3);
+        grid.done();
+    }
 }
 
 // lists alone: positions copied and checked, counts cleared, then the build
@@ -545,8 +560,9 @@ cudaError_t front_configure(Dev& d) {
 }
 
 cudaError_t launch_front(const Dev& d, const Regions& r, const SeedRule& sr, cudaStream_t s, int integrate, double dt,
-                         double h, int force_rebuild) {
+                         double h, int force_rebuild, bool prof) {
     FrontOpt o{};
+    o.prof = prof ? 1 : 0;
     o.integrate = integrate;
     o.force_rebuild = force_rebuild;
     o.dt = dt;

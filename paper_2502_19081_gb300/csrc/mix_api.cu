@@ -735,15 +735,13 @@ cudaError_t enqueue_evaluation(mix_ctx* c, cudaStream_t s, int integrate, double
     const double h = half_kick(dt, c->sys.mass);
     const unsigned ef = captured ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (prof) cudaEventRecordWithFlags(c->ev[0], s, ef);
-    const cudaError_t ef_front = launch_front(c->dev, c->regions, c->seedrule, s, integrate, dt, h, force_rebuild);
+    const cudaError_t ef_front = launch_front(c->dev, c->regions, c->seedrule, s, integrate, dt, h, force_rebuild, prof);
     if (ef_front != cudaSuccess) {
         cudaGetLastError();   // the caller reports it
         return ef_front;
     }
-    // one kernel: its time is the first phase's, the list and set phases are empty
-    if (prof) cudaEventRecordWithFlags(c->ev[1], s, ef);
-    if (prof) cudaEventRecordWithFlags(c->ev[2], s, ef);
-    if (prof) cudaEventRecordWithFlags(c->ev[3], s, ef);
+    // one kernel for the first three phases, divided by its own clock (evaluate)
+    if (prof) cudaEventRecordWithFlags(c->ev[MIX_PHASE_EXP], s, ef);
     const void* at = c->precision == MIX_FP64 ? (const void*)&c->ace64 : (const void*)&c->ace32;
     const void* st = c->precision == MIX_FP64 ? (const void*)&c->spl64 : (const void*)&c->spl32;
     auto exp_kernel = [&]() {
@@ -842,9 +840,17 @@ int evaluate(mix_ctx* c, int integrate, double dt) {
     if (rc || !prof) return rc;
     cudaError_t e = cudaEventSynchronize(c->ev[MIX_PHASES]);
     if (e != cudaSuccess) return cuda_fail(c, e, "profile event");
+    e = cudaMemcpyAsync(c->pinned + SW_CLOCK, c->dev.status + SW_CLOCK, 4 * sizeof(long long), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(c, e, "profile clock");
+    long long t[4];
+    std::memcpy(t, c->pinned + SW_CLOCK, sizeof t);
     for (int p = 0; p < MIX_PHASES; ++p) {
+        // the front's time from its events, shared out by the clock of one of its blocks
+        const bool front = p < MIX_PHASE_EXP;
         float ms = 0.f;
-        cudaEventElapsedTime(&ms, c->ev[p], c->ev[p + 1]);
+        cudaEventElapsedTime(&ms, c->ev[front ? 0 : p], c->ev[front ? MIX_PHASE_EXP : p + 1]);
+        if (front) ms = t[3] > t[0] ? (float)(ms * ((double)(t[p + 1] - t[p]) / (double)(t[3] - t[0]))) : 0.f;
         c->prof_last[p] = ms;
         c->prof_total[p] += ms;
     }

@@ -40,6 +40,8 @@ enum StatusWord : int {
     SW_GRID_COUNT = 32, // arrivals at the grid barriers of the running front kernel (0 between launches;
                         // a 128-byte line of its own)
     SW_GRID_DONE = 16,  // CTAs of the front kernel that have left (0 between launches)
+    SW_CLOCK = 18,      // 18..25, when profiling: SM clock of one CTA of the front at its start, behind the
+                        // displacement, behind the lists and at its end (64 bits each)
     SW_COUNT = 64,
 };
 

@@ -9,7 +9,7 @@ namespace mixd {
 // launch (k_front.cu).  front_configure fills d.grid_front_max.
 cudaError_t front_configure(Dev& d);
 cudaError_t launch_front(const Dev& d, const Regions& r, const SeedRule& sr, cudaStream_t s, int integrate, double dt,
-                         double h, int force_rebuild);
+                         double h, int force_rebuild, bool prof);
 // the lists alone, of the positions x_in (copied to d.x and folded there)
 cudaError_t launch_front_lists(const Dev& d, const double4* x_in, cudaStream_t s);
 
