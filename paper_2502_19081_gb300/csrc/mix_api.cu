@@ -1649,7 +1649,7 @@ void set_grid_divisor(mix_ctx* c, int div) {
     c->ace_grid = std::max(1, c->ace_grid_max / div);
     c->spl_grid = std::max(1, c->spl_grid_max / div);
     c->dev.grid_gather = std::max(1, sm_count() * 8 / div);
-    c->dev.grid_buffer = std::max(1, sm_count() * 8 / div);
+    c->dev.grid_buffer = std::max(1, c->dev.grid_front_max / div);
     drop_graph(c);
 }
 
