@@ -395,8 +395,8 @@ int mix_tc_selftest(const void* a_dev, const void* b_dev, int m, int n, int k, f
  * cheap kernel (a narrower group is tried only where the largest 3-body
  * neighbour count measured so far fills at most two thirds of its on-chip
  * slots; a later overflow reports MIX_EOVERFLOW and widens the groups again),
- * the persistent grid of each potential kernel and the grids of the gather and
- * of the kernel that forms the sets, and keeps the fastest (reported by mix_get_info); the
+ * the persistent grid of each potential kernel and the grid of the gather, and
+ * keeps the fastest (reported by mix_get_info); the
  * forces do not depend on any of them.
  * reps: timed evaluations per candidate (median). */
 int mix_tune(mix_ctx* ctx, int reps);

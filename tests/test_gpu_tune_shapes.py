@@ -36,3 +36,14 @@ def test_batch_divisor_divides_the_resident_front():
         assert a.stats()["rebuilds"] > 1
         assert np.array_equal(c.get_state()[0], a.get_state()[0])
     b.close()
+
+
+def test_tuned_alone_keeps_the_whole_front():
+    from paper_2502_19081_gb300 import mix
+    c = _members(mix, 1)[0]
+    b = mix.Batch([c])
+    b.tune(reps=1)
+    c.tune(reps=2)
+    assert c.info()["buffer_grid"] == 0
+    b.close()
+    c.close()
