@@ -368,6 +368,8 @@ struct mix_ctx {
     size_t ace_smem, spl_smem;
     int ace_grid, spl_grid;
     int ace_wn;                       // warps (atoms) a CTA of the CUDA-core expensive kernel
+    size_t ace_shape_smem[2];         // its launch shapes with ACE_GROUP and ACE_MAX_WARPS warps
+    int ace_shape_grid[2];
     int ace_tcm;                      // 0: CUDA-core nu = 3; 1, 2: tensor-core readout (bf16, bf16 hi/lo)
     int ace_nbuf;                     // tile buffers of the tensor-core kernel
     int spl_lpa;                      // lanes per atom of the cheap kernel (32, 16 or 8)
@@ -670,6 +672,45 @@ void fill_tabs(mix_ctx* c, unsigned char* base, AceTab<T>& at, SplTab<T>& st) {
     st.invhc = (T)(5.0 / (2.0 * c->spl_rc3));
     st.na = c->spl_na;
     st.pad = 0;
+}
+
+// Atoms of the CUDA-core expensive kernel's CTA.  4 warps share the coefficient tiles
+// between twice the atoms of 2, so more warps fit an SM where the tiles are large
+// (n = 12, lmax = 5: 16 against 12); 2 spread a set that fits one wave over more SMs.
+// The line is therefore one wave of CTAs of 2 (2 x ace_shape_grid[0] atoms: 1,824
+// for n = 12, lmax = 5, 2,432 for n = 10, lmax = 4), on the set's size as the regions
+// give it.  Expensive kernel, us, 2 / 4 warps, by evaluated atoms: n = 12: 1,012
+// 109 / 135, 1,242 133 / 136, 3,705 280 / 225, 13,004 773 / 676, 19,284 1122 / 1023; n = 10:
+// 1,012 73 / 73, 3,705 119 / 121, 13,004 346 / 342, 36,739 979 / 930; silicon the same
+// with both.  From 50,000 atoms on always 4 (1,578 evaluated: 139 / 136), below
+// 20,000 always 2.
+bool ace_wide_allowed(const mix_ctx* c) { return c->precision != MIX_FP64 && c->sys.n_atoms >= 20000; }
+
+void choose_ace_shape(mix_ctx* c, double evaluated) {
+    if (c->ace_tcm) return;
+    const bool wide = ace_wide_allowed(c) &&
+                      (c->sys.n_atoms >= 50000 || evaluated > (double)ACE_GROUP * c->ace_shape_grid[0]);
+    const int wn = wide ? ACE_MAX_WARPS : ACE_GROUP;
+    if (wn == c->ace_wn && c->ace_grid > 0) return;
+    c->ace_wn = wn;
+    c->ace_smem = c->ace_shape_smem[wide];
+    c->ace_grid = c->ace_grid_max = c->ace_shape_grid[wide];
+}
+
+// atoms the regions make the expensive potential evaluate, from the mean density:
+// each region with its ramp and buffer, a cylinder across the whole box
+double regions_evaluated(const mix_ctx* c, const Regions& r) {
+    const double* L = c->dev.box.L;
+    const double rho = (double)c->sys.n_atoms / (L[0] * L[1] * L[2]);
+    double v = 0.0;
+    for (int k = 0; k < r.n; ++k) {
+        const double* q = r.r[k];
+        const double R = q[7] + q[8] + c->dev.bufe;
+        v += (int)q[0] == MIX_REGION_CYLINDER
+                 ? M_PI * R * R * (std::fabs(q[4]) * L[0] + std::fabs(q[5]) * L[1] + std::fabs(q[6]) * L[2])
+                 : 4.0 / 3.0 * M_PI * R * R * R;
+    }
+    return std::min(rho * v, (double)c->sys.n_atoms);
 }
 
 void layout(mix_ctx* c) {
@@ -1060,15 +1101,19 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
         return st;
     }
     layout(c);
-    // large float systems: CTAs of 4 warps share the coefficient tiles between
-    // twice the atoms, so more warps fit an SM (their expensive sets are many
-    // waves large); small sets keep groups of 2, which spread them more evenly
-    c->ace_wn = (c->precision != MIX_FP64 && sys->n_atoms >= 20000) ? ACE_MAX_WARPS : ACE_GROUP;
-    cudaError_t e = c->ace_tcm
-                        ? ace_tc_configure(c->ace_tcm, c->L, c->n, c->cap, c->tile_max, c->qb, &c->ace_smem,
-                                           &c->ace_grid, &c->ace_nbuf)
-                        : ace_configure(c->precision, c->L, c->n, c->cap, c->tile_max, c->qb, &c->ace_smem,
-                                        &c->ace_grid, c->ace_wn);
+    cudaError_t e = cudaSuccess;
+    c->ace_wn = ACE_GROUP;
+    if (c->ace_tcm) {
+        e = ace_tc_configure(c->ace_tcm, c->L, c->n, c->cap, c->tile_max, c->qb, &c->ace_smem, &c->ace_grid, &c->ace_nbuf);
+    } else {
+        // both shapes of the CUDA-core kernel; choose_ace_shape picks one when the regions are known
+        for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+            if (k == 1 && !ace_wide_allowed(c)) break;
+            e = ace_configure(c->precision, c->L, c->n, c->cap, c->tile_max, c->qb, &c->ace_shape_smem[k],
+                              &c->ace_shape_grid[k], k ? ACE_MAX_WARPS : ACE_GROUP);
+        }
+        if (e == cudaSuccess) choose_ace_shape(c, 0.0);
+    }
     if (e != cudaSuccess) {
         delete c;
         return e == cudaErrorInvalidValue ? MIX_EINVAL : MIX_ECUDA;
@@ -1226,6 +1271,7 @@ int mix_set_regions(mix_ctx* c, const mix_region* r, int n) {
         R.iLf[t] = (float)c->dev.box.invL[t];
     }
     c->regions = R;
+    choose_ace_shape(c, regions_evaluated(c, R));
     c->seedrule.mode = 0;
     c->regions_version++;
     c->forces_valid = false;
