@@ -22,8 +22,8 @@
  *    the mix_get_* exports, mix_get_state() and the *_host entry points.
  *  - MIX_EOVERFLOW has two causes.  A neighbour row longer than the context's
  *    capacity is fatal for the context until it is re-created with a larger
- *    one.  A three-body neighbour count above what the cheap kernel's narrow
- *    lane groups hold (chosen at mix_init from the mean density) makes the
+ *    one.  A three-body neighbour count above what the cheap kernel's quarter
+ *    warps hold (16; chosen at mix_init from the mean density) makes the
  *    context switch to a warp per atom for later evaluations; the forces of
  *    the failing evaluation are incomplete and the caller repeats it.
  *  - Ownership: positions, velocities, forces and the workspace are caller-owned

@@ -909,7 +909,8 @@ int read_status(mix_ctx* c) {
     if (st & ST_NBR_OVERFLOW)
         return fail(c, MIX_EOVERFLOW, "neighbour list overflow: %d neighbours, capacity %d", c->pinned[SW_MAXNB], c->cap);
     if (st & ST_NB3_OVERFLOW) {
-        const int seen = c->pinned[SW_NB3MAX], lim = spline_nb3(c->spl_lpa), lpa = c->spl_lpa;
+        // (half warps hand what does not fit them to the whole warp: their limit is the warp's)
+        const int seen = c->pinned[SW_NB3MAX], lpa = c->spl_lpa, lim = spline_nb3(lpa == 16 ? 32 : lpa);
         if (lpa < 32 && seen <= spline_nb3(32)) {
             // the cheap kernel's narrow lane groups were chosen from the mean
             // density and this system has denser spots: widen them to a warp for
