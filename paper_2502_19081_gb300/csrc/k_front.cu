@@ -572,12 +572,6 @@ cudaError_t launch_front(const Dev& d, const Regions& r, const SeedRule& sr, cud
     // by side), the resident CTAs in a large one
     const int64_t want = (d.n + FRONT_WARPS - 1) / FRONT_WARPS;
     int64_t lim = d.grid_front_max;
-    // One CTA an SM while that leaves a warp at most three atoms to scan: two fill an
-    // SM's registers, so that nothing of another stream runs beside them.  5,831
-    // silicon atoms, us a step and system, one / two CTAs an SM: alone 44.5 / 43.4, 24
-    // of them on streams of their own 27.0 / 39.4 (before the one-launch front: 55.9
-    // and 20.0).  With a seed rule every phase takes a warp an atom: alone 63 / 58.
-    if (sr.mode == 0 && d.n <= (int64_t)3 * FRONT_WARPS * sm_count()) lim = std::min<int64_t>(lim, sm_count());
     if (d.grid_buffer > 0 && d.grid_buffer < lim) lim = d.grid_buffer;
     const int grid = (int)std::max<int64_t>(1, std::min(want, lim));
     // atoms per warp of the buffer scan: one up to 512 atoms per SM (a
