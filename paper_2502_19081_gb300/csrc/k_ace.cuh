@@ -12,10 +12,11 @@
 //   3. nu <= 2 readout; omega = dE/dA initialised;
 //   4. nu = 3, one l-triple (l1, l2, l3) after the other.  The triple's tables
 //      (W[q1 q2][q3]; float64 also the Gaunt entries in two orderings and their
-//      offsets) form one tile; the CTA streams the tiles from global memory into two
-//      shared-memory buffers with cp.async, fetching tile t+1 while the warps
-//      work on tile t, so a tile crosses L2 once per group of atoms rather
-//      than once per atom.  Float: k_nu3.cuh.  Float64, per warp: one pass over
+//      offsets) form one tile, brought from global memory into one of two
+//      shared-memory buffers by a bulk copy two tiles ahead (TileRing; with the
+//      tensor-core readout by cp.async, one tile ahead or, with one buffer, at the
+//      triple's start), so a tile crosses L2 once per group of atoms rather than
+//      once per atom.  Float: k_nu3.cuh.  Float64, per warp: one pass over
 //      lane units (q1, block of qb consecutive q2; the W rows of the block sit
 //      in registers) does all of
 //        U[m3][q1][q2] = sum_q3 W[q1 q2][q3] A3[m3][q3]
@@ -73,46 +74,15 @@ __device__ __forceinline__ void ld_gent(const GEnt<double>* p, int& pk, double& 
     g = __hiloint2double(v.w, v.z);
 }
 
-// QB consecutive values from shared memory (QB in {1, 2, 4}, aligned to QB;
-// QB = 6, float only, aligned to 2)
-template <typename T, int QB>
-__device__ __forceinline__ void ld_blk(const T* p, T* out) {
-    if constexpr (QB == 6) {
-        static_assert(sizeof(T) == 4, "6-wide blocks are float only");
+// QB (2 or 4) consecutive float64 values from shared memory, aligned to QB
+template <int QB>
+__device__ __forceinline__ void ld_blk(const double* p, double* out) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float2 v = reinterpret_cast<const float2*>(p)[k];
-            out[2 * k] = v.x;
-            out[2 * k + 1] = v.y;
-        }
-    } else if constexpr (QB == 4) {
-        const V4<T> v = ld4<T>(p);
-        out[0] = v.x;
-        out[1] = v.y;
-        out[2] = v.z;
-        out[3] = v.w;
-    } else if constexpr (QB == 2) {
-        if constexpr (sizeof(T) == 4) {
-            const float2 v = *reinterpret_cast<const float2*>(p);
-            out[0] = v.x;
-            out[1] = v.y;
-        } else {
-            const double2 v = *reinterpret_cast<const double2*>(p);
-            out[0] = v.x;
-            out[1] = v.y;
-        }
-    } else {
-        out[0] = p[0];
+    for (int k = 0; k < QB / 2; ++k) {
+        const double2 v = reinterpret_cast<const double2*>(p)[k];
+        out[2 * k] = v.x;
+        out[2 * k + 1] = v.y;
     }
-}
-
-// s += a . b as one chain of four fused multiply-adds
-template <typename T>
-__device__ __forceinline__ void dot4_acc(T& s, const V4<T>& a, const V4<T>& b) {
-    s += a.x * b.x;
-    s += a.y * b.y;
-    s += a.z * b.z;
-    s += a.w * b.w;
 }
 
 // Pi[l][m] = d^m P_l / dz^m for 0 <= m <= l <= L (flattened l(l+1)/2 + m),
@@ -285,10 +255,11 @@ __device__ __forceinline__ void tile_fetch(const unsigned char* tiles, const int
 // All three l's equal: U is not formed (no adjoint needs it) and the energy is
 // taken as sum A3 (W^T Z), the same sum reordered.  This is the float64 pass
 // (float: k_nu3.cuh).
-template <typename T, int NP, int QB>
-__device__ __forceinline__ void nu3_units(const AceTileHdr& h, const T* W, const GEnt<T>* ge3, const int* g3o,
-                                          const T* A1, const T* A2, const T* A3, int n, int lane, T* U1, T* P1,
-                                          T* o3, T mult3, T& ep) {
+template <int NP, int QB>
+__device__ __forceinline__ void nu3_units(const AceTileHdr& h, const double* W, const GEnt<double>* ge3, const int* g3o,
+                                          const double* A1, const double* A2, const double* A3, int n, int lane, double* U1, double* P1,
+                                          double* o3, double mult3, double& ep) {
+    using T = double;
     constexpr int nqb = NP / QB;
     const int units = n * nqb;
     const int d3 = 2 * h.l3 + 1;
@@ -353,7 +324,7 @@ __device__ __forceinline__ void nu3_units(const AceTileHdr& h, const T* W, const
                 ld_gent(ge3 + e, pk, g);
                 const T ga = g * A1q[(pk & 255) * NP];
                 T a2[QB];
-                ld_blk<T, QB>(A2q + ((pk >> 8) & 255) * NP, a2);
+                ld_blk<QB>(A2q + ((pk >> 8) & 255) * NP, a2);
 #pragma unroll
                 for (int r = 0; r < QB; ++r) z[r] += ga * a2[r];
                 if (withu) {
@@ -415,9 +386,9 @@ __device__ __forceinline__ void nu3_tile(const unsigned char* tile, const AceTab
     const T* A3 = At + h.l3 * h.l3 * NP;
     T* o3 = om + h.l3 * h.l3 * NP;
     if (qb == 4)
-        nu3_units<T, NP, 4>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
+        nu3_units<NP, 4>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
     else
-        nu3_units<T, NP, 2>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
+        nu3_units<NP, 2>(h, W, ge3, g3o, A1, A2, A3, n, lane, U1, P1, o3, mult3, ep);
     __syncwarp();
     // omega1 (equal to omega3 when all three l's coincide): sum the unit
     // partials of each (m1, q1) and clear them for the next triple
@@ -838,14 +809,12 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
         // Zhi Wlo); the warps take omega1 and omega2 meanwhile, then wait for
         // the MMAs and read their own rows of V: omega3 += mult3 V,
         // E += sum A3 V (lane-local, summed with the atom's other terms).
-        // this warp's 16 rows of the MMA tile, placed so that their
-        // accumulator rows lie in the TMEM lanes 32 (w % 4) .. + 31 the warp may
-        // read: M = 128 puts row i in lane i, M = 64 rows 16 w .. 16 w + 15 in
-        // lanes 32 w .. 32 w + 15
-        const int slot_w = TC_M == 128 ? 2 * (warp & 3) + (warp >> 2) : warp;
-        unsigned char* zh = tc->zhi + 2 * slot_w * tc->sbo;
-        unsigned char* zl = TCM == 2 ? tc->zlo + 2 * slot_w * tc->sbo : nullptr;
-        const bool own = TC_M == 128 ? (lane >> 4) == (warp >> 2) : lane < 16;   // TMEM lane 32 (w % 4) + lane
+        // this warp's 16 rows of the MMA tile: M = 64 puts the accumulators of rows
+        // 16 w .. 16 w + 15 in the TMEM lanes 32 w .. 32 w + 15, which the warp may read
+        static_assert(TC_M == 64, "the rows' TMEM lanes");
+        unsigned char* zh = tc->zhi + 2 * warp * tc->sbo;
+        unsigned char* zl = TCM == 2 ? tc->zlo + 2 * warp * tc->sbo : nullptr;
+        const bool own = lane < 16;   // TMEM lane 32 w + lane
         const int m3r = lane & 15;
         const uint32_t idesc = tc_idesc_bf16(TC_M, 16);
         const int kp = tc->kp, sbo_b = (kp / 8) * TC_LBO_B;

@@ -213,9 +213,8 @@ __device__ __forceinline__ void nb_run(const Dev& d, int cx, int cy, int cz, int
     }
 }
 
-// The longest row a warp wrote, once at its end: reductions to one address run at
-// some 3 ns each on this part, so one an atom alone would take 60 us of a
-// 20,000-atom build (which took 60) and 0.6 ms of a 200,000-atom one.
+// The longest row a warp wrote, once at its end rather than once a row: reductions to
+// one address run at some 3 ns each on this part, 60 us for 20,000 rows.
 __device__ __forceinline__ void nb_report_max(const Dev& d, int most, int lane) {
     if (lane == 0 && most > 0) atomicMax(d.status + SW_MAXNB, most);
 }

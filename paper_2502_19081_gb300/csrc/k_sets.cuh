@@ -198,7 +198,7 @@ __device__ __forceinline__ void blend_body(const Dev& d, const SeedRule& sr, int
 }
 
 // Buffer membership through the neighbour list.  A warp takes apw <= 32
-// consecutive atoms: each lane tests its atom's flags (and the hints k_lambda
+// consecutive atoms: each lane tests its atom's flags (and the hints lambda_atom
 // left), then groups of LPA lanes scan the lists of the atoms that need it,
 // 32 / LPA atoms at a time (the flags are ORs over a row, so the result does
 // not depend on LPA).  In a large system most atoms need no scan and then cost
@@ -218,7 +218,7 @@ __device__ __forceinline__ void buffer_body(const Dev& d, int bx, int gx, int ap
         const bool valid = lane < apw && im < d.n;
         const int fl = valid ? (int)d.flags[im] : 0;
         const int f = fl & 3;
-        // scan unless k_lambda's hints (bits 4, 5; geometric regions only) rule it out
+        // scan unless lambda_atom's hints (bits 4, 5; geometric regions only) rule it out
         const bool my_ne = valid && !(f & 1) && !(fl & 16), my_nc = valid && !(f & 2) && !(fl & 32);
         unsigned todo = __ballot_sync(0xffffffffu, my_ne || my_nc);
         bool my_he = false, my_hc = false;
