@@ -502,7 +502,7 @@ struct TileRing {
     uint32_t full;       // two mbarriers, 8 bytes apart (shared address)
     int* left;           // [2] warps still to finish the buffer's tile
     uint32_t phase;      // bit b: parity of buffer b's next completion
-    int abort;           // a wait ran out: no further waits (uniform over the warp)
+    int abort;           // a wait ran out: no further waits (the same for all threads)
 };
 
 __device__ __forceinline__ void bulk_fetch(void* dst, const void* src, int bytes, uint32_t bar) {
@@ -770,19 +770,19 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
     // 4. nu = 3, tile by tile
     if constexpr (TCM == 0) {
         for (int t = 0; t < ntau; ++t) {
-            // the CTA's warps start a triple together: each triple is code of its own
+            // The CTA's warps start a triple together: each triple is code of its own
             // (some 10 KB), and warps a triple apart fetch it one after the other (n =
-            // 12, lmax = 5: 1.26 ms without this barrier, 1.05 with it)
-            __syncthreads();
+            // 12, lmax = 5: 1.26 ms without this barrier, 1.05 with it).  The barrier also
+            // carries the wait's verdict, so abort is the same for all threads (a vote of
+            // each warp after the barrier took 0.7 % of the kernel).
             const int bsel = t & 1;
             unsigned char* tile = smem + bsel * lay.tile;
-            // (abort is the same for all lanes of a warp: see mbar_wait_warp)
-            if (!ring->abort && !mbar_wait_warp(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, d.tile_polls))
+            if (!ring->abort && !mbar_wait_cta(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, d.tile_polls))
                 ring->abort = 1;
-            if (ring->abort) {   // no tile: the barrier above is all that is left to do
+            if (ring->abort) {   // no tile, for any warp
                 // (said for every group that goes without: a batch's next one may be another system's)
-                if (lane == 0) set_status(d.status, ST_TC_TIMEOUT);
-                continue;
+                if (tid == 0) set_status(d.status, ST_TC_TIMEOUT);
+                break;
             }
             ring->phase ^= 1u << bsel;
             if constexpr (sizeof(T) == 8) {

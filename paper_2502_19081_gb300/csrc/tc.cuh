@@ -115,12 +115,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int lim
     return false;
 }
 
-// mbar_wait by a whole warp with one verdict: true when every lane saw the phase
-// complete.  Each lane polls on its own, so near the limit some may see it and
-// others not; a warp whose lanes then part (to a CTA barrier and to a warp-wide
-// shuffle) would never leave.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int limit) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit)) != 0;
+// mbar_wait by a whole CTA with one verdict, and a CTA barrier: true when every
+// thread saw the phase complete.  Each polls on its own, so near the limit some may
+// see it and others not; a warp whose lanes then part (to a CTA barrier and to a
+// warp-wide shuffle) would never leave.
+__device__ __forceinline__ bool mbar_wait_cta(uint32_t bar, uint32_t parity, int limit) {
+    return __syncthreads_or(mbar_wait(bar, parity, limit) ? 0 : 1) == 0;
 }
 
 // byte offset of element (row, k) in a K-major no-swizzle operand

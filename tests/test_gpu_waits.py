@@ -31,7 +31,7 @@ def _gives_up(mx, call):
 
 PROBE = """
 #include "tc.cuh"
-// lanes below 16 may poll, the others not at all: the wait's verdicts, one a lane
+// all threads but half of the last warp may poll: the wait's verdicts, one a thread
 __global__ void k_probe(int* out) {
     __shared__ __align__(8) unsigned long long bar;
     if (threadIdx.x == 0) {
@@ -39,17 +39,17 @@ __global__ void k_probe(int* out) {
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mixd::smem_u32(&bar)) : "memory");
     }
     __syncthreads();
-    out[threadIdx.x] = mixd::mbar_wait_warp(mixd::smem_u32(&bar), 0u, threadIdx.x < 16 ? 1 << 10 : 0);
-    out[32 + threadIdx.x] = mixd::mbar_wait_warp(mixd::smem_u32(&bar), 0u, 1 << 10);
+    out[threadIdx.x] = mixd::mbar_wait_cta(mixd::smem_u32(&bar), 0u, threadIdx.x < 48 ? 1 << 10 : 0);
+    out[64 + threadIdx.x] = mixd::mbar_wait_cta(mixd::smem_u32(&bar), 0u, 1 << 10);
 }
 extern "C" int probe(int* out) {
-    k_probe<<<1, 32>>>(out);
+    k_probe<<<1, 64>>>(out);
     return (int)cudaDeviceSynchronize();
 }
 """
 
 
-def test_a_warp_has_one_verdict(tmp_path):
+def test_a_block_has_one_verdict(tmp_path):
     import torch
     from paper_2502_19081_gb300 import build
     nvcc = build.nvcc()
@@ -59,11 +59,11 @@ def test_a_warp_has_one_verdict(tmp_path):
     src.write_text(PROBE)
     subprocess.run([nvcc, *build.ARCH, "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", build.CSRC, "-I",
                     build.INCLUDE, str(src), "-o", str(so)], check=True)
-    out = torch.full((64,), -1, dtype=torch.int32, device="cuda")
+    out = torch.full((128,), -1, dtype=torch.int32, device="cuda")
     torch.cuda.synchronize()
     assert ctypes.CDLL(str(so)).probe(ctypes.c_void_p(out.data_ptr())) == 0
     v = out.cpu().numpy()
-    assert (v[:32] == 0).all() and (v[32:] == 1).all()
+    assert (v[:64] == 0).all() and (v[64:] == 1).all()
 
 
 @pytest.mark.parametrize("prec", [0, 1])
