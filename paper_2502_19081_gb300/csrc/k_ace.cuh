@@ -773,17 +773,14 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
             // The CTA's warps start a triple together: each triple is code of its own
             // (some 10 KB), and warps a triple apart fetch it one after the other (n =
             // 12, lmax = 5: 1.26 ms without this barrier, 1.05 with it).  The barrier also
-            // carries the wait's verdict, so abort is the same for all threads (a vote of
-            // each warp after the barrier took 0.7 % of the kernel).
+            // carries the wait's verdict, so abort is the same for all threads.  (The code
+            // of this loop is near the instruction cache's limit: leaving it by break, or
+            // setting the status inside, cost 1 to 4 % of the 19,284-atom kernel.)
             const int bsel = t & 1;
             unsigned char* tile = smem + bsel * lay.tile;
             if (!ring->abort && !mbar_wait_cta(ring->full + 8 * bsel, (ring->phase >> bsel) & 1u, d.tile_polls))
                 ring->abort = 1;
-            if (ring->abort) {   // no tile, for any warp
-                // (said for every group that goes without: a batch's next one may be another system's)
-                if (tid == 0) set_status(d.status, ST_TC_TIMEOUT);
-                break;
-            }
+            if (ring->abort) continue;   // no tile, for any warp
             ring->phase ^= 1u << bsel;
             if constexpr (sizeof(T) == 8) {
                 if (has) nu3_tile<NP>(tile, tab, At, om, U1, P1, lane, ep);
@@ -802,6 +799,8 @@ __device__ __forceinline__ void ace_group(const Dev& d, const AceTab<T>& tab, in
                     ring_fetch(*ring, tab.tiles, tab.tile_off, t + 2, tile, WN);
             }
         }
+        // said for every group that goes without: a batch's next one may be another system's
+        if (ring->abort && tid == 0) set_status(d.status, ST_TC_TIMEOUT);
     } else {
         // Per triple: the warps write Z rows (and form U, omega1, omega2 as in
         // the CUDA-core pass); one thread issues V = Z W over K = kp (one MMA
