@@ -34,7 +34,10 @@
  *    allocate device memory of their own, described at their calls.
  *  - Layout: per-atom vectors are [N][4] float64 (x, y, z, unused), 32-byte rows,
  *    16-byte aligned or better.  Units: Angstrom, fs, eV, amu.
- *  - A context is not thread-safe; distinct contexts are independent.
+ *  - A context is not thread-safe; distinct contexts are independent.  On streams of
+ *    their own their kernels share the GPU, but the kernel that opens an evaluation
+ *    takes all of it for some 10 to 20 us; small systems that are stepped
+ *    together are much faster as a batch (mix_batch_*).
  */
 #ifndef MIX_H
 #define MIX_H

@@ -10,7 +10,12 @@
 // 15.7 us in all (as ten kernels 55 by their events), 1,000 atoms 11.4 (40),
 // 200,000 atoms 54 (79).  The phases are separated by grid barriers, so the launch
 // is cooperative (all CTAs resident, at most FRONT_CTAS an SM); every wait is
-// bounded.
+// bounded.  The price: two CTAs fill an SM's registers, so contexts on streams of
+// their own no longer overlap their small kernels (24 silicon systems of 5,831 atoms,
+// us a step and system: 39, as ten kernels 20; 8 iron dumbbells 116, as ten kernels
+// 151).  One CTA an SM brought the first to 27 and cost a system alone up to 5 %;
+// systems stepped together belong in a batch (15.8), whose front has kernels of
+// its own.
 #include <algorithm>
 #include <map>
 #include <mutex>

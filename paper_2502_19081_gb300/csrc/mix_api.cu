@@ -1120,11 +1120,13 @@ int mix_init(const mix_system* sys, const mix_ace* a, const mix_spline* sp, cons
         return e == cudaErrorInvalidValue ? MIX_EINVAL : MIX_ECUDA;
     }
     // Fewer lanes per cheap atom where atoms have few neighbours.  In a periodic bulk
-    // whose mean count inside the 3-body cutoff is at most a third of what a quarter
-    // warp holds on chip (16 slots), a quarter warp: Si has about 5.  Up to a mean
+    // whose mean count inside the 3-body cutoff, at uniform density, is at most a third
+    // of what a quarter warp holds on chip (16 slots), a quarter warp.  Up to a mean
     // of two thirds of a half warp's pair table (24), half a warp (whose atoms with
     // up to 32 neighbours are taken by the whole warp, spl_again): bcc Fe has 12 to
-    // 14 (198,128 atoms 360 -> 306 us).  A warp otherwise.
+    // 14 (198,128 atoms 360 -> 306 us), diamond Si 8.2 by this estimate, of which its
+    // open lattice has about 5: read_status moves it to a quarter warp after the first
+    // evaluation.  A warp otherwise.
     {
         bool bulk = vol > 0;
         for (int k = 0; k < 3; ++k) bulk = bulk && sys->periodic[k];
