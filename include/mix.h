@@ -422,8 +422,9 @@ int mix_batch_step(mix_batch* b, double dt_fs, int nsteps);
 int mix_batch_sync(mix_batch* b);
 
 /* Autotune the batch: for grid divisors 1, 2, 4, 8, 16 applied to every
- * member's persistent and gather grids, times launches of a graph of all
- * members' force evaluations (state unchanged) and keeps the fastest divisor. */
+ * member's persistent, front and gather grids, times launches of a graph of all
+ * members' force evaluations (state unchanged) and keeps the fastest divisor.
+ * (Members that a step has to evaluate one by one take the front's whole grid.) */
 int mix_batch_tune(mix_batch* b, int reps, int* chosen_divisor);
 
 int mix_batch_destroy(mix_batch* b);

@@ -2056,7 +2056,13 @@ int batch_prepare(mix_batch* b) {
         mix_ctx* c = b->m[k];
         if (!c->bound) return bfail(b, MIX_ESTATE, "member " + std::to_string(k) + " is not bound");
         if (c->need_build || !c->forces_valid) {
+            // one member after the other: each front takes what is resident, not its share
+            // among members that step side by side (24 silicon systems of 5,831 atoms,
+            // tuned, with new regions: a step 3,880 us with a sixteenth, 3,381 with all)
+            const int share = c->dev.grid_buffer;
+            c->dev.grid_buffer = 0;
             int st = evaluate(c, 0, 0.0);
+            c->dev.grid_buffer = share;
             if (st) return bfail(b, st, "member " + std::to_string(k) + ": " + c->err);
             c->forces_valid = true;
             fresh.push_back(k);
