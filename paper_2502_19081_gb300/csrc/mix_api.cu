@@ -370,6 +370,7 @@ struct mix_ctx {
     int ace_wn;                       // warps (atoms) a CTA of the CUDA-core expensive kernel
     size_t ace_shape_smem[2];         // its launch shapes with ACE_GROUP and ACE_MAX_WARPS warps
     int ace_shape_grid[2];
+    bool ace_settled;                 // seed atoms: the shape was chosen from a measured set
     int ace_tcm;                      // 0: CUDA-core nu = 3; 1, 2: tensor-core readout (bf16, bf16 hi/lo)
     int ace_nbuf;                     // tile buffers of the tensor-core kernel
     int spl_lpa;                      // lanes per atom of the cheap kernel (32, 16 or 8)
@@ -683,7 +684,8 @@ void fill_tabs(mix_ctx* c, unsigned char* base, AceTab<T>& at, SplTab<T>& st) {
 // 109 / 135, 1,242 133 / 136, 3,705 280 / 225, 13,004 773 / 676, 19,284 1122 / 1023; n = 10:
 // 1,012 73 / 73, 3,705 119 / 121, 13,004 346 / 342, 36,739 979 / 930; silicon the same
 // with both.  From 50,000 atoms on always 4 (1,578 evaluated: 139 / 136), below
-// 20,000 always 2.
+// 20,000 always 2.  The weights of seed atoms have no size beforehand: read_status
+// chooses from the first set they give.
 bool ace_wide_allowed(const mix_ctx* c) { return c->precision != MIX_FP64 && c->sys.n_atoms >= 20000; }
 
 void choose_ace_shape(mix_ctx* c, double evaluated) {
@@ -941,6 +943,15 @@ int read_status(mix_ctx* c) {
     if (st & ST_REV_MISSING) return fail(c, MIX_EINVAL, "asymmetric neighbour list");
     if (st & ST_GRID_TIMEOUT) return fail(c, MIX_ETIMEOUT, "a wait at a grid barrier gave up");
     if (st & ST_TC_TIMEOUT) return fail(c, MIX_ETIMEOUT, "a wait for a coefficient tile or the tensor-core readout gave up");
+    if (c->seedrule.mode != 0 && !c->ace_settled && c->forces_valid && c->pinned[SW_NEXP] > 0) {
+        c->ace_settled = true;
+        const int wn = c->ace_wn;
+        choose_ace_shape(c, c->pinned[SW_NEXP]);
+        if (c->ace_wn != wn) {
+            drop_graph(c);
+            c->regions_version++;   // any batch holding the context re-plans
+        }
+    }
     // The uniform-density estimate behind the initial lane groups overstates
     // open lattices (diamond holds half of it inside 3.4 A).  Once an
     // evaluation has measured the largest 3-body count, a periodic bulk moves
@@ -2295,6 +2306,7 @@ int mix_set_seeds(mix_ctx* c, const int* seeds, int n_seeds, double r_core, doub
     if (e != cudaSuccess) return cuda_fail(c, e, "mix_set_seeds");
     SeedRule& r = c->seedrule;
     r = SeedRule();
+    c->ace_settled = false;
     r.mode = 1;
     r.blend = c->opt.blend;
     r.rcore2 = r_core * r_core;
@@ -2322,6 +2334,7 @@ int mix_set_seed_rule(mix_ctx* c, double r_coord, double z_lo, double z_hi, int 
     if (e != cudaSuccess) return cuda_fail(c, e, "mix_set_seed_rule");
     SeedRule& r = c->seedrule;
     r = SeedRule();
+    c->ace_settled = false;
     r.mode = 2;
     r.blend = c->opt.blend;
     r.rcore2 = r_core * r_core;

@@ -32,3 +32,25 @@ def test_block_follows_the_evaluated_set(atoms, core, threads):
         assert c.info()["exp_threads"] == 64
     c.close()
     m.close()
+
+
+@pytest.mark.gpu
+def test_block_follows_the_set_of_seed_atoms():
+    """Seed atoms give no size beforehand: the first synchronising call chooses."""
+    from paper_2502_19081_gb300 import mix
+    pots = {"Fe": I.element_potentials("Fe", np.random.default_rng(3), 5.5, 12, 5, 4)}
+    wl = I.serve_request(3, "Fe", 20500, 0.005, 300.0, pots)
+    c = mix.open_context(wl, precision=mix.MIX_FP32)
+    for seeds, threads in ((np.arange(0, c.n, 5), 128), (np.array([100]), 64)):
+        c.set_seeds(seeds, 3.0, 4.0)
+        c.forces()
+        c.sync()
+        F = c.get_state()[2]
+        assert c.stats()["n_exp"] > 2000 if threads == 128 else c.stats()["n_exp"] < 1500
+        assert c.info()["exp_threads"] == threads
+        c.forces()
+        assert np.array_equal(F, c.get_state()[2])
+        c.step(1.0, 2)
+        c.sync()
+        assert c.info()["exp_threads"] == threads
+    c.close()
